@@ -6,7 +6,7 @@
 // Time (SSP-RK3, Shu-Osher form):
 //   u1 = u + dt L(u); u2 = 3/4 u + 1/4 (u1 + dt L(u1)); u' = 1/3 u + 2/3 (u2 + dt L(u2)).
 //
-// GPU design.  The grids of the cycle (the Ne coarse members, Algorithm 3
+// GPU design, FP32 (FP64 states: burgers_seg64, halo'd segments).  The grids of the cycle (the Ne coarse members, Algorithm 3
 // step 2, and the fine run, Algorithm 4 step 2) advance by all nsteps of an
 // observation interval inside one kernel pass:
 //   * a grid segment lives in registers for the whole launch: thread t owns
@@ -24,6 +24,7 @@
 //     launch_burgers); the generic kernel runs both in one launch.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <string>
@@ -602,6 +603,292 @@ static cudaError_t launch_burgers(BurgersArgs<T> A, cudaStream_t stream) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP64: grids cut into halo'd segments, one CTA each.
+//
+// GB300 issues one FP64 instruction of a warp per SM sub-partition in 64
+// cycles, however many of its lanes are active and with no further latency
+// (measured with dependent chains; 76 cycles with all four sub-partitions
+// busy), so a model step costs the FP64 instructions of the busiest
+// sub-partition and nothing else matters much.  One point per thread and 128
+// points per CTA put one warp on each sub-partition: 26 instructions, about
+// 1 us, per step.  Measured, one 16384-point grid, 4331 steps: 157 ms on one
+// cluster of four CTAs of 4096 points (36 us per step), 8.0 ms in segments
+// (1.86 us per step, 147 CTAs of 190 points with their halo).
+//
+// A CTA advances the points of its segment and H = 3 steps of halo on both
+// sides by a few steps with one barrier per RK stage; the halo's outermost
+// point goes stale per stage, so after `steps` steps exactly the segment is
+// valid, and the next launch reads it from the other of two buffers.  A grid
+// that is one segment needs no halo: its CTA wraps around and runs all steps
+// in one launch, in place.  seg_plan() picks the segment length and the steps
+// per launch from the cost of a step and of a launch.
+//
+// Arithmetic (per stage, edge differences e_j = u_{j+1} - u_j, exact for
+// neighbours within a factor 2): with c = 4 nu / dx, a = dt / (4 dx),
+//   k = c (e_j - e_{j-1}) - (e_j + e_{j-1}) (u_{j-1} + u_{j+1}),  dt L = a k,
+//   u1 = u + a k0,  u2 = u + a/4 (k0 + k1),  u' = u + a/6 (k0 + k1 + 4 k2),
+// one rounding at the size of u per stage, as the form it replaces.
+// ---------------------------------------------------------------------------
+struct SegGroup {
+    const double *src;
+    double *dst;
+    int n, W, H, P, nseg;  // points per grid, per segment, halo, points a CTA holds, segments per grid
+    int ring;              // one segment per grid, wrapped around
+    double a, c;
+};
+struct SegArgs {
+    SegGroup g[2];
+    int ctas0, steps;  // CTAs of group 0, steps of this launch
+};
+
+constexpr int kSegMaxThreads = 576;  // eight points per thread: grids of up to 4096 points and their halo
+template <int Q>
+__global__ void __launch_bounds__(Q == 1 ? 1024 : kSegMaxThreads) burgers_seg64(SegArgs A) {
+    extern __shared__ double seg_sh[];  // [2 buffers][first | last][blockDim]
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int t = threadIdx.x, nt = blockDim.x;
+    const bool second = (int)blockIdx.x >= A.ctas0;
+    const SegGroup G = second ? A.g[1] : A.g[0];
+    const int bid = (int)blockIdx.x - (second ? A.ctas0 : 0);
+    const int prob = bid / G.nseg, seg = bid - prob * G.nseg;
+    const int s0 = min(seg * G.W, G.n - G.W);  // the last segment overlaps its neighbour (same values)
+    const int P = G.P, last = (P - 1) / Q;
+    const int p0 = t * Q;
+    const bool act = p0 < P;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    double u[Q], s[Q], kk[Q];
+    if (act) {
+        const double *src = G.src + (size_t)prob * G.n;
+        int j = (s0 - G.H + p0) % G.n;
+        if (j < 0) j += G.n;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            u[k] = s[k] = src[j];
+            kk[k] = 0.0;
+            if (++j == G.n) j = 0;
+        }
+    }
+    const double a = G.a, c = G.c, a4 = 0.25 * a, a6 = a / 6.0;
+    const int lt = t == 0 ? last : t - 1, rt = t == last ? 0 : t + 1;
+    int buf = 0, lo = 0, hi = P;  // points [lo, hi) hold current values
+    for (int step = 0; step < A.steps; ++step) {
+#pragma unroll
+        for (int stage = 0; stage < 3; ++stage) {
+            double *sf = seg_sh + buf * 2 * nt, *sl = Q == 1 ? sf : sf + nt;
+            if (act) {
+                sf[t] = s[0];
+                if (Q > 1) sl[t] = s[Q - 1];
+            }
+            __syncthreads();
+            if (!G.ring) {
+                ++lo;
+                --hi;
+            }
+            if (act && p0 + Q > lo && p0 < hi) {
+                const double lft = sl[lt], rgt = sf[rt];
+                double prev = lft, el = s[0] - lft;
+#pragma unroll
+                for (int k = 0; k < Q; ++k) {
+                    const double cur = s[k], nxt = k + 1 < Q ? s[k + 1] : rgt;
+                    const double er = nxt - cur;
+                    const double kq = fma(c, er - el, -(er + el) * (prev + nxt));
+                    if (stage == 0) {
+                        kk[k] = kq;
+                        s[k] = fma(a, kq, u[k]);
+                    } else if (stage == 1) {
+                        kk[k] += kq;
+                        s[k] = fma(a4, kk[k], u[k]);
+                    } else {
+                        u[k] = fma(a6, fma(4.0, kq, kk[k]), u[k]);
+                        s[k] = u[k];
+                    }
+                    prev = cur;
+                    el = er;
+                }
+            }
+            buf ^= 1;
+        }
+    }
+    if (act) {
+        double *dst = G.dst + (size_t)prob * G.n;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const int p = p0 + k - G.H;
+            if (p >= 0 && p < G.W) dst[s0 + p] = u[k];
+        }
+    }
+}
+
+// points per thread for CTAs of at most P points
+static int seg_q(int P) { return P <= 128 ? 1 : P <= 256 ? 2 : P <= 512 ? 4 : 8; }
+
+// Segments of at most W points of a grid of n points, and the points a CTA
+// holds with a halo of 3 m (none for one segment of whole threads: a ring).
+struct SegShape {
+    int W, H, P, nseg, ring;
+};
+static SegShape seg_shape(int n, int W, int m, int Q) {
+    SegShape x;
+    x.nseg = ceil_div(n, W);
+    x.ring = x.nseg == 1 && n % Q == 0;
+    x.W = ceil_div(n, x.nseg);
+    x.H = x.ring ? 0 : 3 * m;
+    x.P = ceil_div(x.W + 2 * x.H, Q) * Q;
+    return x;
+}
+
+// The cheapest segment lengths and steps per launch: segments that fill P
+// points (warps on all four sub-partitions of the SM) for every step count m
+// per launch, W = P - 6 m, and whole grids as rings, alone or (the members)
+// beside a segmented fine run.  A CTA's step costs its FP64 instructions per
+// warp (6 + 1/Q per point and stage, 5 per point and step) at 19 cycles per
+// warp, at least 64 each, and 100 cycles per stage for the barrier and the
+// exchange; CTAs on one SM add up; a launch costs
+// kSegLaunch (16384 points, m = 3, 110-point segments: 1.66 us per step of
+// which 1.56 / 3 us the launches), and one shorter than kSegShortest would
+// leave the host's launch rate in charge (m = 2: 6.1 us per step).
+struct SegPlan {
+    int W[2] = {0, 0}, m = 0, launches = 0, Q = 0;
+    bool rings = false;  // no halo: every step in one launch, in place
+};
+constexpr double kSegLaunch = 3100.0, kSegShortest = 14000.0;
+static void seg_try(SegPlan &best, double &tbest, const int (&n)[2], const int (&np)[2], int nsteps, int sms,
+                    const int (&W)[2], int m, int Q) {
+    const int ops = 3 * (6 * Q + 1) + 5 * Q;
+    long long ctas = 0;
+    double slowest = 0.0, total = 0.0;
+    bool rings = true;
+    for (int g = 0; g < 2; ++g) {
+        if (np[g] <= 0) continue;
+        const SegShape x = seg_shape(n[g], W[g], m, Q);
+        const int threads = ceil_div(x.P, Q), warps = ceil_div(threads, 32);
+        if (threads > (Q == 1 ? 1024 : kSegMaxThreads)) return;
+        ctas += (long long)np[g] * x.nseg;
+        slowest = std::max(slowest, ops * (warps <= 3 ? 64.0 : 76.0 * ceil_div(warps, 4)));
+        total += (double)np[g] * x.nseg * ops * warps * 19.0;
+        rings = rings && x.ring;
+    }
+    int launches = rings ? 1 : ceil_div(nsteps, m);
+    if (launches > 1) launches += launches & 1;  // an even number: the state ends in its own buffer
+    const int per_sm = ceil_div(ctas, sms);
+    const double step = std::max(slowest, per_sm * total / ctas) + 300.0 * per_sm;
+    if (launches > 2 && step * m < kSegShortest) return;
+    // a single segmented launch is followed by a copy back
+    const double t = step * nsteps + kSegLaunch * (launches + (!rings && launches == 1));
+    if (t < tbest) {
+        tbest = t;
+        best = SegPlan{{W[0], W[1]}, rings ? nsteps : m, launches, Q, rings};
+    }
+}
+static SegPlan seg_plan(int n0, int np0, int n1, int np1, int nsteps, int sms) {
+    SegPlan best;
+    double tbest = 1e300;
+    const int n[2] = {n0, n1}, np[2] = {np0, np1};
+    const bool both = np0 > 0 && np1 > 0;
+    for (int P : {96, 128, 192, 256, 384, 512, 1024, 2048, 4096, 8 * kSegMaxThreads})
+        for (int m : {1, 2, 3, 4, 5, 6, 8, 10, 13, 16, 24, 32}) {
+            const int mm = std::min(m, nsteps), w = std::min(P - 6 * mm, kBurgersMaxPtsPerCta) & ~7;
+            if (w < 32) continue;
+            seg_try(best, tbest, n, np, nsteps, sms, {w, w}, mm, seg_q(P));
+            if (both && n0 <= kBurgersMaxPtsPerCta && w < n0)
+                seg_try(best, tbest, n, np, nsteps, sms, {n0, w}, mm, seg_q(std::max(n0, P)));
+        }
+    if ((np0 <= 0 || n0 <= kBurgersMaxPtsPerCta) && (np1 <= 0 || n1 <= kBurgersMaxPtsPerCta))
+        for (int Q : {1, 2, 4, 8}) seg_try(best, tbest, n, np, nsteps, sms, {n0, n1}, 1, Q);
+    return best;
+}
+
+template <int Q>
+static cudaError_t seg_launch(const SegArgs &A, int ctas, int threads, bool follows, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = sizeof(double) * 4 * threads;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = follows ? 1 : 0;  // after the first launch: start while the previous one ends
+    count_launches(1);
+    return cudaLaunchKernelEx(&cfg, burgers_seg64<Q>, A);
+}
+
+static int device_sms() {
+    static OncePerDevice once;
+    static int sms[kMaxDevices];
+    once.run([](int dev) { return cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev); });
+    const int dev = OncePerDevice::current();
+    return dev >= 0 && sms[dev] > 0 ? sms[dev] : kNumSMs;
+}
+
+size_t burgers64_scratch_elems(int n_whole, int n_whole_probs, int n_split, int n_split_probs, int nsteps) {
+    if (nsteps <= 0 || (n_whole_probs <= 0 && n_split_probs <= 0)) return 0;
+    if (seg_plan(n_whole, n_whole_probs, n_split, n_split_probs, nsteps, device_sms()).rings) return 0;
+    return (size_t)n_whole * std::max(n_whole_probs, 0) + (size_t)n_split * std::max(n_split_probs, 0);
+}
+
+cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, double *split, int n_split,
+                               int n_split_probs, double length, double dt, double nu, int nsteps, double *scratch,
+                               cudaStream_t stream) {
+    double *st[2] = {whole, split};
+    const int n[2] = {n_whole, n_split}, np[2] = {n_whole_probs, n_split_probs};
+    if (nsteps <= 0 || (np[0] <= 0 && np[1] <= 0)) return cudaSuccess;
+    const SegPlan pl = seg_plan(n[0], np[0], n[1], np[1], nsteps, device_sms());
+    if (pl.Q == 0) return cudaErrorInvalidConfiguration;
+    SegArgs A = {};
+    const size_t off[2] = {0, np[0] > 0 ? (size_t)n[0] * np[0] : 0};
+    const bool rings = pl.rings;
+    int ctas = 0, P = 0;
+    for (int g = 0; g < 2; ++g) {
+        if (np[g] <= 0) continue;
+        const SegShape x = seg_shape(n[g], pl.W[g], pl.rings ? 1 : pl.m, pl.Q);
+        const double dx = length / n[g];
+        A.g[g].n = n[g];
+        A.g[g].W = x.W;
+        A.g[g].nseg = x.nseg;
+        A.g[g].ring = x.ring;
+        A.g[g].a = dt / (4.0 * dx);
+        A.g[g].c = 4.0 * nu / dx;
+        ctas += np[g] * x.nseg;
+        if (g == 0) A.ctas0 = ctas;
+        P = std::max(P, x.P);
+    }
+    if (!rings && !scratch) return cudaErrorInvalidValue;
+    const int threads = ceil_div(ceil_div(P, pl.Q), 32) * 32;
+    int done = 0;
+    for (int l = 0; l < pl.launches; ++l) {
+        A.steps = (int)((long long)nsteps * (l + 1) / pl.launches) - done;
+        done += A.steps;
+        for (int g = 0; g < 2; ++g) {
+            if (np[g] <= 0) continue;
+            SegGroup &G = A.g[g];
+            double *other = rings ? st[g] : scratch + off[g];
+            G.src = l & 1 ? other : st[g];
+            G.dst = l & 1 ? st[g] : other;
+            G.H = G.ring ? 0 : 3 * A.steps;
+            G.P = G.ring ? G.n : ceil_div(G.W + 2 * G.H, pl.Q) * pl.Q;
+        }
+        cudaError_t e;
+        switch (pl.Q) {
+            case 1: e = seg_launch<1>(A, ctas, threads, l > 0, stream); break;
+            case 2: e = seg_launch<2>(A, ctas, threads, l > 0, stream); break;
+            case 4: e = seg_launch<4>(A, ctas, threads, l > 0, stream); break;
+            default: e = seg_launch<8>(A, ctas, threads, l > 0, stream); break;
+        }
+        if (e != cudaSuccess) return e;
+    }
+    if (!rings && pl.launches == 1)
+        for (int g = 0; g < 2; ++g)
+            if (np[g] > 0) {
+                const cudaError_t e = cudaMemcpyAsync(st[g], scratch + off[g], (size_t)n[g] * np[g] * sizeof(double),
+                                                      cudaMemcpyDeviceToDevice, stream);
+                if (e != cudaSuccess) return e;
+            }
+    return cudaSuccess;
+}
+
 int burgers_split_factor(int n) {
     // CTAs per grid: the smallest power of two cs with n / cs <= 4096 and n % cs == 0
     for (int cs = 1; cs <= 8; cs <<= 1)
@@ -639,7 +926,5 @@ cudaError_t burgers_forecast(T *whole, int n_whole, int n_whole_probs, T *split,
 
 template cudaError_t burgers_forecast<float>(float *, int, int, float *, int, int, double, double,
                                              double, int, cudaStream_t);
-template cudaError_t burgers_forecast<double>(double *, int, int, double *, int, int, double,
-                                              double, double, int, cudaStream_t);
 
 }  // namespace mgk

@@ -52,6 +52,7 @@ struct mgenkf_ctx {
     double *Tm = nullptr;                               // T, (ne+1) x ne (points at Bt or own buffer)
     double *truth_d = nullptr, *rmse_part = nullptr, *rmse_d = nullptr, *scratch = nullptr;
     void *ns_scratch = nullptr;  // NS-2D stage buffers
+    double *bur_scratch = nullptr;  // FP64 Burgers: the second state of the alternating launches
     void *fine_prev = nullptr;   // fine state one model step before the end of the last forecast
     void *fine_tmp = nullptr;    // output of the final fine iteration
     double alpha = 0.0;          // relaxation of the final fine iteration (0: none)
@@ -149,7 +150,7 @@ static void free_all(mgenkf_ctx *h) {
     void *ptrs[] = {h->fine, h->members, h->xstar, h->dC, h->tap_idx, h->tap_w, h->tap_wh, h->tap_wl, h->yf, h->yo,
                     h->ybar, h->eps, h->Y, h->Z, h->X64, h->X16, h->Tt, h->S, h->Lt, h->Bt, h->C,
                     h->Ct, h->W, h->truth_d, h->rmse_part, h->rmse_d, h->scratch, h->status,
-                    h->ns_scratch, h->gemm_part, h->cycle_d, h->fine_prev, h->fine_tmp,
+                    h->ns_scratch, h->bur_scratch, h->gemm_part, h->cycle_d, h->fine_prev, h->fine_tmp,
                     h->df.Yh, h->df.Yl, h->df.Zh, h->df.Zl, h->d_fc};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -324,6 +325,8 @@ static mgenkf_status create_impl(mgenkf_ctx *h, const mgenkf_config *cfg, const 
     }
     if (cfg->model == MGENKF_NS2D)
         H_ALLOC(h->ns_scratch, ns2d_scratch_elems(h->nc, h->ne, h->nf, 1) * ts);
+    else if (!h->mixed)
+        H_ALLOC(h->bur_scratch, (ne * nx + h->nxf) * ts);
     {
         const size_t p1 = (size_t)gemm_nt_splits((int)ne, (int)ne, (int)ne + 1, (int)ny) * ne * (2 * ne + 1);
         const size_t p2 = (size_t)gemm_nt_splits((int)ne, 0, (int)ne + 1, (int)ny) * ne * (ne + 1);
@@ -570,8 +573,8 @@ static mgenkf_status advance_impl(mgenkf_ctx *h, int nsteps) {
             e = burgers_forecast<float>((float *)h->members, h->nc, h->ne, (float *)h->fine, h->nf, 1,
                                         c.length, c.dt, c.nu, nsteps, h->stream);
         else
-            e = burgers_forecast<double>((double *)h->members, h->nc, h->ne, (double *)h->fine, h->nf, 1,
-                                         c.length, c.dt, c.nu, nsteps, h->stream);
+            e = burgers_forecast64((double *)h->members, h->nc, h->ne, (double *)h->fine, h->nf, 1, c.length, c.dt,
+                                   c.nu, nsteps, (double *)h->bur_scratch, h->stream);
     } else {
         // with the filter the model step is an RK3 step followed by the filter
         // of every grid (the stage buffers are free in between)
@@ -1143,9 +1146,18 @@ extern "C" mgenkf_status mgk_forecast(int32_t model, int32_t precision, void *st
         if (precision == MGENKF_MIXED)
             e = whole ? burgers_forecast<float>((float *)state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, s)
                       : burgers_forecast<float>(nullptr, 0, 0, (float *)state, n, nprob, length, dt, nu, nsteps, s);
-        else
-            e = whole ? burgers_forecast<double>((double *)state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, s)
-                      : burgers_forecast<double>(nullptr, 0, 0, (double *)state, n, nprob, length, dt, nu, nsteps, s);
+        else {
+            // stream-ordered scratch
+            double *scratch = nullptr;
+            const size_t elems = burgers64_scratch_elems(n, nprob, 0, 0, nsteps);
+            e = elems ? cudaMallocAsync((void **)&scratch, elems * sizeof(double), s) : cudaSuccess;
+            if (e == cudaSuccess)
+                e = burgers_forecast64((double *)state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, scratch, s);
+            if (scratch) {
+                const cudaError_t e2 = cudaFreeAsync(scratch, s);
+                if (e == cudaSuccess) e = e2;
+            }
+        }
     } else if (model == MGENKF_NS2D) {
         const char *why = ns2d_check_size(n, n);
         if (why) {
