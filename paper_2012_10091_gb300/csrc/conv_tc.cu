@@ -41,10 +41,13 @@
 // rows of a CTA.  Input rows live in a ring, so each is loaded once.  Five warps
 // issue two taps each (the last layer: 187 us with one issuing thread, 138 with
 // five warps); each MMA then takes about 54 cycles, 32 of them the reads of
-// its 4 KB A operand from shared memory.
+// its 4 KB A operand from shared memory.  Every FLUSH rows the accumulators are
+// added to sums in registers (10 us more for the last layer): the tensor cores
+// truncate, and over a whole run of rows the bias grew to 2e-6 of the gradient
+// against 9e-7 now and 8e-7 on the FP32 pipes.
 //
 // Measured, 8 samples of 256^2 coarse points: the loss and all gradients 5.4 ms
-// with the backward pass on the CUDA cores, 0.68 ms here; inference of one
+// with the backward pass on the CUDA cores, 0.70 ms here; inference of one
 // sample 80 us, 27 us here.
 //
 // Rows and pixels past the map's edge are computed from wrapped inputs (zeros
@@ -129,8 +132,13 @@ constexpr int tmem_cols(int used) { return used <= 32 ? 32 : used <= 64 ? 64 : u
 // that no more are resident, so no CTA waits in alloc
 constexpr int tmem_min_smem(int cols) { return 228 * 1024 / (512 / cols + 1) + 2048; }
 
+// The tensor cores truncate their FP32 sums, a bias of up to one ulp of the
+// accumulator per MMA.  A gradient's leading split therefore has an accumulator
+// per row of taps (12 MMAs at most), its two remainders one of their own (2^-8
+// of the size), and the four are added in registers.
 template <int CG, int NSPLIT, int COUT, int ROWS>
 struct ConvShape {
+    static constexpr int NACC = NSPLIT == 1 ? 1 : 4;
     static constexpr int CGK = CG < 2 ? 2 : CG;               // channel groups of K (padded to 16 channels)
     // channel groups per chunk: a forward layer is one chunk (its MMAs run tap by
     // tap, and the order decides the FP32 sums that the BF16 activations round);
@@ -141,10 +149,10 @@ struct ConvShape {
     static constexpr int STAGE = GPC * PLANE;
     static constexpr int NST = NC < 4 ? NC : 4;
     static constexpr int W_BYTES = 9 * CGK * COUT * 16;
-    static constexpr int TMEM_COLS = tmem_cols(ROWS * COUT);
+    static constexpr int TMEM_COLS = tmem_cols(ROWS * NACC * COUT);
     static constexpr int NEED = 1024 + NST * STAGE + W_BYTES;
     static constexpr int SMEM = NEED > tmem_min_smem(TMEM_COLS) ? NEED : tmem_min_smem(TMEM_COLS);
-    static_assert(ROWS * COUT <= 512, "accumulators of one CTA fit TMEM");
+    static_assert(ROWS * NACC * COUT <= 512, "accumulators of one CTA fit TMEM");
     static_assert(COUT % 16 == 0 && COUT >= 16 && COUT <= 256, "N of an M = 128 MMA");
     static_assert(CGK % 2 == 0, "K steps of 16 channels");
 };
@@ -259,7 +267,8 @@ __global__ void __launch_bounds__(kConvThreads, EPI == kLoss ? 3 : 2) k_conv_tc(
             const bool lead = tc::elect_one();
             const uint32_t ac = a0 + (uint32_t)((c % S::NST) * S::STAGE + uwarp * kRowW * 16);
             const uint32_t bc = b0 + (uint32_t)(S::GPC * (c % (S::CGK / S::GPC)) * COUT * 16);
-            const uint32_t acc = tmem + (uint32_t)(uwarp * COUT);
+            const uint32_t acc = tmem + (uint32_t)(uwarp * S::NACC * COUT);
+            constexpr int CPS = S::CGK / S::GPC;  // chunks per split
             if (uwarp < rows) {
 #pragma unroll
                 for (int t = 0; t < 9; ++t) {
@@ -269,7 +278,13 @@ __global__ void __launch_bounds__(kConvThreads, EPI == kLoss ? 3 : 2) k_conv_tc(
                             ac + (uint32_t)(2 * k * S::PLANE + ((t / 3) * kRowW + t % 3) * 16), S::PLANE, 128);
                         const uint64_t bd = tc::smem_desc_interleave(
                             bc + (uint32_t)((t * S::CGK + 2 * k) * COUT * 16), COUT * 16, 128);
-                        tc::mma_bf16_lead(lead, acc, ad, bd, idesc, (c | t | k) ? 1u : 0u);
+                        if (NSPLIT == 1) {
+                            tc::mma_bf16_lead(lead, acc, ad, bd, idesc, (c | t | k) ? 1u : 0u);
+                        } else {
+                            const bool first = c < CPS;  // the leading split
+                            tc::mma_bf16_lead(lead, acc + (uint32_t)((first ? t / 3 : 3) * COUT), ad, bd, idesc,
+                                              (first ? (c | (t % 3) | k) : ((c - CPS) | t | k)) ? 1u : 0u);
+                        }
                     }
                 }
             }
@@ -307,7 +322,14 @@ __global__ void __launch_bounds__(kConvThreads, EPI == kLoss ? 3 : 2) k_conv_tc(
             for (int c0 = 0; c0 < COUT; c0 += 16) {
                 float v[16];
                 __syncwarp();
-                tc::tmem_ld16(lane_base + (uint32_t)(r * COUT + c0), v);
+                tc::tmem_ld16(lane_base + (uint32_t)(r * S::NACC * COUT + c0), v);
+#pragma unroll
+                for (int h = 1; h < S::NACC; ++h) {
+                    float v1[16];
+                    tc::tmem_ld16(lane_base + (uint32_t)((r * S::NACC + h) * COUT + c0), v1);
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) v[q] += v1[q];
+                }
                 if (x < n) {
                     if (EPI != kBackward) {
 #pragma unroll
@@ -469,9 +491,13 @@ struct WgradShape {
     static constexpr int AG = COUT / 8;                     // channel groups of one split
     static constexpr int PXS = COUT == 64 ? kPix / 2 : kPix;  // pixels of a row of d per stage
     static constexpr int APL = PXS * 16;                    // bytes of one group's plane of a stage
-    static constexpr int A_STAGE = 4 * AG * APL;            // [hi][mid][lo][zeros]
+    static constexpr int A_STAGE = 4 * AG * APL;            // COUT 32: [hi][mid][lo][zeros], 64: [hi][mid][zeros][lo]
     static constexpr int NST = 4;                           // stages: three in flight beside the one in use
-    static constexpr int NM = COUT / 32;                    // M = 128 MMAs per K step: (hi, mid[, lo, 0]) [, (lo, 0)]
+    // M = 128 MMAs per K step: (hi, mid, lo, 0), or (hi, mid) and (0, lo) into the
+    // same accumulator rows (the remainders together: see ConvShape)
+    static constexpr int NM = COUT / 32;
+    static constexpr int LO = COUT == 64 ? 3 : 2, ZERO = 5 - LO;  // which quarter of a stage holds lo, zeros
+    static constexpr int FLUSH = 2;                         // rows of d summed in TMEM before the registers
     static constexpr int BPL = kRowW * 16;
     static constexpr int B_ROW = CGB * BPL;                 // one row of the input
     static constexpr int USED = 9 * N + 16;                 // TMEM columns: nine taps and the bias
@@ -519,7 +545,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
     // constant parts: the zero planes of the stages, the padded input group, the ones
     for (int e = tid; e < S::NST * S::AG * S::PXS; e += kConvThreads) {
         const int st = e / (S::AG * S::PXS), k = e - st * (S::AG * S::PXS);
-        reinterpret_cast<uint4 *>(sa + st * S::A_STAGE + 3 * S::AG * S::APL)[k] = make_uint4(0, 0, 0, 0);
+        reinterpret_cast<uint4 *>(sa + st * S::A_STAGE + S::ZERO * S::AG * S::APL)[k] = make_uint4(0, 0, 0, 0);
     }
     if (CGI < 2)
         for (int e = tid; e < 8 * kRowW; e += kConvThreads)
@@ -558,7 +584,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
             const __nv_bfloat16 *src = d + (size_t)split * d_split +
                                        (((size_t)b * S::AG + (g - split * S::AG)) * pl + (size_t)(r0 + i) * n +
                                         (in_map ? x0 + j : 0)) * 8;
-            cp_async16_zfill(dst + e * 16, src, in_map);
+            const int shift = split == 2 ? (S::LO - 2) * S::AG * S::APL : 0;
+            cp_async16_zfill(dst + e * 16 + shift, src, in_map);
         }
         if (q % SPR == 0) load_in(r0 + i + 1);
     };
@@ -570,6 +597,13 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
     }
     uint32_t tmem = 0;
     bool ok = true;
+    // the running sums: warps 0-3 hold taps 0-4 of their 32 accumulator rows,
+    // warps 4-7 taps 5-8 and the bias
+    const int half = warp >> 2;
+    constexpr int HT = 5;
+    float sum[HT * S::N];
+#pragma unroll
+    for (int e = 0; e < HT * S::N; ++e) sum[e] = 0.f;
     for (int q = 0; q < steps; ++q) {
         cp_async_wait<S::NST - 2>();  // step q has landed (one group per iteration below)
         fence_async_proxy();
@@ -605,7 +639,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
                 for (int m = 0; m < S::NM; ++m) {
                     const uint64_t ad =
                         tc::smem_desc_interleave(aa + (uint32_t)(m * 16 * S::APL + k * 256), 128, S::APL);
-                    const uint32_t acc = (q | k | m) ? 1u : 0u;
+                    const uint32_t acc = ((q % (S::FLUSH * SPR)) | k | m) ? 1u : 0u;
                     tc::mma_bf16_lead(lead, dt, ad, tc::smem_desc_interleave(bt[0] + k * 256, 128, S::BPL), idesc, acc);
                     tc::mma_bf16_lead(lead, dt + S::N, ad, tc::smem_desc_interleave(bt[1] + k * 256, 128, pitch1), id1,
                                       acc);
@@ -618,28 +652,50 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
             if (ok) load_step(q - 1 + S::NST);
         }
         cp_async_commit();
+        if ((q + 1) % (S::FLUSH * SPR) == 0 || q + 1 == steps) {
+            // the sums of these rows into the registers; the next step's MMAs
+            // start anew (after the barrier at the top)
+            ok = ok && tc::mbar_wait(&bar[q % S::NST], (q / S::NST) & 1);
+            if (__syncthreads_or(!ok)) {
+                ok = false;
+                break;
+            }
+            tc::fence_after_sync();
+            const uint32_t src = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(half * HT * S::N);
+#pragma unroll
+            for (int t = 0; t < HT; ++t) {
+                if (half && t == HT - 1) {
+                    float v[16];
+                    tc::tmem_ld16(src + (uint32_t)(t * S::N), v);
+                    sum[t * S::N] += v[0];
+                } else {
+#pragma unroll
+                    for (int c0 = 0; c0 < S::N; c0 += 16) {
+                        float v[16];
+                        tc::tmem_ld16(src + (uint32_t)(t * S::N + c0), v);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) sum[t * S::N + c0 + e] += v[e];
+                    }
+                }
+            }
+        }
     }
     cp_async_wait<0>();
-    if (ok) ok = tc::mbar_wait(&bar[(steps - 1) % S::NST], ((steps - 1) / S::NST) & 1);
     ok = !__syncthreads_or(!ok);
     if (!ok) {
         if (tid == 0 && status) atomicCAS(status, 0, tc::kStTimeout);
     } else {
-        tc::fence_after_sync();
         // per tap: the 128 accumulator rows to shared memory, the splits' rows
         // added (hi + mid) + lo in order
         float *tile = reinterpret_cast<float *>(sa);
         constexpr int LD = S::N + 1;
         float *out = part + (size_t)blockIdx.x * (9 * COUT * CIN + COUT);
-        for (int t = 0; t <= 9; ++t) {
-            if (warp < 4) {
-                const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * S::N);
-                for (int c0 = 0; c0 < (t < 9 ? S::N : 16); c0 += 16) {
-                    float v[16];
-                    tc::tmem_ld16(lane_base + c0, v);
+        const int m = (warp & 3) * 32 + lane;
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) tile[tid * LD + c0 + q] = v[q];
-                }
+        for (int t = 0; t <= 9; ++t) {
+            if (half == t / HT) {
+#pragma unroll
+                for (int c = 0; c < (t < 9 ? S::N : 1); ++c) tile[m * LD + c] = sum[(t % HT) * S::N + c];
             }
             __syncthreads();
             const int count = t < 9 ? COUT * CIN : COUT, width = t < 9 ? CIN : 1;
