@@ -51,6 +51,16 @@ constexpr int kNumSMs = 152;  // GB300: 2 dies x 76 SMs (grids are sized from th
 
 __host__ __device__ inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
+// Dynamic shared memory that lets `ctas` CTAs (1 to 3), and no more, share an
+// SM (228 KB, 1 KB of it per CTA), or `need` where that is more or no limit is
+// asked for.  A launch that becomes ready while another one drains (programmatic
+// serialisation above all) is placed on whatever SMs have room at that moment:
+// without a limit some SMs take several of its CTAs and others none.
+inline size_t residency_smem(size_t need, int ctas) {
+    const size_t limit = ctas >= 1 && ctas <= 3 ? (size_t)228 * 1024 / (ctas + 1) - 512 : 0;
+    return need > limit ? need : limit;
+}
+
 // device status word values (a subset of mgenkf_status)
 constexpr int kStatusOk = 0;
 

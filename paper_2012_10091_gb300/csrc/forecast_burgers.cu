@@ -613,8 +613,8 @@ static cudaError_t launch_burgers(BurgersArgs<T> A, cudaStream_t stream) {
 // sub-partition and nothing else matters much.  One point per thread and 128
 // points per CTA put one warp on each sub-partition: 26 instructions, about
 // 1 us, per step.  Measured, one 16384-point grid, 4331 steps: 157 ms on one
-// cluster of four CTAs of 4096 points (36 us per step), 8.0 ms in segments
-// (1.86 us per step, 147 CTAs of 190 points with their halo).
+// cluster of four CTAs of 4096 points (36 us per step), 6.7 ms in segments
+// (1.56 us per step, 149 CTAs of 128 points with their halo, 3 steps a launch).
 //
 // A CTA advances the points of its segment and H = 3 steps of halo on both
 // sides by a few steps with one barrier per RK stage; the halo's outermost
@@ -646,7 +646,6 @@ constexpr int kSegMaxThreads = 576;  // eight points per thread: grids of up to 
 template <int Q>
 __global__ void __launch_bounds__(Q == 1 ? 1024 : kSegMaxThreads) burgers_seg64(SegArgs A) {
     extern __shared__ double seg_sh[];  // [2 buffers][first | last][blockDim]
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int t = threadIdx.x, nt = blockDim.x;
     const bool second = (int)blockIdx.x >= A.ctas0;
     const SegGroup G = second ? A.g[1] : A.g[0];
@@ -656,7 +655,9 @@ __global__ void __launch_bounds__(Q == 1 ? 1024 : kSegMaxThreads) burgers_seg64(
     const int P = G.P, last = (P - 1) / Q;
     const int p0 = t * Q;
     const bool act = p0 < P;
+    // the previous launch has completed; the next one may be placed
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     double u[Q], s[Q], kk[Q];
     if (act) {
         const double *src = G.src + (size_t)prob * G.n;
@@ -745,14 +746,13 @@ static SegShape seg_shape(int n, int W, int m, int Q) {
 // warp (6 + 1/Q per point and stage, 5 per point and step) at 19 cycles per
 // warp, at least 64 each, and 100 cycles per stage for the barrier and the
 // exchange; CTAs on one SM add up; a launch costs
-// kSegLaunch (16384 points, m = 3, 110-point segments: 1.66 us per step of
-// which 1.56 / 3 us the launches), and one shorter than kSegShortest would
-// leave the host's launch rate in charge (m = 2: 6.1 us per step).
+// kSegLaunch (16384 points, 110-point segments, m = 3: 1.56 us per step, 1.25 / 3
+// of it the launches).
 struct SegPlan {
     int W[2] = {0, 0}, m = 0, launches = 0, Q = 0;
     bool rings = false;  // no halo: every step in one launch, in place
 };
-constexpr double kSegLaunch = 3100.0, kSegShortest = 14000.0;
+constexpr double kSegLaunch = 2600.0;
 static void seg_try(SegPlan &best, double &tbest, const int (&n)[2], const int (&np)[2], int nsteps, int sms,
                     const int (&W)[2], int m, int Q) {
     const int ops = 3 * (6 * Q + 1) + 5 * Q;
@@ -773,7 +773,6 @@ static void seg_try(SegPlan &best, double &tbest, const int (&n)[2], const int (
     if (launches > 1) launches += launches & 1;  // an even number: the state ends in its own buffer
     const int per_sm = ceil_div(ctas, sms);
     const double step = std::max(slowest, per_sm * total / ctas) + 300.0 * per_sm;
-    if (launches > 2 && step * m < kSegShortest) return;
     // a single segmented launch is followed by a copy back
     const double t = step * nsteps + kSegLaunch * (launches + (!rings && launches == 1));
     if (t < tbest) {
@@ -788,7 +787,7 @@ static SegPlan seg_plan(int n0, int np0, int n1, int np1, int nsteps, int sms) {
     const bool both = np0 > 0 && np1 > 0;
     for (int P : {96, 128, 192, 256, 384, 512, 1024, 2048, 4096, 8 * kSegMaxThreads})
         for (int m : {1, 2, 3, 4, 5, 6, 8, 10, 13, 16, 24, 32}) {
-            const int mm = std::min(m, nsteps), w = std::min(P - 6 * mm, kBurgersMaxPtsPerCta) & ~7;
+            const int mm = std::min(m, nsteps), w = std::min(P - 6 * mm, kBurgersMaxPtsPerCta);
             if (w < 32) continue;
             seg_try(best, tbest, n, np, nsteps, sms, {w, w}, mm, seg_q(P));
             if (both && n0 <= kBurgersMaxPtsPerCta && w < n0)
@@ -800,11 +799,16 @@ static SegPlan seg_plan(int n0, int np0, int n1, int np1, int nsteps, int sms) {
 }
 
 template <int Q>
-static cudaError_t seg_launch(const SegArgs &A, int ctas, int threads, bool follows, cudaStream_t stream) {
+static cudaError_t seg_launch(const SegArgs &A, int ctas, int threads, int per_sm, bool follows,
+                              cudaStream_t stream) {
+    static OncePerDevice once;
+    once.run([](int) {
+        return cudaFuncSetAttribute(burgers_seg64<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024);
+    });
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = sizeof(double) * 4 * threads;
+    cfg.dynamicSmemBytes = residency_smem(sizeof(double) * 4 * threads, per_sm);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -857,6 +861,8 @@ cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, do
     }
     if (!rings && !scratch) return cudaErrorInvalidValue;
     const int threads = ceil_div(ceil_div(P, pl.Q), 32) * 32;
+    // segments: the CTAs spread over the SMs (rings run once, whatever their place)
+    const int per_sm = rings ? 0 : ceil_div(ctas, device_sms());
     int done = 0;
     for (int l = 0; l < pl.launches; ++l) {
         A.steps = (int)((long long)nsteps * (l + 1) / pl.launches) - done;
@@ -872,10 +878,10 @@ cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, do
         }
         cudaError_t e;
         switch (pl.Q) {
-            case 1: e = seg_launch<1>(A, ctas, threads, l > 0, stream); break;
-            case 2: e = seg_launch<2>(A, ctas, threads, l > 0, stream); break;
-            case 4: e = seg_launch<4>(A, ctas, threads, l > 0, stream); break;
-            default: e = seg_launch<8>(A, ctas, threads, l > 0, stream); break;
+            case 1: e = seg_launch<1>(A, ctas, threads, per_sm, l > 0, stream); break;
+            case 2: e = seg_launch<2>(A, ctas, threads, per_sm, l > 0, stream); break;
+            case 4: e = seg_launch<4>(A, ctas, threads, per_sm, l > 0, stream); break;
+            default: e = seg_launch<8>(A, ctas, threads, per_sm, l > 0, stream); break;
         }
         if (e != cudaSuccess) return e;
     }
