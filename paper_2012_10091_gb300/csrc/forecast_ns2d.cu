@@ -32,10 +32,8 @@
 // shared-memory access is 64 bits wide and every arithmetic instruction is a
 // packed FFMA2 / FADD2 / FMUL2 on both points.
 //
-// FP64 states use one launch per stage: a CTA owns a 32 x 8 tile, loads the
-// stage input of the tile and its one-point halo into shared memory, forms the
-// primitives once per loaded point, and each thread evaluates the 9-point
-// stencil of its point; s1 and s2 live in two scratch buffers.
+// FP64 states use one launch per stage, a row march with every flux formed once
+// (ns2d_march64); s1 and s2 live in two scratch buffers.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -49,128 +47,259 @@
 namespace mgk {
 
 constexpr int kNsTx = 32;
-// tile rows of the per-handle kernels: 32 FP32 rows (the fused step, 32 x 32
-// points), 8 FP64 rows
-template <typename T>
-constexpr int ns_tile_rows() { return std::is_same<T, float>::value ? 32 : 8; }
+constexpr int kNsTileRows = 32;  // rows of a tile of the fused FP32 step (32 x 32 points)
 
-template <typename T>
-struct NsArgs {
-    NsGroup<T> g[2];
-    int tiles0;  // tiles of group 0
-    T gm1, mu, kappa;
+// ---------------------------------------------------------------------------
+// FP64: one launch per RK stage, a march down the rows
+//
+// GB300 issues an FP64 instruction of a warp per SM sub-partition in 64 cycles,
+// whatever its lanes do (76 with all four sub-partitions busy), so the stage
+// costs its FP64 instructions times the warps on the busiest sub-partition;
+// shared memory, integer work and barriers are nearly free beside them.  The
+// march therefore forms every quantity once: primitives and nodal fluxes at
+// their node (the reciprocal of rho by a third-order iteration), the x-face
+// fluxes by the thread west of the face, the y-face fluxes once per row, and
+// hands them on through shared memory or registers; 80 FP64 instructions per
+// point and stage, against about 180 for 32 x 8 tiles that formed the fluxes at
+// every neighbour, four faces per node, a division per node and a 1.33-fold
+// halo of nodes.
+//
+// Four warps per CTA, one point of a row per thread.  A unit is a strip of
+// columns (the whole periodic width up to 128 points per side, else equal
+// strips of at most 128) by `rows` rows of one grid; narrow grids put several
+// units side by side in a CTA, so that all four sub-partitions work.  A strip's
+// two halo columns (and the face west of its first column) are formed for all
+// of its rows at once before the march, a lane per node: an instruction for two
+// lanes per row would cost as much as one for 32.  Step k of the march takes in
+// row k - 1 of the unit and finishes row k - 2, two barriers per step.
+//
+// Measured (10 steps): one 512^2 grid 2.74 -> 1.49 ms, 32 members of 64^2 and a
+// 256^2 fine run 2.38 -> 1.34 ms; 80 instructions at 608 G/s would be 1.03, 0.78 ms.
+// ---------------------------------------------------------------------------
+constexpr int kN64Threads = 128;
+
+struct Ns64Args {
+    NsGroup<double> g[2];  // tx: strips per grid, ty: runs of rows
+    int ctas0, rows;       // CTAs of group 0, rows per unit
+    double gm1, k2;        // gamma - 1, 2 kappa / mu
+    double c1[2], c2[2];   // -dt / (2h), dt mu / h^2 of each group
 };
 
-// The stencil body is written for a tile shape TX x TY (TX * TY = 256
-// threads); the batched path picks the shape per grid size (autotuned).
-template <typename T, int STAGE, int TX, int TY>
-__device__ __forceinline__ void ns2d_stage_tile(const NsGroup<T> &G, int tile, T gm1, T mu, T kap) {
-    constexpr int HX = TX + 2, HY = TY + 2, HALO = HX * HY;
-    __shared__ T sq[4][HALO];   // conserved variables of the tile + halo
-    __shared__ T spr[4][HALO];  // u, v, p, T
-    const int tiles_per_prob = G.tx * G.ty;
-    const int prob = tile / tiles_per_prob;
-    const int tt = tile % tiles_per_prob;
-    const int x0 = (tt % G.tx) * TX, y0 = (tt / G.tx) * TY;
-    const int n = G.n;
-    const size_t plane = (size_t)n * n;
-    T *u0 = G.u0 + (size_t)prob * 4 * plane;
-    const T *in = STAGE == 0 ? u0 : (STAGE == 1 ? G.s1 : G.s2) + (size_t)prob * 4 * plane;
-    T *out = STAGE == 0 ? G.s1 + (size_t)prob * 4 * plane
-                        : (STAGE == 1 ? G.s2 + (size_t)prob * 4 * plane : u0);
+// 1 / x to about one unit in the last place: with e = 1 - x y of an approximate
+// reciprocal y (relative error 2^-20 or better), y (1 + e + e^2) = (1 - e^3) / x
+// (third-order Newton / Householder iteration)
+__device__ __forceinline__ double recip64(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
 
-    // load the tile and its halo, form the primitives
-    for (int e = threadIdx.x; e < HALO; e += blockDim.x) {
-        const int ly = e / HX, lx = e % HX;
-        int gy = y0 + ly - 1, gx = x0 + lx - 1;  // periodic wrap without integer division
-        if (gy < 0) gy += n;
-        if (gx < 0) gx += n;
-        while (gy >= n) gy -= n;
-        while (gx >= n) gx -= n;
-        const size_t o = (size_t)gy * n + gx;
-        const T rho = in[o], mx = in[plane + o], my = in[2 * plane + o], E = in[3 * plane + o];
-        const T rinv = T(1) / rho;  // one division per point
-        const T u = mx * rinv, v = my * rinv;
-        const T p = gm1 * (E - T(0.5) * rho * (u * u + v * v));
-        sq[0][e] = rho;
-        sq[1][e] = mx;
-        sq[2][e] = my;
-        sq[3][e] = E;
-        spr[0][e] = u;
-        spr[1][e] = v;
-        spr[2][e] = p;
-        spr[3][e] = p * rinv;
-    }
-    __syncthreads();
-    const int lx = threadIdx.x % TX, ly = threadIdx.x / TX;
-    const int x = x0 + lx, y = y0 + ly;
-    if (x >= n || y >= n) return;
-    const int c = (ly + 1) * HX + (lx + 1);
-    const int e_ = c + 1, w_ = c - 1, n_ = c + HX, s_ = c - HX;
-    const T *U = spr[0], *V = spr[1], *P = spr[2], *TT = spr[3];
-    const T ih = G.inv_h, i2h = G.inv_2h;
-    const T c43 = T(4.0 / 3.0), c23 = T(2.0 / 3.0), half = T(0.5);
-    // inviscid part: central differences of the nodal fluxes
-    T r[4];
-    {
-        const T mxe = sq[1][e_], mxw = sq[1][w_], myn = sq[2][n_], mys = sq[2][s_];
-        const T Fe1 = mxe * U[e_] + P[e_], Fw1 = mxw * U[w_] + P[w_];
-        const T Fe2 = mxe * V[e_], Fw2 = mxw * V[w_];
-        const T Fe3 = (sq[3][e_] + P[e_]) * U[e_], Fw3 = (sq[3][w_] + P[w_]) * U[w_];
-        const T Gn1 = myn * U[n_], Gs1 = mys * U[s_];
-        const T Gn2 = myn * V[n_] + P[n_], Gs2 = mys * V[s_] + P[s_];
-        const T Gn3 = (sq[3][n_] + P[n_]) * V[n_], Gs3 = (sq[3][s_] + P[s_]) * V[s_];
-        r[0] = -((mxe - mxw) + (myn - mys)) * i2h;
-        r[1] = -((Fe1 - Fw1) + (Gn1 - Gs1)) * i2h;
-        r[2] = -((Fe2 - Fw2) + (Gn2 - Gs2)) * i2h;
-        r[3] = -((Fe3 - Fw3) + (Gn3 - Gs3)) * i2h;
-    }
-    // viscous and heat fluxes on the four faces of the node
-    T fx[2][3], fy[2][3];
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-        {   // x-face between columns a = x-1+side and b = a+1
-            const int a = side ? c : w_, b = side ? e_ : c;
-            const T ux = (U[b] - U[a]) * ih, vx = (V[b] - V[a]) * ih;
-            const T uy = half * ((U[a + HX] - U[a - HX]) + (U[b + HX] - U[b - HX])) * i2h;
-            const T vy = half * ((V[a + HX] - V[a - HX]) + (V[b + HX] - V[b - HX])) * i2h;
-            const T txx = mu * (c43 * ux - c23 * vy), txy = mu * (uy + vx);
-            const T uf = half * (U[a] + U[b]), vf = half * (V[a] + V[b]);
-            fx[side][0] = txx;
-            fx[side][1] = txy;
-            fx[side][2] = txx * uf + txy * vf + kap * (TT[b] - TT[a]) * ih;
-        }
-        {   // y-face between rows a = y-1+side and b = a+1
-            const int a = side ? c : s_, b = side ? n_ : c;
-            const T uy = (U[b] - U[a]) * ih, vy = (V[b] - V[a]) * ih;
-            const T ux = half * ((U[a + 1] - U[a - 1]) + (U[b + 1] - U[b - 1])) * i2h;
-            const T vx = half * ((V[a + 1] - V[a - 1]) + (V[b + 1] - V[b - 1])) * i2h;
-            const T tyy = mu * (c43 * vy - c23 * ux), txy = mu * (uy + vx);
-            const T uf = half * (U[a] + U[b]), vf = half * (V[a] + V[b]);
-            fy[side][0] = txy;
-            fy[side][1] = tyy;
-            fy[side][2] = txy * uf + tyy * vf + kap * (TT[b] - TT[a]) * ih;
-        }
-    }
-    T L[4];
-    L[0] = r[0];
-#pragma unroll
-    for (int k = 1; k < 4; ++k)
-        L[k] = r[k] + ((fx[1][k - 1] - fx[0][k - 1]) + (fy[1][k - 1] - fy[0][k - 1])) * ih;
+// what a node contributes: u, v, T' = k2 T, rho u, rho v and the nodal fluxes
+// F = (rho u, F1, F2, F3), G = (rho v, F2, G2, G3)
+struct Node64 {
+    double U, V, T, mx, my, F1, F2, F3, G2, G3;
+};
+__device__ __forceinline__ Node64 node64(double rho, double mx, double my, double E, double gm1, double k2) {
+    Node64 q;
+    const double ri = recip64(rho);
+    q.mx = mx;
+    q.my = my;
+    q.U = mx * ri;
+    q.V = my * ri;
+    const double p = fma(-0.5 * gm1, fma(mx, q.U, my * q.V), gm1 * E);
+    q.T = p * (k2 * ri);
+    const double H = E + p;
+    q.F1 = fma(mx, q.U, p);
+    q.F2 = mx * q.V;
+    q.F3 = H * q.U;
+    q.G2 = fma(my, q.V, p);
+    q.G3 = H * q.V;
+    return q;
+}
 
-    const size_t o = (size_t)y * n + x;
+// viscous and heat flux of the face between a and b in units of mu / h (normal
+// stress, shear stress, twice the work and heat): dn, dt differences across the
+// face of the normal and tangential velocity, sn, st their sums, tn (tt) the sum
+// over a and b of the tangential difference of the normal (tangential) velocity
+struct Face64 {
+    double n, t, e;
+};
+__device__ __forceinline__ Face64 face64(double dn, double dt, double sn, double st, double tn, double tt, double dT) {
+    Face64 f;
+    f.n = fma(4.0 / 3.0, dn, (-1.0 / 6.0) * tt);
+    f.t = fma(0.25, tn, dt);
+    f.e = fma(f.n, sn, fma(f.t, st, dT));
+    return f;
+}
+
+// doubles of shared memory: two rows of seven published values, the y
+// differences of u, v, the x faces, and the halo columns of a strip
+__host__ __device__ constexpr int n64_smem_doubles(int rows) { return 19 * kN64Threads + (rows + 2) * 22; }
+
+template <int STAGE>
+__global__ void __launch_bounds__(kN64Threads) ns2d_march64(Ns64Args A) {
+    extern __shared__ double n64_sm[];
+    constexpr int NT = kN64Threads;
+    const int tid = threadIdx.x;
+    const int gi = (int)blockIdx.x >= A.ctas0 ? 1 : 0;
+    const NsGroup<double> G = gi ? A.g[1] : A.g[0];
+    const double c1 = gi ? A.c1[1] : A.c1[0], c2 = gi ? A.c2[1] : A.c2[0];
+    const int n = G.n, TX = (n + G.tx - 1) / G.tx, pitch = (TX + 31) & ~31, upc = NT / pitch;
+    const int sub = tid / pitch, i = tid - sub * pitch;
+    const long long unit = (long long)((int)blockIdx.x - (gi ? A.ctas0 : 0)) * upc + sub;
+    const int per_grid = G.tx * G.ty;
+    const int prob = (int)(unit / per_grid), rem = (int)(unit - (long long)prob * per_grid);
+    const int strip = rem / G.ty, seg = rem - strip * G.ty;
+    const int x0 = strip * TX, w = min(TX, n - x0), y0 = seg * A.rows, rows = min(A.rows, n - y0);
+    const bool act = sub < upc && prob < G.nprob && i < w;
+    const bool halo = G.tx > 1;  // one unit per CTA then
+    const size_t plane = (size_t)n * n, off = (size_t)(act ? prob : 0) * 4 * plane;
+    const double *u0 = G.u0 + off;
+    const double *in = STAGE == 0 ? u0 : (STAGE == 1 ? G.s1 : G.s2) + off;
+    double *out = (STAGE == 0 ? G.s1 : STAGE == 1 ? G.s2 : G.u0) + off;
+    const double gm1 = A.gm1, k2 = A.k2;
+    auto wrap = [n](int g) { return g < 0 ? g + n : g >= n ? g - n : g; };
+
+    double *P = n64_sm;             // [row parity][U V T mx F1 F2 F3][thread]
+    double *D = P + 14 * NT;        // [u, v differences in y][thread]
+    double *F = D + 2 * NT;         // [face east of the thread][thread]
+    double *HP = F + 3 * NT;        // [row][west, east column][7]
+    double *HC = HP + (A.rows + 2) * 14;  // [row][U V T] of the first column
+    double *HD = HC + (A.rows + 2) * 3;   // [row][2] y differences of the east column
+    double *HF = HD + (A.rows + 2) * 2;   // [row][3] the face west of the first column
+    const bool he = halo && i == w - 1, hw = halo && i == 0;
+    const int te = i == w - 1 ? tid - (w - 1) : tid + 1, tw = i == 0 ? tid + w - 1 : tid - 1;
+    // the previous launch has completed; the next one may be placed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    if (halo) {  // uniform over the CTA
+        for (int e = tid; e < 3 * (rows + 2); e += NT) {
+            const int k = e / 3, c = e - 3 * k;
+            const size_t o = (size_t)wrap(y0 - 1 + k) * n + wrap(c == 0 ? x0 - 1 : c == 1 ? x0 : x0 + w);
+            const Node64 q = node64(in[o], in[plane + o], in[2 * plane + o], in[3 * plane + o], gm1, k2);
+            if (c == 1) {
+                HC[3 * k] = q.U;
+                HC[3 * k + 1] = q.V;
+                HC[3 * k + 2] = q.T;
+            } else {
+                const double v[7] = {q.U, q.V, q.T, q.mx, q.F1, q.F2, q.F3};
+                double *h = HP + 14 * k + (c ? 7 : 0);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const T kq = G.dt * L[k];
-        const T s = sq[k][c];
-        T res;
-        if (STAGE == 0) {
-            res = s + kq;
-        } else {
-            const T base = u0[k * plane + o];
-            res = fma(STAGE == 1 ? T(0.25) : T(2.0 / 3.0), (s - base) + kq, base);
+                for (int f = 0; f < 7; ++f) h[f] = v[f];
+            }
         }
-        out[k * plane + o] = res;
+        __syncthreads();
+        for (int e = tid; e < rows; e += NT) {
+            const int k = e + 1;
+            const double *a = HP + 14 * k, *b = HC + 3 * k;
+            const double uy = (a[14] - a[-14]) + (b[3] - b[-3]), vy = (a[15] - a[-13]) + (b[4] - b[-2]);
+            const Face64 f = face64(b[0] - a[0], b[1] - a[1], a[0] + b[0], a[1] + b[1], uy, vy, b[2] - a[2]);
+            HF[3 * k] = f.n;
+            HF[3 * k + 1] = f.t;
+            HF[3 * k + 2] = f.e;
+            HD[2 * k] = a[14 + 7] - a[-14 + 7];
+            HD[2 * k + 1] = a[15 + 7] - a[-13 + 7];
+        }
+        // read after the first barrier of the march
+    }
+
+    double q[4] = {1.0, 0.0, 0.0, 0.0}, qc[4] = {0.0, 0.0, 0.0, 0.0};
+    const size_t col = (size_t)(act ? x0 + i : 0);
+    auto load = [&](int k) {
+        const size_t o = (size_t)wrap(y0 - 1 + k) * n + col;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) q[f] = in[f * plane + o];
+    };
+    if (act) load(0);
+    Node64 m1{}, cc{}, p1{};
+    double uxc = 0.0, vxc = 0.0;
+    Face64 yf{};
+    for (int k = 0; k < A.rows + 2; ++k) {
+        const bool have = act && k < rows + 2, fin = have && k >= 2;
+        double *Pk = P + (k & 1) * 7 * NT, *Pc = P + ((k + 1) & 1) * 7 * NT;
+        double qn[4] = {0.0, 0.0, 0.0, 0.0}, base[4] = {0.0, 0.0, 0.0, 0.0};
+        if (have) {
+            m1 = cc;
+            cc = p1;
+            p1 = node64(q[0], q[1], q[2], q[3], gm1, k2);
+            Pk[tid] = p1.U;
+            Pk[NT + tid] = p1.V;
+            Pk[2 * NT + tid] = p1.T;
+            Pk[3 * NT + tid] = p1.mx;
+            Pk[4 * NT + tid] = p1.F1;
+            Pk[5 * NT + tid] = p1.F2;
+            Pk[6 * NT + tid] = p1.F3;
+        }
+        double uy = 0.0, vy = 0.0;
+        const size_t oc = (size_t)wrap(y0 - 2 + k) * n + col;
+        if (fin) {
+            uy = p1.U - m1.U;
+            vy = p1.V - m1.V;
+            D[tid] = uy;
+            D[NT + tid] = vy;
+            if (STAGE > 0)
+#pragma unroll
+                for (int f = 0; f < 4; ++f) base[f] = u0[f * plane + oc];
+        }
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            qn[f] = qc[f];  // the row to finish in this step
+            qc[f] = q[f];
+        }
+        if (act && k + 1 < rows + 2) load(k + 1);
+        __syncthreads();
+        double uxk = 0.0, vxk = 0.0;
+        Face64 top{}, fe{};
+        double r[4] = {0.0, 0.0, 0.0, 0.0};
+        if (have) {
+            const double *hk = HP + 14 * k;
+            uxk = (he ? hk[7] : Pk[te]) - (hw ? hk[0] : Pk[tw]);
+            vxk = (he ? hk[8] : Pk[NT + te]) - (hw ? hk[1] : Pk[NT + tw]);
+            if (k >= 1)
+                top = face64(p1.V - cc.V, p1.U - cc.U, cc.V + p1.V, cc.U + p1.U, vxk + vxc, uxk + uxc, p1.T - cc.T);
+        }
+        if (fin) {
+            const double *hc = HP + 14 * (k - 1);
+            const double Ue = he ? hc[7] : Pc[te], Ve = he ? hc[8] : Pc[NT + te], Te = he ? hc[9] : Pc[2 * NT + te];
+            const double uye = he ? HD[2 * (k - 1)] : D[te], vye = he ? HD[2 * (k - 1) + 1] : D[NT + te];
+            fe = face64(Ue - cc.U, Ve - cc.V, cc.U + Ue, cc.V + Ve, uy + uye, vy + vye, Te - cc.T);
+            F[tid] = fe.n;
+            F[NT + tid] = fe.t;
+            F[2 * NT + tid] = fe.e;
+            double dx[4];
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+                dx[f] = (he ? hc[10 + f] : Pc[(3 + f) * NT + te]) - (hw ? hc[3 + f] : Pc[(3 + f) * NT + tw]);
+            r[0] = dx[0] + (p1.my - m1.my);
+            r[1] = dx[1] + (p1.F2 - m1.F2);
+            r[2] = dx[2] + (p1.G2 - m1.G2);
+            r[3] = dx[3] + (p1.G3 - m1.G3);
+        }
+        __syncthreads();
+        if (fin) {
+            const double *hf = HF + 3 * (k - 1);
+            const double wn = hw ? hf[0] : F[tw], wt = hw ? hf[1] : F[NT + tw], we = hw ? hf[2] : F[2 * NT + tw];
+            const double v[4] = {0.0, (fe.n - wn) + (top.t - yf.t), (fe.t - wt) + (top.n - yf.n),
+                                 (fe.e - we) + (top.e - yf.e)};
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                const double cv = f == 3 ? 0.5 * c2 : c2;
+                double res;
+                if (STAGE == 0) {
+                    res = qn[f] + (f == 0 ? c1 * r[0] : fma(cv, v[f], c1 * r[f]));
+                } else {
+                    double t = fma(c1, r[f], qn[f] - base[f]);
+                    if (f > 0) t = fma(cv, v[f], t);
+                    res = fma(STAGE == 1 ? 0.25 : 2.0 / 3.0, t, base[f]);
+                }
+                out[f * plane + oc] = res;
+            }
+        }
+        uxc = uxk;
+        vxc = vxk;
+        yf = top;
     }
 }
 
@@ -1045,14 +1174,88 @@ void ns2d_march_layout(int n, int shape, int *bands, int *segs, int *threads) {
     *threads = march_threads(n, narrow);
 }
 
-// per-handle FP64 launch: two groups (members, fine run) passed by value, 32 x 8 tiles
-template <typename T, int STAGE>
-__global__ void __launch_bounds__(256) ns2d_stage_kernel(NsArgs<T> A) {
-    int tile = blockIdx.x;
-    const int gi = tile < A.tiles0 ? 0 : 1;
-    if (gi) tile -= A.tiles0;
-    const NsGroup<T> G = gi ? A.g[1] : A.g[0];  // no runtime index into the parameter array
-    ns2d_stage_tile<T, STAGE, 32, 8>(G, tile, A.gm1, A.mu, A.kappa);
+// strips of an n x n grid in the FP64 march, and the CTAs of `grids` grids cut
+// into runs of `rows` rows
+static int n64_strips(int n) { return ceil_div(n, kN64Threads); }
+static long long n64_ctas(int n, int grids, int rows) {
+    const int pitch = ceil_div(ceil_div(n, n64_strips(n)), 32) * 32, upc = kN64Threads / pitch;
+    return ((long long)grids * n64_strips(n) * ceil_div(n, rows) + upc - 1) / upc;
+}
+
+template <int STAGE>
+static cudaError_t n64_launch(const Ns64Args &A, long long ctas, int per_sm, bool follows, cudaStream_t s) {
+    static OncePerDevice once;
+    once.run([](int) {
+        return cudaFuncSetAttribute(ns2d_march64<STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024);
+    });
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(kN64Threads);
+    cfg.dynamicSmemBytes = residency_smem(sizeof(double) * n64_smem_doubles(A.rows), per_sm);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = follows ? 1 : 0;
+    count_launches(1);
+    return cudaLaunchKernelEx(&cfg, ns2d_march64<STAGE>, A);
+}
+
+static cudaError_t n64_forecast(const NsGroup<double> (&g)[2], double gm1, double mu, double kappa, int nsteps,
+                                cudaStream_t s) {
+    Ns64Args A = {};
+    static OncePerDevice once;
+    static int sm_count[kMaxDevices];
+    once.run([](int dev) { return cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev); });
+    const int dev = OncePerDevice::current(), sms = dev >= 0 && sm_count[dev] > 0 ? sm_count[dev] : kNumSMs;
+    auto ctas = [&](int rows) {
+        long long c = 0;
+        for (int k = 0; k < 2; ++k)
+            if (g[k].nprob > 0) c += n64_ctas(g[k].n, g[k].nprob, rows);
+        return c;
+    };
+    // rows per unit and CTAs per SM at once: the FP64 instructions of a CTA (80
+    // per row, about 60 for the two extra rows) times the CTAs an SM runs; one,
+    // two, three CTAs at a time leave 20%, 10%, 2% of the pipe idle at barriers
+    // and loads (512^2: 1.62 ms with 14 rows, 1.56 with two of 7, 1.61 with three
+    // of 5; 64^2 x 32 and 256^2: 1.31 with 11 rows, 1.37, 1.33)
+    double best = 1e300;
+    int per_sm = 1;
+    const int nmax = std::max(g[0].nprob > 0 ? g[0].n : 0, g[1].nprob > 0 ? g[1].n : 0);
+    for (int rows = 2; rows <= std::min(nmax, 64); ++rows) {
+        const long long c = ctas(rows);
+        for (int r = 1; r <= 3; ++r) {
+            const double idle[3] = {1.2, 1.1, 1.02};
+            const double t = (double)((c + (long long)sms * r - 1) / ((long long)sms * r)) * r * idle[r - 1] *
+                             (80.0 * rows + 60.0);
+            if (t < best) {
+                best = t;
+                A.rows = rows;
+                per_sm = r;
+            }
+        }
+    }
+    for (int k = 0; k < 2; ++k) {
+        A.g[k] = g[k];
+        if (g[k].nprob <= 0) continue;
+        A.g[k].tx = n64_strips(g[k].n);
+        A.g[k].ty = ceil_div(g[k].n, A.rows);
+        A.c1[k] = -g[k].dt * g[k].inv_2h;
+        A.c2[k] = g[k].dt * mu * g[k].inv_h * g[k].inv_h;
+    }
+    A.gm1 = gm1;
+    A.k2 = mu > 0.0 ? 2.0 * kappa / mu : 0.0;
+    A.ctas0 = g[0].nprob > 0 ? (int)n64_ctas(g[0].n, g[0].nprob, A.rows) : 0;
+    const long long total = ctas(A.rows);
+    if (total > INT32_MAX) return cudaErrorInvalidConfiguration;
+    cudaError_t e = cudaSuccess;
+    for (int st = 0; st < nsteps && e == cudaSuccess; ++st) {
+        e = n64_launch<0>(A, total, per_sm, st > 0, s);
+        if (e == cudaSuccess) e = n64_launch<1>(A, total, per_sm, true, s);
+        if (e == cudaSuccess) e = n64_launch<2>(A, total, per_sm, true, s);
+    }
+    return e;
 }
 
 const char *ns2d_check_size(int n_whole, int n_split) {
@@ -1071,13 +1274,13 @@ cudaError_t ns2d_forecast_scratch(T *whole, int n_whole, int n_whole_probs, T *s
                                   int n_split_probs, double length, double dt, double mu,
                                   double gamma, double prandtl, int nsteps, T *scratch,
                                   cudaStream_t stream) {
-    NsArgs<T> A = {};
+    NsGroup<T> gr[2] = {};
     const int ns[2] = {n_whole, n_split}, np[2] = {n_whole_probs, n_split_probs};
     T *st[2] = {whole, split};
     T *sc = scratch;
     int tiles[2] = {0, 0};
     for (int g = 0; g < 2; ++g) {
-        NsGroup<T> &G = A.g[g];
+        NsGroup<T> &G = gr[g];
         G.n = ns[g];
         G.nprob = np[g];
         G.u0 = st[g];
@@ -1087,7 +1290,7 @@ cudaError_t ns2d_forecast_scratch(T *whole, int n_whole, int n_whole_probs, T *s
         sc += 2 * sz;
         if (np[g] > 0) {
             G.tx = ceil_div(ns[g], kNsTx);
-            G.ty = ceil_div(ns[g], ns_tile_rows<T>());
+            G.ty = ceil_div(ns[g], kNsTileRows);
             const double h = length / ns[g];
             G.inv_h = (T)(1.0 / h);
             G.inv_2h = (T)(1.0 / (2.0 * h));
@@ -1095,10 +1298,7 @@ cudaError_t ns2d_forecast_scratch(T *whole, int n_whole, int n_whole_probs, T *s
             tiles[g] = G.tx * G.ty * np[g];
         }
     }
-    A.tiles0 = tiles[0];
-    A.gm1 = (T)(gamma - 1.0);
-    A.mu = (T)mu;
-    A.kappa = (T)(mu * gamma / ((gamma - 1.0) * prandtl));
+    const T gm1 = (T)(gamma - 1.0), m = (T)mu, kappa = (T)(mu * gamma / ((gamma - 1.0) * prandtl));
     const int grid = tiles[0] + tiles[1];
     if (grid == 0 || nsteps == 0) return cudaSuccess;
     if constexpr (std::is_same<T, float>::value) {
@@ -1109,28 +1309,24 @@ cudaError_t ns2d_forecast_scratch(T *whole, int n_whole, int n_whole_probs, T *s
         if (n_split_probs > 0) {
             // a handle (members and fine run): both groups in one persistent
             // launch of the tile kernel per step
-            PairTiles P{{A.g[0], A.g[1]}};
+            PairTiles P{{gr[0], gr[1]}};
             P.g[0].tile_begin = 0;
             P.g[1].tile_begin = tiles[0];
-            step_sequence<32, 16, 2>(P, 2, grid, nsteps, A.gm1, A.mu, A.kappa, stream);
+            step_sequence<32, 16, 2>(P, 2, grid, nsteps, gm1, m, kappa, stream);
         } else {
             // grids of one size (truth runs, the stateless entry point): the
             // column march
-            OneUnits U{A.g[0]};
+            OneUnits U{gr[0]};
             int bands = 0, segs = 0, threads = 0;
             ns2d_march_layout(ns[0], np[0] == 1 ? 1 : 0, &bands, &segs, &threads);
             U.g.tx = bands;
             U.g.ty = segs;
             U.g.tile_begin = 0;
-            march_sequence(U, 1, bands * segs * np[0], threads, nsteps, A.gm1, A.mu, A.kappa, stream);
+            march_sequence(U, 1, bands * segs * np[0], threads, nsteps, gm1, m, kappa, stream);
         }
     } else {
-        for (int s = 0; s < nsteps; ++s) {
-            ns2d_stage_kernel<T, 0><<<grid, 256, 0, stream>>>(A);
-            ns2d_stage_kernel<T, 1><<<grid, 256, 0, stream>>>(A);
-            ns2d_stage_kernel<T, 2><<<grid, 256, 0, stream>>>(A);
-            count_launches(3);
-        }
+        const cudaError_t e = n64_forecast(gr, gm1, m, kappa, nsteps, stream);
+        if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }
