@@ -13,15 +13,13 @@
 #include <type_traits>
 #include <vector>
 
-#include <cooperative_groups.h>
-
 #include "analysis.h"
 #include "batch_analysis.h"
 #include "common.cuh"
+#include "spd_solve.cuh"
 #include "update_tc.h"
 
 namespace mgk {
-namespace cg = cooperative_groups;
 
 static inline int grid_for(size_t n, int block, int cap = 8 * kNumSMs) {
     long long g = (long long)((n + block - 1) / block);
@@ -752,27 +750,19 @@ void launch_gemm_tn_f64(const double *Y, int ne, int ny, double diag, double *C,
 }
 
 // ---------------------------------------------------------------------------
-// Cholesky (right-looking, one CTA) and the two triangular solves
+// SPD solves: up to order 256 spd_solve.cuh, above (direct form) a Cholesky
+// factorisation in global memory by one CTA and a substitution per column
 // ---------------------------------------------------------------------------
-template <bool SMEM>
-__device__ __forceinline__ void cholesky_body(double *A, double *Lt, int n, int *status) {
-    // Right-looking Cholesky by one CTA.  Column k: pivot l = sqrt(A_kk) and its
+__global__ void __launch_bounds__(256) k_cholesky(double *M, double *Lt, int n, int *status) {
+    // Right-looking Cholesky by one CTA.  Column k: pivot l = sqrt(M_kk) and its
     // reciprocal (one division per column), scale the column below it, then the
-    // rank-1 update of the trailing lower triangle.  Rows padded to n+1 doubles
-    // in shared memory.
-    extern __shared__ double sm[];
+    // rank-1 update of the trailing lower triangle.
     __shared__ double s_inv;
     if (*status) return;
     const int tid = threadIdx.x, nth = blockDim.x;
     const int tx = tid & 31, ty = tid >> 5, nty = nth >> 5;
-    const int ld = SMEM ? n + 1 : n;
-    double *M = SMEM ? sm : A;
-    if (SMEM) {
-        for (int e = tid; e < n * n; e += nth) sm[(e / n) * ld + e % n] = A[e];
-        __syncthreads();
-    }
     for (int k = 0; k < n; ++k) {
-        const double d = M[(size_t)k * ld + k];
+        const double d = M[(size_t)k * n + k];
         if (!(d > 0.0) || !isfinite(d)) {  // uniform: every thread read the same pivot
             if (tid == 0) atomicCAS(status, 0, kStNotSpd);
             return;
@@ -780,285 +770,75 @@ __device__ __forceinline__ void cholesky_body(double *A, double *Lt, int n, int 
         __syncthreads();  // every thread has read the pivot before it is overwritten
         if (tid == 0) {
             const double l = sqrt(d);
-            M[(size_t)k * ld + k] = l;
+            M[(size_t)k * n + k] = l;
             s_inv = 1.0 / l;
         }
         __syncthreads();
         const double inv = s_inv;
-        for (int i = k + 1 + tid; i < n; i += nth) M[(size_t)i * ld + k] *= inv;
+        for (int i = k + 1 + tid; i < n; i += nth) M[(size_t)i * n + k] *= inv;
         __syncthreads();
         for (int i = k + 1 + ty; i < n; i += nty) {
-            const double lik = M[(size_t)i * ld + k];
+            const double lik = M[(size_t)i * n + k];
             for (int j = k + 1 + tx; j <= i; j += 32)
-                M[(size_t)i * ld + j] = fma(-lik, M[(size_t)j * ld + k], M[(size_t)i * ld + j]);
+                M[(size_t)i * n + j] = fma(-lik, M[(size_t)j * n + k], M[(size_t)i * n + j]);
         }
         __syncthreads();
     }
     for (int e = tid; e < n * n; e += nth) {
         const int i = e / n, j = e % n;
-        const double val = j <= i ? M[(size_t)i * ld + j] : 0.0;
-        A[e] = val;
+        const double val = j <= i ? M[(size_t)i * n + j] : 0.0;
+        M[e] = val;
         Lt[(size_t)j * n + i] = val;
     }
 }
 
-template <bool SMEM>
-__global__ void __launch_bounds__(256) k_cholesky(double *A, double *Lt, int n, int *status) {
-    cholesky_body<SMEM>(A, Lt, n, status);
+template <int C>
+__global__ void __launch_bounds__(kSpdThreads) k_spd_factor(double *A, double *At, int n, int *status) {
+    spd_factor_body<C>(A, At, n, status);
 }
 
-// Cholesky by a cluster of 8 CTAs (n <= 256).  CTA q owns the columns
-// [q w, q w + w), w = ceil(n / 8), all n rows, in shared memory.  Panel p is
-// CTA p's block of columns.  For p = 0 .. 7: CTA p factors its panel column by
-// column (pivot sqrt and one reciprocal, scale the column, rank-1 update of
-// the panel's remaining columns; a ninth warp updates the next diagonal entry
-// and forms its pivot while the eight others update the rest, so the pivot's
-// FP64 chain is off the update's path); cluster barrier; every CTA q > p copies the
-// rows >= q w of panel p from CTA p's shared memory (distributed shared
-// memory) and subtracts the panel's rank-w product from its own columns.  One
-// cluster barrier per panel; the FP64 work of the trailing updates spreads
-// over 8 SMs.  A non-positive pivot sets the status and the kernel runs to
-// the end (every CTA must reach every cluster barrier) without writing L.
-constexpr int kCholCluster = 8;
-
-// y = 1/sqrt(d) for a Cholesky pivot: FP32 rsqrtf seed, then two Newton steps
-// y <- y (3 - d y^2) / 2 in FP64 (each squares the relative error: 2^-23 ->
-// 2^-46 -> FP64 rounding).  A pivot that is not positive and finite sets the
-// status and yields y = 1 so the factorisation runs on without dividing.
-__device__ __forceinline__ void chol_pivot(double d, double *y_out, int *status, int *fail) {
-    if (!(d > 0.0) || !isfinite(d)) {
-        atomicCAS(status, 0, kStNotSpd);
-        *fail = 1;
-        *y_out = 1.0;
-        return;
-    }
-    double y;
-    if (d > 1e-30 && d < 1e30) {
-        y = (double)rsqrtf((float)d);
-        y = y * fma(-0.5 * d, y * y, 1.5);
-        y = y * fma(-0.5 * d, y * y, 1.5);
-    } else {
-        y = 1.0 / sqrt(d);
-    }
-    *y_out = y;
+template <int C>
+static void spd_factor_launch(double *A, double *At, int n, int *status, cudaStream_t s) {
+    static OncePerDevice attr;
+    attr.run([](int) {
+        cudaError_t e = cudaFuncSetAttribute(k_spd_factor<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)spd_factor_smem(kSpdMax, C));
+        if (e == cudaSuccess && C > 8)
+            e = cudaFuncSetAttribute(k_spd_factor<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        return e;
+    });
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(kSpdThreads);
+    cfg.dynamicSmemBytes = spd_factor_smem(n, C);
+    cfg.stream = s;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeClusterDimension;
+    a[0].val.clusterDim.x = C;
+    a[0].val.clusterDim.y = 1;
+    a[0].val.clusterDim.z = 1;
+    cfg.attrs = a;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_spd_factor<C>, A, At, n, status);
 }
 
-__device__ __forceinline__ void cholesky_cluster_body(double *A, double *Lt, int n, int *status) {
-    extern __shared__ double csm[];
-    __shared__ int s_fail;
-    __shared__ double s_y[32];  // 1/sqrt of the panel's pivots
-    cg::cluster_group cl = cg::this_cluster();
-    if (*status) return;  // every CTA reads it before any CTA can write it (after the first barrier)
-    const int q = (int)cl.block_rank();
-    const int w = (n + kCholCluster - 1) / kCholCluster, ldp = w + 1;
-    const int c0 = q * w, c1 = min(n, c0 + w), wq = max(0, c1 - c0);
-    const int tid = threadIdx.x, nth = blockDim.x;
-    // 2-D view of the CTA for column-parallel loops: nx2 column lanes x ny2 row lanes
-    const int nupd = 256, kPiv = 256;  // threads [0, 256) update, thread 256 forms the pivots
-    const int nx2 = w <= 8 ? 8 : (w <= 16 ? 16 : 32), ny2 = nupd / nx2;
-    const int tx2 = tid % nx2, ty2 = tid / nx2;
-    double *P = csm;             // [n][ldp]: rows of this CTA's columns
-    double *Lp = csm + n * ldp;  // [n][ldp]: copy of the panel being applied
-    if (tid == 0) s_fail = 0;
-    for (int e = tid; e < n * wq; e += nth) {
-        const int i = e / wq, c = e - i * wq;
-        P[i * ldp + c] = A[(size_t)i * n + c0 + c];
-    }
-    cl.sync();
-    for (int p = 0; p < kCholCluster; ++p) {
-        const int pc0 = p * w, wp = min(n, pc0 + w) - pc0;
-        if (wp <= 0) break;  // the same for every CTA
-        if (q == p) {
-            // Outer-product form on unscaled columns: with d_k the pivot,
-            // A_ij -= A_ik A_jk / d_k for the panel's later columns, one barrier
-            // per column.  The thread that updates the next diagonal entry
-            // (thread 0) forms that pivot's 1/sqrt(d) at once; the square roots
-            // and column scalings follow once per panel.
-            __syncthreads();
-            if (tid == kPiv) chol_pivot(P[pc0 * ldp], &s_y[0], status, &s_fail);
-            for (int c = 0; c < wp; ++c) {
-                const int k = pc0 + c;
-                __syncthreads();
-                const double y = s_y[c], idk = y * y;
-                if (tid < nupd) {
-                    // thread (tx, ty): panel column c + 1 + tx, rows k + 1 + ty, + ny, ... (rows >= that column)
-                    const int cc = c + 1 + tx2;
-                    if (cc < wp) {
-                        const int r = pc0 + cc;
-                        const double ljk = P[r * ldp + c] * idk;
-                        for (int ii = k + 1 + ty2; ii < n; ii += ny2)
-                            if (ii > r || (ii == r && cc != c + 1)) P[ii * ldp + cc] = fma(-P[ii * ldp + c], ljk, P[ii * ldp + cc]);
-                    }
-                } else if (tid == kPiv && c + 1 < wp) {
-                    // the next diagonal entry, updated here, and its pivot
-                    const int r = k + 1;
-                    const double ljk = P[r * ldp + c] * idk;
-                    const double dn = fma(-P[r * ldp + c], ljk, P[r * ldp + c + 1]);
-                    P[r * ldp + c + 1] = dn;
-                    chol_pivot(dn, &s_y[c + 1], status, &s_fail);
-                }
-            }
-            __syncthreads();
-            // L_ik = A_ik / sqrt(d_k) below the diagonal, L_kk = sqrt(d_k) = d_k y_k
-            for (int e = tid; e < n * wp; e += nth) {
-                const int i = e / wp, c = e - i * wp, k = pc0 + c;
-                if (i > k) P[i * ldp + c] *= s_y[c];
-            }
-            __syncthreads();
-            for (int c = tid; c < wp; c += nth) {
-                const int k = pc0 + c;
-                const double d = P[k * ldp + c];
-                P[k * ldp + c] = (d > 0.0 && isfinite(d)) ? d * s_y[c] : 1.0;
-            }
-        }
-        cl.sync();
-        if (q > p && wq > 0) {
-            const double *rp = cl.map_shared_rank(P, p);
-            for (int e = tid; e < (n - c0) * wp; e += nth) {
-                const int i = c0 + e / wp, c = e % wp;
-                Lp[i * ldp + c] = rp[i * ldp + c];
-            }
-            __syncthreads();
-            // thread (tx, ty): own column jj = tx, tx + nx2, ...; rows j + ty, + ny2, ...
-            for (int jj = tx2; tid < nupd && jj < wq; jj += nx2) {
-                const int j = c0 + jj;
-                for (int i = j + ty2; i < n; i += ny2) {
-                    double acc = P[i * ldp + jj];
-                    for (int c = 0; c < wp; ++c) acc = fma(-Lp[i * ldp + c], Lp[j * ldp + c], acc);
-                    P[i * ldp + jj] = acc;
-                }
-            }
-        }
-    }
-    __syncthreads();
-    if (!s_fail && !*status) {
-        for (int e = tid; e < n * wq; e += nth) {
-            const int i = e / wq, c = e - i * wq, j = c0 + c;
-            const double val = i >= j ? P[i * ldp + c] : 0.0;
-            A[(size_t)i * n + j] = val;
-            Lt[(size_t)j * n + i] = val;
-        }
-    }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
+__global__ void __launch_bounds__(kSpdThreads) k_spd_apply(const double *__restrict__ A, const double *__restrict__ At,
+                                                           int n, const double *rhs, double *out, int ncol,
+                                                           __nv_bfloat16 *out16, int ld16, const int *status) {
+    spd_apply_body<1>(A, At, n, rhs, out, ncol, out16, ld16, status, blockIdx.x);
 }
 
-__global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(288)
-    k_cholesky_cluster(double *A, double *Lt, int n, int *status) {
-    cholesky_cluster_body(A, Lt, n, status);
-}
-
-// dynamic shared memory of the clustered Cholesky of order n
-static size_t cholesky_cluster_smem(int n) {
-    return sizeof(double) * 2 * (size_t)n * ((n + kCholCluster - 1) / kCholCluster + 1);
-}
-
-void launch_cholesky(double *A, double *Lt, int n, int *status, cudaStream_t s) {
+void launch_spd_factor(double *A, double *At, int n, int *status, cudaStream_t s) {
     count_launches(1);
-    if (n >= 32 && n <= 256) {
-        const size_t bytes = cholesky_cluster_smem(n);
-        static OncePerDevice attr;
-        attr.run([](int) {
-            return cudaFuncSetAttribute(k_cholesky_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-        });
-        k_cholesky_cluster<<<kCholCluster, 288, bytes, s>>>(A, Lt, n, status);
-        return;
-    }
-    const size_t bytes = sizeof(double) * (size_t)n * (n + 1);
-    if (bytes <= 210 * 1024) {
-        static OncePerDevice attr;
-        attr.run([](int) {
-            return cudaFuncSetAttribute(k_cholesky<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
-        });
-        k_cholesky<true><<<1, 256, bytes, s>>>(A, Lt, n, status);
+    if (n <= kSpdMax) {
+        if (spd_cluster(n) == 16)
+            spd_factor_launch<16>(A, At, n, status, s);
+        else
+            spd_factor_launch<8>(A, At, n, status, s);
     } else {
-        k_cholesky<false><<<1, 256, 0, s>>>(A, Lt, n, status);
+        k_cholesky<<<1, 256, 0, s>>>(A, At, n, status);
     }
 }
-
-// Triangular solves with the factor staged in shared memory: one warp per
-// right-hand side, lanes own rows lane + 32 m.  A CTA solves the columns
-// c0 .. c0 + ncols - 1 (warp w: column c0 + w): one column per CTA spreads the
-// FP64 work of one problem's columns over the SMs; the grouped analysis of many
-// problems gives each CTA several columns, so the factor is staged once for them.
-template <int MAXR>
-__device__ __forceinline__ void chol_solve_body(const double *__restrict__ L, int n, const double *rhs, double *out,
-                                                int ncol, __nv_bfloat16 *out16, int ld16, const int *status, int c0,
-                                                int ncols) {
-    // the CTA stages the unit lower factor U = L D^-1 (D = diag L) in shared
-    // memory, then each solving warp runs both substitutions for its
-    // right-hand side: S x = U D^2 U^T x = b as U y = b, then U^T x = D^-2 y.
-    // With the unit diagonal no step of either substitution waits on an FP64
-    // multiplication before its broadcast.
-    extern __shared__ double sL[];  // [n][n+1]: U strictly below the diagonal; then inv_diag[n]
-    if (*status) return;
-    const int c = c0 + (threadIdx.x >> 5), lane = threadIdx.x & 31, ld = n + 1;
-    double *inv = sL + (size_t)n * ld;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) inv[j] = 1.0 / L[(size_t)j * n + j];
-    __syncthreads();
-    for (int i = threadIdx.x >> 5; i < n; i += blockDim.x >> 5)
-        for (int j = lane; j < i; j += 32) sL[(size_t)i * ld + j] = L[(size_t)i * n + j] * inv[j];
-    __syncthreads();
-    if ((threadIdx.x >> 5) >= ncols || c >= ncol) return;
-    double b[MAXR];
-#pragma unroll
-    for (int m = 0; m < MAXR; ++m) {
-        const int i = lane + 32 * m;
-        b[m] = i < n ? rhs[(size_t)c * n + i] : 0.0;
-    }
-    // forward, column by column: y_j is final once the columns before j are applied
-#pragma unroll
-    for (int s = 0; s < MAXR; ++s) {
-        if (s * 32 >= n) break;
-        for (int l = 0; l < 32; ++l) {
-            const int j = s * 32 + l;
-            if (j >= n) break;
-            const double yj = __shfl_sync(0xffffffffu, b[s], l);
-#pragma unroll
-            for (int m = s; m < MAXR; ++m) {
-                const int i = lane + 32 * m;
-                if (i > j && i < n) b[m] = fma(-sL[(size_t)i * ld + j], yj, b[m]);
-            }
-        }
-    }
-    // right-hand side of the backward substitution: D^-2 y
-#pragma unroll
-    for (int m = 0; m < MAXR; ++m) {
-        const int i = lane + 32 * m;
-        if (i < n) b[m] *= inv[i] * inv[i];
-    }
-#pragma unroll
-    for (int s = MAXR - 1; s >= 0; --s) {
-        if (s * 32 >= n) continue;
-        for (int l = 31; l >= 0; --l) {
-            const int j = s * 32 + l;
-            if (j >= n) continue;
-            const double xj = __shfl_sync(0xffffffffu, b[s], l);
-#pragma unroll
-            for (int m = 0; m <= s; ++m) {
-                const int i = lane + 32 * m;
-                if (i < j) b[m] = fma(-sL[(size_t)j * ld + i], xj, b[m]);
-            }
-        }
-    }
-#pragma unroll
-    for (int m = 0; m < MAXR; ++m) {
-        const int i = lane + 32 * m;
-        if (i < n) {
-            out[(size_t)c * n + i] = b[m];
-            if (out16) out16[(size_t)c * ld16 + i] = __double2bfloat16(b[m]);
-        }
-    }
-}
-
-template <int MAXR>
-__global__ void __launch_bounds__(256) k_chol_solve_smem(const double *__restrict__ L, int n, const double *rhs,
-                                                         double *out, int ncol, __nv_bfloat16 *out16, int ld16,
-                                                         const int *status) {
-    chol_solve_body<MAXR>(L, n, rhs, out, ncol, out16, ld16, status, blockIdx.x, 1);
-}
-
-// shared memory of the staged factor of order n
-static size_t chol_solve_smem(int n) { return sizeof(double) * ((size_t)n * (n + 1) + n); }
 
 template <int MAXR>
 __global__ void __launch_bounds__(32) k_chol_solve(const double *__restrict__ L,
@@ -1118,33 +898,15 @@ __global__ void __launch_bounds__(32) k_chol_solve(const double *__restrict__ L,
     }
 }
 
-void launch_chol_solve(const double *L, const double *Lt, int n, const double *rhs, double *out,
-                       int ncol, __nv_bfloat16 *out16, int ld16, const int *status, cudaStream_t s) {
+void launch_spd_solve(const double *A, const double *At, int n, const double *rhs, double *out, int ncol,
+                      __nv_bfloat16 *out16, int ld16, const int *status, cudaStream_t s) {
     count_launches(1);
-    const size_t smem = chol_solve_smem(n);
-    if (n <= 160 && smem <= 210 * 1024) {
-        static OncePerDevice attr[2];
-        if (n <= 128) {
-            attr[0].run([](int) {
-                return cudaFuncSetAttribute(k_chol_solve_smem<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            210 * 1024);
-            });
-            k_chol_solve_smem<4><<<ncol, 256, smem, s>>>(L, n, rhs, out, ncol, out16, ld16, status);
-        } else {
-            attr[1].run([](int) {
-                return cudaFuncSetAttribute(k_chol_solve_smem<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            210 * 1024);
-            });
-            k_chol_solve_smem<8><<<ncol, 256, smem, s>>>(L, n, rhs, out, ncol, out16, ld16, status);
-        }
-        return;
-    }
-    if (n <= 128)
-        k_chol_solve<4><<<ncol, 32, 0, s>>>(L, Lt, n, rhs, out, ncol, out16, ld16, status);
+    if (n <= kSpdMax)
+        k_spd_apply<<<ncol, kSpdThreads, 0, s>>>(A, At, n, rhs, out, ncol, out16, ld16, status);
     else if (n <= 512)
-        k_chol_solve<16><<<ncol, 32, 0, s>>>(L, Lt, n, rhs, out, ncol, out16, ld16, status);
+        k_chol_solve<16><<<ncol, 32, 0, s>>>(A, At, n, rhs, out, ncol, out16, ld16, status);
     else
-        k_chol_solve<64><<<ncol, 32, 0, s>>>(L, Lt, n, rhs, out, ncol, out16, ld16, status);
+        k_chol_solve<64><<<ncol, 32, 0, s>>>(A, At, n, rhs, out, ncol, out16, ld16, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -1547,24 +1309,18 @@ __global__ void __launch_bounds__(256) kg_gemm_reduce(const GroupProb *__restric
 }
 
 // cluster c = blocks 8 c .. 8 c + 7, all of one problem (map entry per cluster)
-__global__ void __cluster_dims__(kCholCluster, 1, 1) __launch_bounds__(288)
-    kg_cholesky_cluster(const GroupProb *__restrict__ P, const int2 *__restrict__ map) {
-    const GroupProb &g = P[map[blockIdx.x / kCholCluster].x];
-    cholesky_cluster_body(g.S, g.Lt, g.ne, g.status);
+__global__ void __cluster_dims__(kSpdGroupCluster, 1, 1) __launch_bounds__(kSpdThreads)
+    kg_spd_factor(const GroupProb *__restrict__ P, const int2 *__restrict__ map) {
+    const GroupProb &g = P[map[blockIdx.x / kSpdGroupCluster].x];
+    spd_factor_body<kSpdGroupCluster>(g.S, g.Lt, g.ne, g.status);
 }
 
-__global__ void __launch_bounds__(256) kg_cholesky(const GroupProb *__restrict__ P, const int2 *__restrict__ map) {
-    const GroupProb &g = P[map[blockIdx.x].x];
-    cholesky_body<true>(g.S, g.Lt, g.ne, g.status);
-}
-
-template <int MAXR>
-__global__ void __launch_bounds__(32 * kSolveColsPerCta)
-    kg_chol_solve(const GroupProb *__restrict__ P, const int2 *__restrict__ map) {
+__global__ void __launch_bounds__(kSpdThreads)
+    kg_spd_apply(const GroupProb *__restrict__ P, const int2 *__restrict__ map) {
     const int2 e = map[blockIdx.x];
     const GroupProb &g = P[e.x];
-    chol_solve_body<MAXR>(g.S, g.ne, g.Bt, g.Bt, g.ne + 1, g.Tt, g.ldx, g.status, e.y * kSolveColsPerCta,
-                          kSolveColsPerCta);
+    spd_apply_body<kSolveColsPerCta>(g.S, g.Lt, g.ne, g.Bt, g.Bt, g.ne + 1, g.Tt, g.ldx, g.status,
+                                     e.y * kSolveColsPerCta);
 }
 
 // prolongation of the coarse intervals vj = kProlongIntervals e.y .. + 7 of
@@ -1598,9 +1354,8 @@ __global__ void __launch_bounds__(256) kg_prolong(const GroupProb *__restrict__ 
 }
 
 bool group_supported(int ne, int ny) {
-    // the solve's registers hold 32 MAXR rows (MAXR <= 8) and its staged
-    // factor fits shared memory; the anomalies' BF16 rows fit the update
-    return ne >= 2 && ne <= 160 && ny >= 1 && chol_solve_smem(ne) <= 210 * 1024;
+    // the BF16 rows of the anomalies and T fit the update's shared memory
+    return ne >= 2 && ne <= 160 && ny >= 1;
 }
 
 void group_plan_free(GroupPlan *plan) {
@@ -1635,25 +1390,12 @@ bool group_plan_build(GroupPlan *plan, const std::vector<GroupProb> &probs, cons
                     for (int bx = by; bx < tx; ++bx) m[kGsGemm].push_back(make_int2(j, (z * ty + by) * tx + bx));
         }
         if (g.splits > 1) add(kGsReduce, ceil_div((long long)g.ne * (2 * g.ne + 1), 256));
-        if (g.ne >= 32 && g.ne <= 256)
-            add(kGsCholCluster, 1);
-        else
-            add(kGsChol, 1);
+        add(kGsFactor, 1);
         add(kGsSolve, ceil_div(g.ne + 1, kSolveColsPerCta));
         add(kGsProlong, ceil_div(4 * g.nc, kProlongIntervals));
     }
     // launch shapes (the largest problem's shared memory)
-    plan->solve_maxr = maxne <= 128 ? 4 : 8;
-    plan->solve_smem = chol_solve_smem(maxne);
-    plan->chol_cluster_smem = 0;
-    plan->chol_smem = 0;
-    for (const GroupProb &g : probs) {
-        if (g.ne >= 32 && g.ne <= 256)
-            plan->chol_cluster_smem = std::max(plan->chol_cluster_smem, cholesky_cluster_smem(g.ne));
-        else
-            plan->chol_smem = std::max(plan->chol_smem, sizeof(double) * (size_t)g.ne * (g.ne + 1));
-    }
-    if (plan->chol_smem > 210 * 1024) return false;
+    plan->factor_smem = spd_factor_smem(maxne, kSpdGroupCluster);
     // update: problems grouped by the CTAs per SM their shared memory and TMEM
     // columns allow, one launch per group of at most kUpdateLaunchMax
     {
@@ -1728,15 +1470,9 @@ bool group_plan_build(GroupPlan *plan, const std::vector<GroupProb> &probs, cons
 
 cudaError_t group_analyse(const GroupPlan &plan, cudaStream_t s) {
     static OncePerDevice attr;
-    cudaError_t ae = attr.run([](int) {
-        cudaError_t e = cudaFuncSetAttribute(kg_cholesky_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kg_cholesky, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kg_chol_solve<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kg_chol_solve<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
-        return e;
+    const cudaError_t ae = attr.run([](int) {
+        return cudaFuncSetAttribute(kg_spd_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)spd_factor_smem(kSpdMax, kSpdGroupCluster));
     });
     if (ae != cudaSuccess) return ae;
     const GroupProb *P = plan.d_probs;
@@ -1754,15 +1490,9 @@ cudaError_t group_analyse(const GroupPlan &plan, cudaStream_t s) {
     if (step(kGsInnov)) kg_innov_rms<<<n(kGsInnov), 256, 0, s>>>(P, M(kGsInnov));
     if (step(kGsGemm)) kg_gemm<<<n(kGsGemm), kDfThreads, 0, s>>>(P, M(kGsGemm));
     if (step(kGsReduce)) kg_gemm_reduce<<<n(kGsReduce), 256, 0, s>>>(P, M(kGsReduce));
-    if (step(kGsCholCluster))
-        kg_cholesky_cluster<<<n(kGsCholCluster) * kCholCluster, 288, plan.chol_cluster_smem, s>>>(P, M(kGsCholCluster));
-    if (step(kGsChol)) kg_cholesky<<<n(kGsChol), 256, plan.chol_smem, s>>>(P, M(kGsChol));
-    if (step(kGsSolve)) {
-        if (plan.solve_maxr == 4)
-            kg_chol_solve<4><<<n(kGsSolve), 32 * kSolveColsPerCta, plan.solve_smem, s>>>(P, M(kGsSolve));
-        else
-            kg_chol_solve<8><<<n(kGsSolve), 32 * kSolveColsPerCta, plan.solve_smem, s>>>(P, M(kGsSolve));
-    }
+    if (step(kGsFactor))
+        kg_spd_factor<<<n(kGsFactor) * kSpdGroupCluster, kSpdThreads, plan.factor_smem, s>>>(P, M(kGsFactor));
+    if (step(kGsSolve)) kg_spd_apply<<<n(kGsSolve), kSpdThreads, 0, s>>>(P, M(kGsSolve));
     count_launches(launches);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

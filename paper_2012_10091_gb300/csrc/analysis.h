@@ -114,14 +114,16 @@ void launch_gemm_df(const DfOperands &df, int ne, int ny, double s2, double *S, 
 void launch_gemm_tn_f64(const double *Y, int ne, int ny, double diag, double *C, const int *status,
                         cudaStream_t s);
 
-// In-place Cholesky of the n x n SPD matrix A (row-major); writes L (lower,
-// row-major, upper zeroed) over A and its transpose to Lt.  Sets NOT_SPD.
-void launch_cholesky(double *A, double *Lt, int n, int *status, cudaStream_t s);
+// Factors the n x n SPD matrix A (row-major, lower triangle read) in place for
+// launch_spd_solve: L and its inverse's products for n <= 256 (spd_solve.cuh),
+// else the Cholesky factor; At receives the transpose.  Sets NOT_SPD.
+void launch_spd_factor(double *A, double *At, int n, int *status, cudaStream_t s);
 
-// Solve L L^T x_c = rhs_c for ncol columns of length n; x -> out (FP64) and,
-// if out16 != NULL, BF16 copy to out16 with row stride ld16.
-void launch_chol_solve(const double *L, const double *Lt, int n, const double *rhs, double *out,
-                       int ncol, __nv_bfloat16 *out16, int ld16, const int *status, cudaStream_t s);
+// Solves A0 x_c = rhs_c (A0 as given to launch_spd_factor) for ncol columns of
+// length n; x -> out (FP64; out = rhs is allowed) and, if out16 != NULL, BF16
+// copy to out16 with row stride ld16.
+void launch_spd_solve(const double *A, const double *At, int n, const double *rhs, double *out, int ncol,
+                      __nv_bfloat16 *out16, int ld16, const int *status, cudaStream_t s);
 
 // members[c] += X T[c] (c < ne), dC = X T[ne]   (T column c contiguous, (ne+1) x ne)
 template <typename T>

@@ -52,15 +52,14 @@ enum GroupStep {
     kGsInnov,        // RMS of d*
     kGsGemm,         // S and Y^T R^-1 [D | d*] in double-FP32 arithmetic (tiles or K chunks)
     kGsReduce,       // sum of the K chunks
-    kGsCholCluster,  // Cholesky of S, 8-CTA clusters (32 <= Ne <= 256)
-    kGsChol,         // Cholesky of S, one CTA (Ne < 32)
+    kGsFactor,       // S = L D L^T and L^-1, one 8-CTA cluster per problem
     kGsSolve,        // T = S^-1 [Y^T R^-1 D | Y^T R^-1 d*], BF16 copy
     kGsUpdate,       // anomalies X, members += X T_i, dC = X T_ne (tensor cores)
     kGsProlong,      // x^F += Pi_F(dC), analysis counter + 1
     kGsSteps
 };
 
-constexpr int kSolveColsPerCta = 8;  // right-hand sides per CTA of the grouped solve
+constexpr int kSolveColsPerCta = 4;  // right-hand sides per CTA of the grouped solve
 
 // host side of a grouped analysis: the device table, the block maps of every
 // step and the launch shapes
@@ -69,8 +68,7 @@ struct GroupPlan {
     int2 *d_maps = nullptr;  // all steps' maps, one allocation: entry = (problem, block of the problem)
     int nprob = 0;
     int map_off[kGsSteps] = {}, nblocks[kGsSteps] = {};
-    size_t chol_cluster_smem = 0, chol_smem = 0, solve_smem = 0;
-    int solve_maxr = 4;
+    size_t factor_smem = 0;  // the largest problem's
     // update: one launch per class of problems that fit the same number of
     // CTAs per SM (at most kUpdateLaunchMax problems each), over the tiles
     // [map_begin, map_end) of the update map (entry = (index in probs, tile))

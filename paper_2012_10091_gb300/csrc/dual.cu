@@ -193,8 +193,8 @@ void gain_solve(mgenkf_dual *d, int gen_eps, const double *xstar) {
                        ny, d->Y, d->Z, s);
     const double s2 = d->cfg.obs_sigma * d->cfg.obs_sigma;
     launch_gemm_nt_f64(d->Y, ne, d->Y, ne, d->Z, ne + 1, ny, s2, 1.0, d->S, d->Bt, d->status, s, d->part);
-    launch_cholesky(d->S, d->Lt, ne, d->status, s);
-    launch_chol_solve(d->S, d->Lt, ne, d->Bt, d->Bt, ne + 1, nullptr, 0, d->status, s);
+    launch_spd_factor(d->S, d->Lt, ne, d->status, s);
+    launch_spd_solve(d->S, d->Lt, ne, d->Bt, d->Bt, ne + 1, nullptr, 0, d->status, s);
 }
 
 }  // namespace

@@ -120,8 +120,8 @@ extern "C" mgenkf_status mgk_gain_ensemble_noalloc(const double *Y, const double
     if (e == cudaSuccess) {
         const double s2 = obs_sigma * obs_sigma;
         mgk::launch_gemm_nt_f64(Y, ne, Y, ne, Z, ne + 1, n_obs, s2, 1.0, S, T, status, s);
-        mgk::launch_cholesky(S, Lt, ne, status, s);
-        mgk::launch_chol_solve(S, Lt, ne, T, T, ne + 1, nullptr, 0, status, s);
+        mgk::launch_spd_factor(S, Lt, ne, status, s);
+        mgk::launch_spd_solve(S, Lt, ne, T, T, ne + 1, nullptr, 0, status, s);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && info) e = cudaMemcpyAsync(info, status, sizeof(int), cudaMemcpyDeviceToDevice, s);

@@ -769,14 +769,14 @@ static void analyse_kernels(mgenkf_ctx *h, int gen_eps) {
         else
             launch_gemm_nt_f64(h->Y, ne, h->Y, ne, h->Z, ne + 1, ny, s2, 1.0, h->S, h->Bt, h->status, s,
                                h->gemm_part);
-        launch_cholesky(h->S, h->Lt, ne, h->status, s);
-        launch_chol_solve(h->S, h->Lt, ne, h->Bt, h->Bt, ne + 1, h->mixed ? h->Tt : nullptr, h->ldx,
+        launch_spd_factor(h->S, h->Lt, ne, h->status, s);
+        launch_spd_solve(h->S, h->Lt, ne, h->Bt, h->Bt, ne + 1, h->mixed ? h->Tt : nullptr, h->ldx,
                           h->status, s);
     } else {
         // C = Y Y^T + R (ny x ny), W = C^-1 [D | d*], T = Y^T W
         launch_gemm_tn_f64(h->Y, ne, ny, s2, h->C, h->status, s);
-        launch_cholesky(h->C, h->Ct, ny, h->status, s);
-        launch_chol_solve(h->C, h->Ct, ny, h->Z, h->W, ne + 1, nullptr, 0, h->status, s);
+        launch_spd_factor(h->C, h->Ct, ny, h->status, s);
+        launch_spd_solve(h->C, h->Ct, ny, h->Z, h->W, ne + 1, nullptr, 0, h->status, s);
         launch_gemm_nt_f64(h->Y, ne, nullptr, 0, h->W, ne + 1, ny, 1.0, 0.0, nullptr, h->Tm, h->status, s,
                            h->gemm_part);
         if (h->mixed) launch_tt_bf16(h->Tm, h->Tt, ne, h->ldx, h->status, s);
