@@ -112,8 +112,7 @@ mgenkf_status mgenkf_forecast(mgenkf_handle h, int32_t nsteps);
  * then run on two streams), or -1 for both grids: the 2-D tile kernel, both
  * grids in one launch per model step.  The per-point arithmetic, and so every
  * result, is the same for all choices.  The default is set at create from the
- * grid sizes: narrow bands above 256 points per side and the longest segments
- * that still give each grid two units per SM.
+ * grid sizes and the member count: the least estimated time of both grids.
  * mgenkf_forecast_autotune times `reps` repetitions (after one warm-up) of
  * ten model steps written to the stage buffers (the states are not touched)
  * for every choice, each grid alone, then both at once as the forecast runs
@@ -330,8 +329,9 @@ mgenkf_status mgenkf_batch_sync(mgenkf_batch_t b);
  * forecast and keep the fastest.  A choice c in [0, 16) sets the rows per
  * segment of the column march (c mod 8: 0 = 32, 1 = 16, 2 = 64, 3 = 128,
  * 4 = 256, 5 = 24, 6 = 48, 7 = 20) and its band width (c / 8: 0 = the whole
- * width up to 512 points per side, 1 = bands of at most 122 columns with
- * recomputed 3-column halos, about 64 threads per CTA).
+ * width up to 256 points per side, 1 = bands of at most 122 columns with
+ * recomputed 3-column halos, at most 128 threads per CTA); the default is the
+ * least estimated time of all sizes stepping at once.
  * Then, size by size from the slowest, every choice is timed again with all
  * grid sizes stepping at once on their own streams, as the forecast runs them,
  * and the fastest joint choice is kept.  The arithmetic does not depend on the

@@ -39,6 +39,7 @@
 #include <cstdint>
 #include <cstring>
 #include <algorithm>
+#include <vector>
 #include <type_traits>
 
 #include "common.cuh"
@@ -318,8 +319,28 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
     memcpy(&d, &rd, 8);
     return d;
 }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+// a b.  A product that goes into one sum only becomes a fused multiply-add of it
+// in the assembler, one with two uses does not; volatile keeps the compiler from
+// sharing a product between two rows of the march, so that each kernel rounds
+// every flux alike and the kernels agree bit for bit.
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    unsigned long long ra, rb, rd;
+    memcpy(&ra, &a, 8);
+    memcpy(&rb, &b, 8);
+    asm volatile("mul.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
+    float2 d;
+    memcpy(&d, &rd, 8);
+    return d;
+}
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// approximate reciprocal in one instruction (__fdividef(1, x) spends six more on
+// |x| above 2^126, where both give 0)
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 
 __device__ __forceinline__ int wrap_index(int g, int n) {
     if (g < 0) g += n;
@@ -330,6 +351,15 @@ __device__ __forceinline__ int wrap_index(int g, int n) {
     return g;
 }
 
+// 4-byte asynchronous global -> shared copy
+__device__ __forceinline__ void cp_async4(float *smem, const float *gmem) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(gmem) : "memory");
+}
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
 // 16-byte asynchronous global -> shared copy (L2 only: each chunk is read once per tile)
 __device__ __forceinline__ void cp_async16(void *smem, const float *gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -460,7 +490,7 @@ __device__ __forceinline__ void x2_rhs(const float2 *cons, const float2 *prim, i
 // reciprocal of rho per point)
 template <int HALO>
 __device__ __forceinline__ void put_prims(float2 *prim, int f, float2 rho, float2 mx, float2 my, float2 E, float gm1) {
-    const float2 rinv = make_float2(__fdividef(1.f, rho.x), __fdividef(1.f, rho.y));
+    const float2 rinv = make_float2(rcp_approx(rho.x), rcp_approx(rho.y));
     const float2 u = mul2(mx, rinv), v = mul2(my, rinv);
     const float2 ke = mul2(mul2(f2(0.5f), rho), fma2(u, u, mul2(v, v)));
     const float2 p = mul2(f2(gm1), sub2(E, ke));
@@ -551,9 +581,8 @@ __device__ __forceinline__ void step_stage(const float2 *Q0, float2 *QS, float2 
             x2_rhs<S::FX, NF>(cons, PR, f, d.inv_h, d.inv_2h, mu, kap, L);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float2 kq = mul2(dt, L[k]);
                 const float2 base = Q0[k * NF + f];
-                res[q][k] = K == 1 ? add2(base, kq) : fma2(f2(0.25f), add2(sub2(QS[k * NF + f], base), kq), base);
+                res[q][k] = K == 1 ? fma2(dt, L[k], base) : fma2(f2(0.25f), fma2(dt, L[k], sub2(QS[k * NF + f], base)), base);
             }
         }
     }
@@ -590,9 +619,8 @@ __device__ __forceinline__ void step_last(const float2 *Q0, const float2 *QS, co
         float *oa = d.out + ya * n + x, *ob = oa + H * n;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float2 kq = mul2(dt, L[k]);
             const float2 base = Q0[k * NF + f];
-            const float2 res = fma2(f2(2.f / 3.f), add2(sub2(QS[k * NF + f], base), kq), base);
+            const float2 res = fma2(f2(2.f / 3.f), fma2(dt, L[k], sub2(QS[k * NF + f], base)), base);
             oa[k * plane] = res.x;
             if (yb < n) ob[k * plane] = res.y;
         }
@@ -648,19 +676,26 @@ __global__ void __launch_bounds__(256, MINB)
 }
 
 // ---------------------------------------------------------------------------
-// The FP32 step as a column march.  A CTA owns a band of columns of one grid
-// and a segment of its rows; thread t owns the column pair (c0 + t, c0 + t +
-// T) as one float2 (T = blockDim.x).  With one band the pair spans the whole
-// periodic width (c0 = 0, 2T = n); with several bands (n > 512) each band
+// The FP32 step as a column march.  A unit (one CTA) is two row segments of
+// grids of one size, each a band of columns; thread t owns column c0 + t of
+// both, as the two halves of a float2, so that the neighbours of a pair are
+// pairs too (with two columns of one row in a pair the values at the fold had
+// to be swapped: 45 of 840 instructions a step).  With one band the T =
+// blockDim.x threads span the whole periodic width; with several each band
 // carries a 3-column halo on both sides, recomputed by its neighbours.  The
-// CTA marches down the rows of its segment: in step j it loads row j of the
-// step-start state (3 rows above the segment first), evaluates stage 1 one row
-// behind, stage 2 three rows behind and stage 3 five rows behind, and stores
-// the new state's row.  Each stage keeps the three rows of its input around
-// the row it evaluates in registers (its own columns); only the east and west
-// neighbours come from shared memory, through ring buffers of the last rows
-// each stage published (one barrier per step).  The face between two rows is
-// evaluated once and carried to the next row.
+// CTA marches down the rows of its segments: in step j it takes row j of the
+// step-start state (3 rows above the segment first; copied asynchronously three
+// steps ahead), evaluates stage 1 one row behind, stage 2 three rows behind and
+// stage 3 five rows behind, and stores the new state's row.  Each stage keeps
+// the three rows of its input around the row it evaluates in registers (its own
+// column); only the east and west neighbours come from shared memory, through
+// ring buffers of the last rows each stage published (one barrier per step).
+// The face between two rows is evaluated once and carried to the next row.
+// Bound by the latency of a step (one or two warps per scheduler, 40% of the
+// issue slots).  512^2 / 128^2 x 64 handle, 10 steps: 514 us with pairs of
+// columns, ring rows of a pitch known at run time and rows moved through the
+// register windows (840 instructions a step), 372 us as below (450); 24
+// problems of 64^2 .. 768^2: 8.13 and 6.2 ms with their analysis.
 // ---------------------------------------------------------------------------
 // one row of a stage input at the thread's column pair
 struct Rec {
@@ -675,7 +710,7 @@ __device__ __forceinline__ Rec make_rec(float2 rho, float2 mx, float2 my, float2
     r.mx = mx;
     r.my = my;
     r.E = E;
-    const float2 rinv = make_float2(__fdividef(1.f, rho.x), __fdividef(1.f, rho.y));
+    const float2 rinv = make_float2(rcp_approx(rho.x), rcp_approx(rho.y));
     r.U = mul2(mx, rinv);
     r.V = mul2(my, rinv);
     const float2 ke = mul2(mul2(f2(0.5f), rho), fma2(r.U, r.U, mul2(r.V, r.V)));
@@ -714,75 +749,58 @@ __device__ __forceinline__ Face face_y(float2 Ua, float2 Ub, float2 Va, float2 V
     return F;
 }
 
-// Shared ring buffers of the march, float2 per thread (T threads; each ring
-// row holds T + 2 pairs: slot t + 1 is thread t's pair, slot 0 the last
-// thread's pair and slot T + 1 the first thread's pair, both with their halves
-// swapped, so that the east and west neighbours across the fold are plain
-// loads):
-//   rows [4k + s]:           u of stage input k (k = 0 u0, 1 s1, 2 s2), ring slot s of 4
-//   rows [12 + 4k + s]:      v
-//   rows [24 + 12k + 3f + s]: rho u, E, p, T (f = 0..3) of stage input k, ring slot s of 3
-//   rows [60 + 4s + f]:      rho, rho u, rho v, E of u0, ring slot s of 8 (own column only)
-constexpr int kMarchRows = 92;
-// shared bytes of a march CTA of T threads
-__host__ __device__ __forceinline__ size_t march_smem_bytes(int threads) {
-    return sizeof(float2) * kMarchRows * (size_t)(threads + 2);
-}
+// Shared ring rows of the march: P pairs each (P >= T, a compile-time pitch, so
+// that every access is a register and an immediate), thread t's pair at slot t.
+// Three steps share a block of rows (slot i = j mod 3 within the block of step
+// j), and the blocks of a ring are taken in turn:
+//   u, v (v = 0, 1) of stage input k (k = 0 u0, 1 s1, 2 s2): two blocks of 18
+//     rows, row 6k + 3v + i
+//   rho u, E, p, T (f = 0..3) of stage input k: one block, row 12k + 3f + i
+//     (read one step after they are published)
+//   rho, rho u, rho v, E (q) of u0, own column only: three blocks of 12 rows,
+//     row 3q + i, filled asynchronously three steps ahead and kept for five
+constexpr int kMarchUV = 18, kMarchFlux = 2 * kMarchUV, kMarchU0 = kMarchFlux + 36, kMarchU0Block = 12;
+constexpr int kMarchRows = kMarchU0 + 3 * kMarchU0Block;
+constexpr int kMarchPitch[] = {32, 64, 96, 128, 192, 256};
+constexpr size_t march_smem_bytes(int pitch) { return sizeof(float2) * kMarchRows * (size_t)pitch; }
 constexpr int kMarchMaxThreads = 256;
-constexpr int kMarchBandMax = 2 * kMarchMaxThreads - 6;  // output columns of a band (even)
-constexpr int kMarchNarrowBand = 122;  // output columns of a narrow band: 64 threads per CTA
+constexpr int kMarchBandMax = kMarchMaxThreads - 6;  // output columns of a band
+constexpr int kMarchNarrowBand = 122;  // output columns of a narrow band: 128 threads per CTA
 
-// Thread t's slot in a ring row (row pitch T + 2), and the slot that holds its
-// pair swapped for the thread at the other end of the fold (-1: none).
-struct Slot {
-    int own, mirror;
+// a thread's places in the ring rows: its own slot, the east and the west
+// neighbour's (cyclic over the T columns)
+struct Ring {
+    float2 *own;
+    const float2 *e, *w;
 };
 
-__device__ __forceinline__ void put_pair(float2 *row, const Slot &sl, float2 v) {
-    row[sl.own] = v;
-    if (sl.mirror >= 0) row[sl.mirror] = make_float2(v.y, v.x);
-}
-
-__device__ __forceinline__ void march_publish(float2 *X, int P, const Slot &sl, int k, int j, const Rec &r) {
-    put_pair(X + (4 * k + (j & 3)) * P, sl, r.U);
-    put_pair(X + (12 + 4 * k + (j & 3)) * P, sl, r.V);
-    float2 *F = X + (24 + 12 * k + j % 3) * P;
-    put_pair(F, sl, r.mx);
-    put_pair(F + 3 * P, sl, r.E);
-    put_pair(F + 6 * P, sl, r.P);
-    put_pair(F + 9 * P, sl, r.T);
-}
-
-// east / west neighbour of the thread's pair in a ring row: the pair of thread
-// t + 1 (t - 1), across the fold the mirrored pair of the other end
-struct Nbr {
-    int te, tw;  // slots t + 2 and t
-    __device__ __forceinline__ float2 e(const float2 *row) const { return row[te]; }
-    __device__ __forceinline__ float2 w(const float2 *row) const { return row[tw]; }
-};
-
-// Stage input k, evaluated in step j at the centre row c of the window
-// (T: ring row pitch)
-// (m1, c, p1 published in steps j - 2, j - 1, j).  yf: in, the face between
-// m1 and c (carried from the previous step); out, the face between c and p1.
-// FULL = false computes only that face (the step before a stage's first row).
-template <bool FULL>
-__device__ __forceinline__ void march_rhs(const float2 *X, int T, const Nbr &nb, int k, int j, const Rec &m1,
-                                          const Rec &c, const Rec &p1, float inv_h, float inv_2h, float mu,
-                                          float kap, Face &yf, float2 (&L)[4]) {
-    const float2 *XU = X + 4 * k * T, *XV = X + (12 + 4 * k) * T;
-    const int sm = ((j - 2) & 3) * T, sc = ((j - 1) & 3) * T, sp = (j & 3) * T;
+// Stage input K, evaluated in step j (I = j mod 3) at the centre row c of the
+// window (m1, c, p1 published in steps j - 2, j - 1, j).  yf: in, the face
+// between m1 and c (carried from the previous step); out, the face between c
+// and p1.  FULL = false computes only that face (the step before a stage's
+// first row).  cur / prev: this step's block of ring rows and the other one.
+template <int P, int I, int K, bool FULL>
+__device__ __forceinline__ void march_rhs(const Ring &cur, const Ring &prev, const Ring &one, const Rec &m1,
+                                          const Rec &c, const Rec &p1, float inv_h, float inv_2h, float mu, float kap,
+                                          Face &yf, float2 (&L)[4]) {
+    // u (v = 0) and v (v = 1) of the east / west neighbour, d rows above p1
+    auto east = [&](int v, int d) {
+        return I >= d ? cur.e[(6 * K + 3 * v + I - d) * P] : prev.e[(6 * K + 3 * v + I - d + 3) * P];
+    };
+    auto west = [&](int v, int d) {
+        return I >= d ? cur.w[(6 * K + 3 * v + I - d) * P] : prev.w[(6 * K + 3 * v + I - d + 3) * P];
+    };
     const float2 k2 = f2(mu > 0.f ? 2.f * kap / mu : 0.f);
-    const float2 Uec = nb.e(XU + sc), Uwc = nb.w(XU + sc), Vec = nb.e(XV + sc), Vwc = nb.w(XV + sc);
-    const float2 Uep = nb.e(XU + sp), Uwp = nb.w(XU + sp), Vep = nb.e(XV + sp), Vwp = nb.w(XV + sp);
+    const float2 Uec = east(0, 1), Uwc = west(0, 1), Vec = east(1, 1), Vwc = west(1, 1);
+    const float2 Uep = east(0, 0), Uwp = west(0, 0), Vep = east(1, 0), Vwp = west(1, 0);
     // face between c and p1
     const Face top = face_y(c.U, p1.U, c.V, p1.V, add2(sub2(Uec, Uwc), sub2(Uep, Uwp)),
                             add2(sub2(Vec, Vwc), sub2(Vep, Vwp)), c.T, p1.T, k2);
     if (FULL) {
-        const float2 Uem = nb.e(XU + sm), Uwm = nb.w(XU + sm), Vem = nb.e(XV + sm), Vwm = nb.w(XV + sm);
-        const float2 *XF = X + (24 + 12 * k + (j - 1) % 3) * T;
-        const float2 mxe = nb.e(XF), mxw = nb.w(XF), Ee = nb.e(XF + 3 * T), Ew = nb.w(XF + 3 * T);
-        const float2 Pe = nb.e(XF + 6 * T), Pw = nb.w(XF + 6 * T), Te = nb.e(XF + 9 * T), Tw = nb.w(XF + 9 * T);
+        const float2 Uem = east(0, 2), Uwm = west(0, 2), Vem = east(1, 2), Vwm = west(1, 2);
+        constexpr int F = (kMarchFlux + 12 * K + (I + 2) % 3) * P, S = 3 * P;
+        const float2 mxe = one.e[F], mxw = one.w[F], Ee = one.e[F + S], Ew = one.w[F + S];
+        const float2 Pe = one.e[F + 2 * S], Pw = one.w[F + 2 * S], Te = one.e[F + 3 * S], Tw = one.w[F + 3 * S];
         // inviscid part: central differences of the nodal fluxes
         const float2 mi2h = f2(-inv_2h);
         const float2 myn = p1.my, mys = m1.my;
@@ -810,44 +828,45 @@ __device__ __forceinline__ void march_rhs(const float2 *X, int T, const Nbr &nb,
     yf = top;
 }
 
-// one unit of a march launch: a band and a row segment of one grid
-struct MarchUnit {
+// row segment of one grid: half of a unit (columns from c0, which may be
+// negative; rows from y0; columns t in [ilo, ihi) and `rows` rows are stored)
+struct MarchHalf {
     const float *in;  // step-start state of the grid (4 planes)
     float *out;       // state after the step
-    int n, c0, y0, rows;  // points per side, first column (may be negative), first row, rows of the segment
-    int ilo, ihi;         // output columns: pair index i (t or t + T) in [ilo, ihi)
+    int c0, y0, rows, ilo, ihi;
+};
+// one unit of a march launch: two row segments of grids of one size
+struct MarchUnit {
+    MarchHalf h[2];
+    int n, rows;  // points per side; rows of the longer half
     float inv_h, inv_2h, dt;
 };
 
 // bands and row segments of one n x n grid (host and device agree)
-// bands of at most kMarchBandMax columns (the whole width up to 512), or
+// bands of at most kMarchBandMax columns (the whole width up to 256), or
 // with `narrow` of at most kMarchNarrowBand (the whole width up to 128)
 __host__ __device__ __forceinline__ int march_bands(int n, bool narrow = false) {
     if (narrow) return n <= 128 ? 1 : (n + kMarchNarrowBand - 1) / kMarchNarrowBand;
-    return n <= 2 * kMarchMaxThreads ? 1 : (n + kMarchBandMax - 1) / kMarchBandMax;
+    return n <= kMarchMaxThreads ? 1 : (n + kMarchBandMax - 1) / kMarchBandMax;
 }
-__host__ __device__ __forceinline__ int march_band_width(int n, int bands) {
-    if (bands == 1) return n;
-    const int w = (n + bands - 1) / bands;
-    return w + (w & 1);
-}
+__host__ __device__ __forceinline__ int march_band_width(int n, int bands) { return (n + bands - 1) / bands; }
 __host__ __device__ __forceinline__ int march_threads(int n, bool narrow = false) {
     const int b = march_bands(n, narrow);
-    return b == 1 ? n / 2 : (march_band_width(n, b) + 6) / 2;
+    return b == 1 ? n : march_band_width(n, b) + 6;
 }
 
-__device__ __forceinline__ MarchUnit march_unit(const NsGroup<float> &G, int local, int parity) {
+// segment `id` of a group (grids, bands and row segments in that order)
+__device__ __forceinline__ MarchHalf march_half(const NsGroup<float> &G, int id, int parity) {
     const int per_grid = G.tx * G.ty;
-    const int prob = local / per_grid;
-    const int rem = local - prob * per_grid;
+    const int prob = id / per_grid;
+    const int rem = id - prob * per_grid;
     const int band = rem / G.ty, seg = rem - band * G.ty;
     const int n = G.n;
     const size_t off = (size_t)prob * 4 * n * n;
     float *u0 = G.u0 + off, *other = G.s1 + off;
-    MarchUnit u;
+    MarchHalf u;
     u.in = parity ? other : u0;
     u.out = parity ? u0 : other;
-    u.n = n;
     const int S = (n + G.ty - 1) / G.ty;
     u.y0 = seg * S;
     u.rows = min(S, n - u.y0);
@@ -861,6 +880,22 @@ __device__ __forceinline__ MarchUnit march_unit(const NsGroup<float> &G, int loc
         u.ilo = 3;
         u.ihi = 3 + min(bw, n - bx0);
     }
+    return u;
+}
+
+// unit `local` of a group: segments 2 local and 2 local + 1 (the last of an
+// odd count goes alone: its partner repeats it and stores nothing)
+__device__ __forceinline__ MarchUnit march_unit(const NsGroup<float> &G, int local, int parity) {
+    const int count = G.nprob * G.tx * G.ty;
+    MarchUnit u;
+    u.h[0] = march_half(G, 2 * local, parity);
+    u.h[1] = u.h[0];
+    if (2 * local + 1 < count)
+        u.h[1] = march_half(G, 2 * local + 1, parity);
+    else
+        u.h[1].rows = 0;
+    u.n = G.n;
+    u.rows = max(u.h[0].rows, u.h[1].rows);
     u.inv_h = G.inv_h;
     u.inv_2h = G.inv_2h;
     u.dt = G.dt;
@@ -868,180 +903,177 @@ __device__ __forceinline__ MarchUnit march_unit(const NsGroup<float> &G, int loc
 }
 
 // where the units of a launch come from: a device table of groups of one grid
-// size (batched path) or one group passed by value
-struct TableUnits {
+// size, or one group passed by value (groups == NULL)
+struct MarchUnits {
     const NsGroup<float> *groups;
     int ngroups;
+    NsGroup<float> one;
     __device__ __forceinline__ MarchUnit unit(int u, int parity) const {
+        if (!groups) return march_unit(one, u, parity);
         int gi = 0;
         while (gi + 1 < ngroups && groups[gi + 1].tile_begin <= u) ++gi;
         const NsGroup<float> G = groups[gi];
         return march_unit(G, u - G.tile_begin, parity);
     }
-    __device__ __forceinline__ NsGroup<float> group(int gi) const { return groups[gi]; }
+    __device__ __forceinline__ NsGroup<float> group(int gi) const { return groups ? groups[gi] : one; }
 };
-struct OneUnits {
-    NsGroup<float> g;
-    __device__ __forceinline__ MarchUnit unit(int u, int parity) const { return march_unit(g, u, parity); }
-    __device__ __forceinline__ NsGroup<float> group(int) const { return g; }
-};
+
+template <int V>
+using Int = std::integral_constant<int, V>;
 
 // One SSP-RK3 step of one unit per CTA (blockDim.x = march_threads(n) of the
 // launch's grid size).  Step j of the march: rows of u0 arrive in steps
-// 0 .. rows + 5 (rows y0 - 3 .. y0 + rows + 2); stage 1 evaluates row
-// y0 - 4 + j in steps 2 .. rows + 5, stage 2 row y0 - 6 + j in steps
+// 0 .. rows + 5 (rows y0 - 3 .. y0 + rows + 2 of each half); stage 1 evaluates
+// row y0 - 4 + j in steps 2 .. rows + 5, stage 2 row y0 - 6 + j in steps
 // 5 .. rows + 6, stage 3 row y0 - 8 + j in steps 8 .. rows + 7; a stage's
-// output row is published one step after it is computed.
-template <class Units>
-__global__ void __launch_bounds__(kMarchMaxThreads, 1)
-    ns2d_rk3_march(Units src, int parity, float gm1, float mu, float kap) {
+// output row is published one step after it is computed.  The steps go in
+// blocks of three, so that the rows of the register windows change their names
+// instead of moving (one at a time, a quarter of the instructions were moves).
+template <int P>
+__global__ void __launch_bounds__(P, 1) ns2d_rk3_march(MarchUnits src, int parity, float gm1, float mu, float kap) {
     extern __shared__ float4 march_smem4[];
     float2 *X = reinterpret_cast<float2 *>(march_smem4);
-    const int T = blockDim.x, t = threadIdx.x, P = T + 2;  // threads, ring row pitch
-    // Steps follow one another with programmatic serialisation (see
-    // march_launch): the next step may be scheduled from here on; each CTA
-    // decodes its unit (static tables only) before it waits for the previous
-    // launch to complete and its writes to be visible.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int T = blockDim.x, t = threadIdx.x;
     const MarchUnit u = src.unit(blockIdx.x, parity);
-    Nbr nb;
-    nb.te = t + 2;
-    nb.tw = t;
-    Slot sl;
-    sl.own = t + 1;
-    sl.mirror = t == 0 ? T + 1 : (t == T - 1 ? 0 : -1);
-    if (T == 1) sl.mirror = -1;  // never: T = n/2 >= 4
     const int n = u.n, plane = n * n;  // 4 planes of one grid stay below 2^31 elements
-    const int xa = wrap_index(u.c0 + t, n), xb = wrap_index(u.c0 + t + T, n);
-    const bool wa = t >= u.ilo && t < u.ihi, wb = t + T >= u.ilo && t + T < u.ihi;
     const int R = u.rows;
+    const Ring one{X + t, X + (t + 1 == T ? 0 : t + 1), X + (t == 0 ? T - 1 : t - 1)};
+    Ring cur = one, prev{one.own + kMarchUV * P, one.e + kMarchUV * P, one.w + kMarchUV * P};
+    // u0's blocks: this step's, the previous and the next one (also the one before the previous)
+    float2 *q0 = one.own + kMarchU0 * P, *qnext = q0 + kMarchU0Block * P, *qprev = qnext + kMarchU0Block * P;
+    const int xa = wrap_index(u.h[0].c0 + t, n), xb = wrap_index(u.h[1].c0 + t, n);
+    // elements of the next row to load and of the next row to store, per half
+    int ia = wrap_index(u.h[0].y0 - 3, n) * n + xa, ib = wrap_index(u.h[1].y0 - 3, n) * n + xb;
+    int oa = u.h[0].y0 * n + xa, ob = u.h[1].y0 * n + xb;
+    // last step in which this thread stores
+    const int enda = t >= u.h[0].ilo && t < u.h[0].ihi ? u.h[0].rows + 8 : 0;
+    const int endb = t >= u.h[1].ilo && t < u.h[1].ihi ? u.h[1].rows + 8 : 0;
+    // Steps follow one another with programmatic serialisation (march_launch):
+    // each CTA has decoded its unit (static tables only); the previous launch has
+    // completed and its writes are visible from here on, and only then may the
+    // next one be placed: placed earlier, its CTAs take the SMs that drain first
+    // and leave others idle (512^2 / 128^2 handle, 10 steps: 514 against 479 us).
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    float ld[8];  // the next u0 row at the two columns: rho, rho u, rho v, E
-    auto load_row = [&](int j) {
-        const float *p = u.in + wrap_index(u.y0 - 3 + j, n) * n;
+    // issue the copies of the next row of u0 into a row of a block
+    auto load_row = [&](float2 *row) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            ld[2 * q] = __ldg(p + q * plane + xa);
-            ld[2 * q + 1] = __ldg(p + q * plane + xb);
+            cp_async4(&row[3 * q * P].x, u.h[0].in + q * plane + ia);
+            cp_async4(&row[3 * q * P].y, u.h[1].in + q * plane + ib);
+        }
+        ia += n;
+        ib += n;
+        if (ia >= plane) ia -= plane;
+        if (ib >= plane) ib -= plane;
+    };
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        load_row(q0 + i * P);
+        cp_async_commit();
+    }
+    const float2 dt = f2(u.dt);
+    // rows of u0, s1, s2 by their step (mod 3): A[j % 3] arrived in step j,
+    // B[j % 3] and C[j % 3] were computed in it
+    Rec A[3] = {}, B[3] = {}, C[3] = {};
+    Face yf1{}, yf2{}, yf3{};  // carried faces
+
+    // step j (I = j mod 3); STEADY: all stages run
+    auto step = [&](auto I_, auto STEADY_, int j) {
+        constexpr int I = decltype(I_)::value, I1 = (I + 1) % 3, I2 = (I + 2) % 3;
+        constexpr bool STEADY = decltype(STEADY_)::value;
+        auto publish = [&](auto K_, const Rec &r) {
+            constexpr int K = decltype(K_)::value, F = (kMarchFlux + 12 * K + I) * P, S = 3 * P;
+            cur.own[(6 * K + I) * P] = r.U;
+            cur.own[(6 * K + 3 + I) * P] = r.V;
+            one.own[F] = r.mx;
+            one.own[F + S] = r.E;
+            one.own[F + 2 * S] = r.P;
+            one.own[F + 3 * S] = r.T;
+        };
+        // the rows that arrive in this step (a thread copies its own column)
+        cp_async_wait<2>();
+        if (STEADY || j <= R + 5) {
+            const float2 *r = q0 + I * P;
+            A[I] = make_rec(r[0], r[3 * P], r[6 * P], r[9 * P], gm1);
+            publish(Int<0>{}, A[I]);
+        }
+        if (STEADY || (j >= 3 && j <= R + 6)) publish(Int<1>{}, B[I2]);
+        if (STEADY || (j >= 6 && j <= R + 7)) publish(Int<2>{}, C[I2]);
+        __syncthreads();
+        if (STEADY || j + 3 <= R + 5) load_row(qnext + I * P);
+        cp_async_commit();
+
+        float2 L3[4], L2[4], L1[4];
+        // in the steady state the three stages run without a branch between them:
+        // their ILP hides the latency (one or two warps per scheduler)
+        if constexpr (!STEADY && I == 1) {
+            if (j == 7) march_rhs<P, I, 2, false>(cur, prev, one, C[I], C[I1], C[I2], u.inv_h, u.inv_2h, mu, kap, yf3, L3);
+            if (j == 4) march_rhs<P, I, 1, false>(cur, prev, one, B[I], B[I1], B[I2], u.inv_h, u.inv_2h, mu, kap, yf2, L2);
+            if (j == 1) march_rhs<P, I, 0, false>(cur, prev, one, A[I1], A[I2], A[I], u.inv_h, u.inv_2h, mu, kap, yf1, L1);
+        }
+        const bool run3 = STEADY || j >= 8, run2 = STEADY || (j >= 5 && j <= R + 6),
+                   run1 = STEADY || (j >= 2 && j <= R + 5);
+        if (run3) march_rhs<P, I, 2, true>(cur, prev, one, C[I], C[I1], C[I2], u.inv_h, u.inv_2h, mu, kap, yf3, L3);
+        if (run3) {  // the new state's row y0 - 8 + j; u0's row arrived in step j - 5
+            const float2 *R0 = I == 2 ? qprev : qnext + (I + 1) * P;
+            const Rec &c = C[I1];
+            const float2 q[4] = {c.rho, c.mx, c.my, c.E};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float2 base = R0[3 * k * P];
+                const float2 res = fma2(f2(2.f / 3.f), fma2(dt, L3[k], sub2(q[k], base)), base);
+                if (j < enda) u.h[0].out[k * plane + oa] = res.x;
+                if (j < endb) u.h[1].out[k * plane + ob] = res.y;
+            }
+            oa += n;
+            ob += n;
+        }
+        if (run2) march_rhs<P, I, 1, true>(cur, prev, one, B[I], B[I1], B[I2], u.inv_h, u.inv_2h, mu, kap, yf2, L2);
+        if (run2) {  // row y0 - 6 + j of s2; u0's row arrived in step j - 3
+            const float2 *R0 = qprev + I * P;
+            const Rec &c = B[I1];
+            const float2 q[4] = {c.rho, c.mx, c.my, c.E};
+            float2 sv[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float2 base = R0[3 * k * P];
+                sv[k] = fma2(f2(0.25f), fma2(dt, L2[k], sub2(q[k], base)), base);
+            }
+            C[I] = make_rec(sv[0], sv[1], sv[2], sv[3], gm1);
+        }
+        if (run1) march_rhs<P, I, 0, true>(cur, prev, one, A[I1], A[I2], A[I], u.inv_h, u.inv_2h, mu, kap, yf1, L1);
+        if (run1) {  // row y0 - 4 + j of s1
+            const Rec &c = A[I2];
+            const float2 q[4] = {c.rho, c.mx, c.my, c.E};
+            float2 sv[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sv[k] = fma2(dt, L1[k], q[k]);
+            B[I] = make_rec(sv[0], sv[1], sv[2], sv[3], gm1);
         }
     };
-    load_row(0);
-    const float2 dt = f2(u.dt);
-    Rec a_m1{}, a_c{}, a_p1{};  // u0 rows around stage 1's row
-    Rec b_m1{}, b_c{}, b_p1{};  // s1 rows around stage 2's row
-    Rec c_m1{}, c_c{}, c_p1{};  // s2 rows around stage 3's row
-    Face yf1{}, yf2{}, yf3{};   // carried faces
-    float2 L[4];
-    const int steps = R + 8;
-    for (int j = 0; j < steps; ++j) {
-        // publish the rows that arrive in this step
-        if (j <= R + 5) {
-            const Rec r = make_rec(make_float2(ld[0], ld[1]), make_float2(ld[2], ld[3]), make_float2(ld[4], ld[5]),
-                                   make_float2(ld[6], ld[7]), gm1);
-            a_m1 = a_c;
-            a_c = a_p1;
-            a_p1 = r;
-            march_publish(X, P, sl, 0, j, r);
-            float2 *R0 = X + (60 + 4 * (j & 7)) * P + sl.own;
-            R0[0] = r.rho;
-            R0[P] = r.mx;
-            R0[2 * P] = r.my;
-            R0[3 * P] = r.E;
+    using No = std::false_type;
+    using Yes = std::true_type;
+    for (int j = 0; j < R + 8; j += 3) {
+        if (j >= 8 && j + 2 <= R + 5) {
+            step(Int<0>{}, Yes{}, j);
+            step(Int<1>{}, Yes{}, j + 1);
+            step(Int<2>{}, Yes{}, j + 2);
+        } else {
+            step(Int<0>{}, No{}, j);
+            if (j + 1 < R + 8) step(Int<1>{}, No{}, j + 1);
+            if (j + 2 < R + 8) step(Int<2>{}, No{}, j + 2);
         }
-        if (j >= 3 && j <= R + 6) march_publish(X, P, sl, 1, j, b_p1);
-        if (j >= 6 && j <= R + 7) march_publish(X, P, sl, 2, j, c_p1);
-        __syncthreads();
-        if (j + 1 <= R + 5) load_row(j + 1);
-
-        if (j >= 8 && j <= R + 5) {
-            // steady state: the three stages without branches between them, so
-            // that the compiler interleaves their independent arithmetic (with
-            // one or two CTAs per SM the latency is hidden by this ILP)
-            float2 L3[4], L2[4], L1[4];
-            march_rhs<true>(X, P, nb, 2, j, c_m1, c_c, c_p1, u.inv_h, u.inv_2h, mu, kap, yf3, L3);
-            march_rhs<true>(X, P, nb, 1, j, b_m1, b_c, b_p1, u.inv_h, u.inv_2h, mu, kap, yf2, L2);
-            march_rhs<true>(X, P, nb, 0, j, a_m1, a_c, a_p1, u.inv_h, u.inv_2h, mu, kap, yf1, L1);
-            {
-                const float2 *R0 = X + (60 + 4 * ((j - 5) & 7)) * P + sl.own;
-                const float2 q[4] = {c_c.rho, c_c.mx, c_c.my, c_c.E};
-                float *o = u.out + wrap_index(u.y0 - 8 + j, n) * n;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float2 base = R0[k * P];
-                    const float2 res = fma2(f2(2.f / 3.f), add2(sub2(q[k], base), mul2(dt, L3[k])), base);
-                    if (wa) o[k * plane + xa] = res.x;
-                    if (wb) o[k * plane + xb] = res.y;
-                }
-            }
-            {
-                const float2 *R0 = X + (60 + 4 * ((j - 3) & 7)) * P + sl.own;
-                const float2 q[4] = {b_c.rho, b_c.mx, b_c.my, b_c.E};
-                float2 sv[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float2 base = R0[k * P];
-                    sv[k] = fma2(f2(0.25f), add2(sub2(q[k], base), mul2(dt, L2[k])), base);
-                }
-                c_m1 = c_c;
-                c_c = c_p1;
-                c_p1 = make_rec(sv[0], sv[1], sv[2], sv[3], gm1);
-            }
-            {
-                const float2 q[4] = {a_c.rho, a_c.mx, a_c.my, a_c.E};
-                float2 sv[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) sv[k] = add2(q[k], mul2(dt, L1[k]));
-                b_m1 = b_c;
-                b_c = b_p1;
-                b_p1 = make_rec(sv[0], sv[1], sv[2], sv[3], gm1);
-            }
-            continue;
-        }
-        // stage 3 at row y0 - 8 + j: the new state
-        if (j == 7) march_rhs<false>(X, P, nb, 2, j, c_m1, c_c, c_p1, u.inv_h, u.inv_2h, mu, kap, yf3, L);
-        if (j >= 8) {
-            march_rhs<true>(X, P, nb, 2, j, c_m1, c_c, c_p1, u.inv_h, u.inv_2h, mu, kap, yf3, L);
-            const float2 *R0 = X + (60 + 4 * ((j - 5) & 7)) * P + sl.own;
-            const float2 q[4] = {c_c.rho, c_c.mx, c_c.my, c_c.E};
-            float *o = u.out + wrap_index(u.y0 - 8 + j, n) * n;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float2 base = R0[k * P];
-                const float2 res = fma2(f2(2.f / 3.f), add2(sub2(q[k], base), mul2(dt, L[k])), base);
-                if (wa) o[k * plane + xa] = res.x;
-                if (wb) o[k * plane + xb] = res.y;
-            }
-        }
-        // stage 2 at row y0 - 6 + j
-        if (j == 4) march_rhs<false>(X, P, nb, 1, j, b_m1, b_c, b_p1, u.inv_h, u.inv_2h, mu, kap, yf2, L);
-        if (j >= 5 && j <= R + 6) {
-            march_rhs<true>(X, P, nb, 1, j, b_m1, b_c, b_p1, u.inv_h, u.inv_2h, mu, kap, yf2, L);
-            const float2 *R0 = X + (60 + 4 * ((j - 3) & 7)) * P + sl.own;
-            const float2 q[4] = {b_c.rho, b_c.mx, b_c.my, b_c.E};
-            float2 s[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float2 base = R0[k * P];
-                s[k] = fma2(f2(0.25f), add2(sub2(q[k], base), mul2(dt, L[k])), base);
-            }
-            c_m1 = c_c;
-            c_c = c_p1;
-            c_p1 = make_rec(s[0], s[1], s[2], s[3], gm1);
-        }
-        // stage 1 at row y0 - 4 + j
-        if (j == 1) march_rhs<false>(X, P, nb, 0, j, a_m1, a_c, a_p1, u.inv_h, u.inv_2h, mu, kap, yf1, L);
-        if (j >= 2 && j <= R + 5) {
-            march_rhs<true>(X, P, nb, 0, j, a_m1, a_c, a_p1, u.inv_h, u.inv_2h, mu, kap, yf1, L);
-            const float2 q[4] = {a_c.rho, a_c.mx, a_c.my, a_c.E};
-            float2 s[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) s[k] = add2(q[k], mul2(dt, L[k]));
-            b_m1 = b_c;
-            b_c = b_p1;
-            b_p1 = make_rec(s[0], s[1], s[2], s[3], gm1);
-        }
+        const Ring s = cur;
+        cur = prev;
+        prev = s;
+        float2 *const q = qprev;
+        qprev = q0;
+        q0 = qnext;
+        qnext = q;
     }
+    cp_async_wait<0>();
 }
 
 // After an odd number of steps the states sit in the scratch buffers: copy
@@ -1110,13 +1142,16 @@ static void step_sequence(const Tiles &src, int ngroups, int total_tiles, int ns
     }
 }
 
-template <class Units>
-static void march_launch(const Units &src, int units, int threads, int parity, float gm1, float mu, float kap,
+template <int I>
+static void march_launch(const MarchUnits &src, int units, int threads, int parity, float gm1, float mu, float kap,
                          cudaStream_t s) {
+    constexpr int P = kMarchPitch[I];
+    if constexpr (I + 1 < (int)(sizeof(kMarchPitch) / sizeof(kMarchPitch[0])))
+        if (threads > P) return march_launch<I + 1>(src, units, threads, parity, gm1, mu, kap, s);
     static OncePerDevice once;
     once.run([](int) {
-        return cudaFuncSetAttribute(ns2d_rk3_march<Units>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)march_smem_bytes(kMarchMaxThreads));
+        return cudaFuncSetAttribute(ns2d_rk3_march<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)march_smem_bytes(P));
     });
     // programmatic stream serialisation: the launch may start while the
     // previous kernel on the stream finishes; the kernel waits for it before
@@ -1124,24 +1159,23 @@ static void march_launch(const Units &src, int units, int threads, int parity, f
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(units);
     cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = march_smem_bytes(threads);
+    cfg.dynamicSmemBytes = march_smem_bytes(P);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, ns2d_rk3_march<Units>, src, parity, gm1, mu, kap);
+    cudaLaunchKernelEx(&cfg, ns2d_rk3_march<P>, src, parity, gm1, mu, kap);
 }
 
 // nsteps steps of every unit (the states end in u0), FP32
-template <class Units>
-static void march_sequence(const Units &src, int ngroups, int units, int threads, int nsteps, float gm1, float mu,
+static void march_sequence(const MarchUnits &src, int ngroups, int units, int threads, int nsteps, float gm1, float mu,
                            float kap, cudaStream_t s) {
-    for (int st = 0; st < nsteps; ++st) march_launch(src, units, threads, st & 1, gm1, mu, kap, s);
+    for (int st = 0; st < nsteps; ++st) march_launch<0>(src, units, threads, st & 1, gm1, mu, kap, s);
     count_launches(nsteps);
     if (nsteps & 1) {
-        ns2d_copy_back<Units><<<dim3(2 * kNumSMs, ngroups), 256, 0, s>>>(src);
+        ns2d_copy_back<MarchUnits><<<dim3(2 * kNumSMs, ngroups), 256, 0, s>>>(src);
         count_launches(1);
     }
 }
@@ -1155,23 +1189,74 @@ int ns2d_seg_rows(int shape) {
 }
 bool ns2d_narrow(int shape) { return shape / kNsSegChoices == 1; }
 
-int ns2d_default_choice(int n, int grids, int sms) {
-    const int base = n > 256 ? kNsSegChoices : 0;
-    constexpr int longest_first[kNsSegChoices] = {4, 3, 2, 6, 0, 5, 7, 1};  // 256, 128, 64, 48, 32, 24, 20, 16 rows
-    for (int r : longest_first) {
-        int bands = 0, segs = 0, threads = 0;
-        ns2d_march_layout(n, base + r, &bands, &segs, &threads);
-        if ((long long)bands * segs * grids >= 2LL * sms) return base + r;
-    }
-    return base + 1;
-}
-
 void ns2d_march_layout(int n, int shape, int *bands, int *segs, int *threads) {
     const int S = std::min(n, ns2d_seg_rows(shape));
     const bool narrow = ns2d_narrow(shape);
     *bands = march_bands(n, narrow);
     *segs = (n + S - 1) / S;
     *threads = march_threads(n, narrow);
+}
+
+// Estimated time of a model step of all sizes at once, in march steps at two
+// warps per scheduler.  A march step's time is its latency: about 0.65 us with
+// one warp per scheduler and 1.05 us with two, which is all that the registers
+// of an SM hold (248 a thread).  While every CTA of the launches is resident
+// the longest march decides; beyond that the work does, plus a tenth of the
+// longest march (and a little of each) for the ends of the launches.  CTAs of
+// more than four warps have an SM to themselves: they lose a tenth at their
+// barriers, and more where CTAs of many sizes leave few SMs empty.  (24
+// problems of 64^2 .. 768^2, one choice for all: the estimates for 32, 48, 64,
+// 128 and 256 rows, wide and narrow, are proportional to the measured 6.2 ..
+// 7.9 ms within 5%; with the defaults 6.2 ms.)
+static double march_estimate(int count, const int *n, const int *grids, const int *choice, int sms) {
+    double load = 0, work = 0;
+    int longest = 0, all = 0;
+    bool large = false;
+    for (int k = 0; k < count; ++k) {
+        int bands = 0, segs = 0, threads = 0;
+        ns2d_march_layout(n[k], choice[k], &bands, &segs, &threads);
+        const int warps = (threads + 31) / 32, per_sm = std::max(1, 8 / warps);
+        const double share = (((long long)bands * segs * grids[k] + 1) / 2) / ((double)per_sm * sms);
+        const int steps = (n[k] + segs - 1) / segs + 8;
+        load += share;
+        all += steps;
+        work += share * steps * (warps > 4 ? (count > 2 ? 1.5 : 1.1) : 1.0);
+        if (steps > longest || (steps == longest && warps > 4)) large = warps > 4;
+        longest = std::max(longest, steps);
+    }
+    if (load <= 1) return longest * (load <= 0.5 && !large ? 0.63 : 1.0);
+    return std::max(work, (double)longest) + 0.1 * longest + 0.003 * all;
+}
+
+void ns2d_default_choices(int count, const int *n, const int *grids, int sms, int *choice) {
+    std::vector<int> c(count);
+    double best = 0;
+    for (int rows = 0; rows < kNsSegChoices; ++rows) {
+        // from segments of these rows everywhere, one size at a time until no
+        // change of one choice helps
+        for (int k = 0; k < count; ++k) c[k] = n[k] > 128 ? kNsSegChoices + rows : rows;
+        double now = march_estimate(count, n, grids, c.data(), sms);
+        bool better = true;
+        for (int pass = 0; pass < 4 && better; ++pass) {
+            better = false;
+            for (int k = 0; k < count; ++k)
+                for (int q = 0; q < kNsTileShapes; ++q) {
+                    const int was = c[k];
+                    c[k] = q;
+                    const double t = march_estimate(count, n, grids, c.data(), sms);
+                    if (t < now * (1 - 1e-9)) {
+                        now = t;
+                        better = true;
+                    } else {
+                        c[k] = was;
+                    }
+                }
+        }
+        if (rows == 0 || now < best * (1 - 1e-9)) {
+            best = now;
+            std::copy(c.begin(), c.end(), choice);
+        }
+    }
 }
 
 // strips of an n x n grid in the FP64 march, and the CTAs of `grids` grids cut
@@ -1316,13 +1401,15 @@ cudaError_t ns2d_forecast_scratch(T *whole, int n_whole, int n_whole_probs, T *s
         } else {
             // grids of one size (truth runs, the stateless entry point): the
             // column march
-            OneUnits U{gr[0]};
+            MarchUnits U{nullptr, 1, gr[0]};
             int bands = 0, segs = 0, threads = 0;
-            ns2d_march_layout(ns[0], np[0] == 1 ? 1 : 0, &bands, &segs, &threads);
-            U.g.tx = bands;
-            U.g.ty = segs;
-            U.g.tile_begin = 0;
-            march_sequence(U, 1, bands * segs * np[0], threads, nsteps, gm1, m, kappa, stream);
+            int choice = 0;
+            ns2d_default_choices(1, ns, np, kNumSMs, &choice);
+            ns2d_march_layout(ns[0], choice, &bands, &segs, &threads);
+            U.one.tx = bands;
+            U.one.ty = segs;
+            U.one.tile_begin = 0;
+            march_sequence(U, 1, ns2d_group_units(U.one), threads, nsteps, gm1, m, kappa, stream);
         }
     } else {
         const cudaError_t e = n64_forecast(gr, gm1, m, kappa, nsteps, stream);
@@ -1351,10 +1438,10 @@ static cudaError_t table_steps(const NsGroup<float> *d_groups, int ngroups, int 
                                bool probe, double gamma, double mu, double prandtl, int shape, cudaStream_t s) {
     if (units == 0 || nsteps == 0) return cudaSuccess;
     const float gm1 = (float)(gamma - 1.0), m = (float)mu, kap = (float)(mu * gamma / ((gamma - 1.0) * prandtl));
-    const TableUnits src{d_groups, ngroups};
+    const MarchUnits src{d_groups, ngroups, {}};
     const int threads = march_threads(n, ns2d_narrow(shape));
     if (probe) {  // one step into the scratch buffers: the states stay as they are
-        march_launch(src, units, threads, 0, gm1, m, kap, s);
+        march_launch<0>(src, units, threads, 0, gm1, m, kap, s);
         count_launches(1);
     } else {
         march_sequence(src, ngroups, units, threads, nsteps, gm1, m, kap, s);

@@ -19,21 +19,23 @@ struct NsGroup {
 // rows per segment of the march (shape mod 8: 0 = 32, 1 = 16, 2 = 64,
 // 3 = 128, 4 = 256, 5 = 24, 6 = 48, 7 = 20; a grid of n rows is cut into
 // ceil(n / rows) segments of equal length but the last) and the band width
-// (shape / 8: 0 = the whole width up to 512 columns, 1 = bands of at most 122
-// columns, 64 threads per CTA).
+// (shape / 8: 0 = the whole width up to 256 columns, 1 = bands of at most 122
+// columns, at most 128 threads per CTA).
 constexpr int kNsSegChoices = 8;
 constexpr int kNsTileShapes = 2 * kNsSegChoices;
 int ns2d_seg_rows(int shape);
 bool ns2d_narrow(int shape);
-// default choice for `grids` n x n grids stepped on their own: narrow bands
-// above 256 points per side, the longest segments that still give two units
-// per SM (`sms` SMs), else 16 rows
-int ns2d_default_choice(int n, int grids, int sms);
+// default choices for `count` sizes stepped at the same time on `sms` SMs
+// (grids[k] grids of n[k] points per side): the least estimated time
+void ns2d_default_choices(int count, const int *n, const int *grids, int sms, int *choice);
 // bands, row segments and threads per CTA of the FP32 step on an n x n grid
 void ns2d_march_layout(int n, int shape, int *bands, int *segs, int *threads);
 
+// units of a group: two row segments each (the last of an odd count alone)
+inline int ns2d_group_units(const NsGroup<float> &g) { return (g.tx * g.ty * g.nprob + 1) / 2; }
+
 // nsteps SSP-RK3 steps of every group of a device table (tile_begin ascending,
-// all groups of grid size n, units = bands x segments x grids in total), FP32
+// all groups of grid size n, units: the sum of ns2d_group_units), FP32
 // states.
 cudaError_t ns2d_forecast_table(const NsGroup<float> *d_groups, int ngroups, int units, int n, int nsteps,
                                 double gamma, double mu, double prandtl, int shape, cudaStream_t s);

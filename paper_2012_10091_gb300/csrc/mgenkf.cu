@@ -404,8 +404,8 @@ static mgenkf_status create_impl(mgenkf_ctx *h, const mgenkf_config *cfg, const 
         H_CUDA(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
         int sms = 0;
         H_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
-        h->fc_choice[0] = ns2d_default_choice(h->nc, h->ne, sms);
-        h->fc_choice[1] = ns2d_default_choice(h->nf, 1, sms);
+        const int sizes[2] = {h->nc, h->nf}, grids[2] = {h->ne, 1};
+        ns2d_default_choices(2, sizes, grids, sms, h->fc_choice);
         mgenkf_status st = upload_fc_table(h);
         if (st) return st;
     }
@@ -521,7 +521,7 @@ static mgenkf_status upload_fc_table(mgenkf_ctx *h) {
         g[k].tx = bands;
         g[k].ty = segs;
         g[k].tile_begin = 0;
-        h->fc_units[k] = bands * segs * g[k].nprob;
+        h->fc_units[k] = ns2d_group_units(g[k]);
     }
     H_CUDA(cudaMemcpyAsync(h->d_fc, g, sizeof(g), cudaMemcpyHostToDevice, h->stream));
     H_CUDA(cudaStreamSynchronize(h->stream));
@@ -1210,6 +1210,7 @@ extern "C" uint64_t mgk_kernel_launches(void) { return g_launches.load(std::memo
 namespace {
 // analysis branches of the captured cycle (problems spread by estimated cost)
 constexpr int kMaxBatchStreams = 128;
+constexpr int kDefaultBatchParts = 2;      // of the grouped cycle
 constexpr int kDefaultBatchBranches = 16;  // measured best for the 96-problem batch (1, 4, 16, 128 tried)
 }
 
@@ -1294,7 +1295,7 @@ static void build_tables(mgenkf_batch *b, std::vector<std::vector<NsGroup<float>
             g[k].tx = bands;
             g[k].ty = segs;
             g[k].tile_begin = units[si];
-            units[si] += bands * segs * g[k].nprob;
+            units[si] += ns2d_group_units(g[k]);
             tab[si].push_back(g[k]);
         }
     }
@@ -1322,7 +1323,7 @@ static mgenkf_status upload_tables(mgenkf_batch *b, const std::vector<std::vecto
         b->ngroups[k] = (int)tab[k].size();
         if (tab[k].empty()) continue;
         const NsGroup<float> &last = tab[k].back();
-        b->units[k] = last.tile_begin + last.tx * last.ty * last.nprob;
+        b->units[k] = last.tile_begin + ns2d_group_units(last);
         B_CUDA(cudaMalloc(&b->d_groups[k], tab[k].size() * sizeof(NsGroup<float>)));
         // on the batch stream: a plain copy from pageable memory may return
         // before it lands and a non-blocking stream does not wait for it
@@ -1355,7 +1356,7 @@ static mgenkf_status upload_part_tables(mgenkf_batch *b) {
             g[k].tx = bands;
             g[k].ty = segs;
             g[k].tile_begin = units[ti];
-            units[ti] += bands * segs * g[k].nprob;
+            units[ti] += ns2d_group_units(g[k]);
             tab[ti].push_back(g[k]);
         }
     }
@@ -1429,6 +1430,19 @@ extern "C" mgenkf_status mgenkf_batch_create(const mgenkf_handle *handles, int32
                 b->sizes.push_back(sz);
                 b->shape.push_back(0);
             }
+    }
+    {
+        // default forecast choices: all sizes step at once, a part's problems at a time
+        std::vector<int> grids(b->sizes.size(), 0);
+        for (const mgenkf_ctx *h : b->hs) {
+            grids[size_index(b, h->nc)] += h->ne;
+            grids[size_index(b, h->nf)] += 1;
+        }
+        for (int &g : grids) g = ceil_div(g, std::min(n, kDefaultBatchParts));
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->hs[0]->device) != cudaSuccess)
+            return fail(MGENKF_ERR_CUDA, "device query");
+        ns2d_default_choices((int)b->sizes.size(), b->sizes.data(), grids.data(), sms, b->shape.data());
     }
     if (!b->s0) {
         // the legacy stream cannot be captured: a blocking stream keeps the
@@ -1560,7 +1574,6 @@ static bool groupable(const mgenkf_ctx *h) {
 
 // parts of the grouped cycle: MGENKF_BATCH_PARTS, default kDefaultBatchParts,
 // at most one per problem
-constexpr int kDefaultBatchParts = 2;
 constexpr int kMaxBatchParts = 8;
 
 static GroupProb group_prob(const mgenkf_batch *b, size_t j) {
@@ -1842,7 +1855,7 @@ static mgenkf_status probe_joint(mgenkf_batch *b, int steps, int reps, float *ms
     for (int k = 0; k < ns && st == MGENKF_OK; ++k) {
         if (tab[k].empty()) continue;
         const NsGroup<float> &last = tab[k].back();
-        units[k] = last.tile_begin + last.tx * last.ty * last.nprob;
+        units[k] = last.tile_begin + ns2d_group_units(last);
         if (cuda(cudaMalloc(&d[k], tab[k].size() * sizeof(NsGroup<float>)), "cudaMalloc"))
             cuda(cudaMemcpyAsync(d[k], tab[k].data(), tab[k].size() * sizeof(NsGroup<float>),
                                  cudaMemcpyHostToDevice, b->s0),
@@ -1893,7 +1906,7 @@ extern "C" mgenkf_status mgenkf_batch_autotune(mgenkf_batch_t b, int32_t reps) {
             const int ng = (int)tab[si].size();
             if (!ng) continue;
             const NsGroup<float> &last = tab[si].back();
-            const int units = last.tile_begin + last.tx * last.ty * last.nprob;
+            const int units = last.tile_begin + ns2d_group_units(last);
             B_CUDA(cudaMalloc(&d, ng * sizeof(NsGroup<float>)));
             B_CUDA(cudaMemcpyAsync(d, tab[si].data(), ng * sizeof(NsGroup<float>), cudaMemcpyHostToDevice, b->s0));
             float ms = 0.f;
