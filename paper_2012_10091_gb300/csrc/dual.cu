@@ -5,7 +5,7 @@
 // Model: nodes x_j = j dx; node 0 holds the inlet u0 (1 + theta1 sin(omega t +
 // theta2)), the outlet node is extrapolated linearly, the interior follows the
 // flux-form central scheme; SSP-RK3 in Shu-Osher form with the inlet set at
-// each stage's time.  One CTA advances one grid held in shared memory.
+// each stage's time.  A CTA or a cluster advances one grid held in shared memory.
 //
 // One cycle (mgenkf_dual_cycle):
 //   fine forecast with the analysed parameter mean of the previous cycle;
@@ -19,6 +19,7 @@
 // ends); H^C is the Pi_F row at each observed fine node.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -32,48 +33,111 @@
 namespace mgk {
 
 constexpr uint64_t kThetaTag = 0x54485441ULL;  // "THTA": parameter random walk
-constexpr int kDualMaxPts = 1024;               // points per grid (one CTA, one point per thread)
+constexpr int kDualMaxPts = 1024;               // points per grid
 
-// SSP-RK3 steps of nprob inlet-Burgers grids of n points (one CTA each)
-__global__ void __launch_bounds__(1024) k_burgers_inlet(double *__restrict__ u, int n, double dx, double nu,
-                                                        double dt, int nsteps, double t0,
+// SSP-RK3 steps of nprob inlet-Burgers grids of n points, each on a cluster of
+// CTAs (gridDim.x / nprob of them; one CTA where CLUSTER is false).  CTA r of a
+// cluster owns nodes [r per, (r + 1) per) and carries 3 nodes of its neighbours
+// on each side, one thread per node: stage 1 is evaluated two nodes into them,
+// stage 2 one node, so that the CTAs exchange values once per step (3 nodes
+// written to each neighbour's shared memory, double-buffered: a neighbour may
+// still be in the step before) and a stage ends in a barrier of the CTA.
+//
+// Bound by the FP64 pipes: a warp instruction takes 64 cycles of its scheduler,
+// so the arithmetic is folded to 17 per step.  With c1 = dt / (4 dx),
+// c2 = dt nu / dx^2, d = v_{j+1} - v_{j-1} and s = v_{j+1} + v_{j-1},
+//   v + dt L(v) = (1 - 2 c2) v + s (c2 - c1 d).
+// The inlet values of 32 steps are formed together by 64 threads (a sine takes
+// some 50 dependent FP64 instructions); the outlet is extrapolated by the one
+// thread that reads it.  30 steps: 100 grids of 200 nodes 176 -> 51 us, one of
+// 800 (a cluster of 8, where one SM did all of it) 441 -> 43 us.
+constexpr int kInletSteps = 32;  // steps of inlet values formed together
+__device__ __forceinline__ void inlet_push(double *local, int rank, double v) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(local), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+template <bool CLUSTER>
+__global__ void __launch_bounds__(1024) k_burgers_inlet(double *__restrict__ u, int n, int ctas, int per, double c1,
+                                                        double c2, double dt, int nsteps, double t0,
                                                         const double *__restrict__ theta, double u0, double omega) {
     extern __shared__ double sh[];
-    double *x = sh, *u1 = sh + n, *u2 = sh + 2 * n;
-    const int j = threadIdx.x;
-    double *g = u + (size_t)blockIdx.x * n;
-    const double th1 = theta[2 * blockIdx.x], th2 = theta[2 * blockIdx.x + 1];
-    if (j < n) x[j] = g[j];
-    const double i2dx = 1.0 / (2.0 * dx), idx2 = 1.0 / (dx * dx);
-    auto L = [&](const double *v) {
-        const double fp = 0.5 * v[j + 1] * v[j + 1], fm = 0.5 * v[j - 1] * v[j - 1];
-        return -(fp - fm) * i2dx + nu * (v[j + 1] - 2.0 * v[j] + v[j - 1]) * idx2;
-    };
-    auto bc = [&](double *v, double t) {  // after the interior of v is complete
-        if (j == 0) v[0] = u0 * (1.0 + th1 * sin(omega * t + th2));
-        if (j == n - 1) v[n - 1] = 2.0 * v[n - 2] - v[n - 3];
-    };
-    const bool in = j > 0 && j < n - 1;
-    for (int s = 0; s < nsteps; ++s) {
-        const double t = t0 + s * dt;
-        __syncthreads();
-        if (in) u1[j] = x[j] + dt * L(x);
-        __syncthreads();
-        bc(u1, t + dt);
-        __syncthreads();
-        if (in) u2[j] = 0.75 * x[j] + 0.25 * (u1[j] + dt * L(u1));
-        __syncthreads();
-        bc(u2, t + 0.5 * dt);
-        __syncthreads();
-        double xn = 0.0;
-        if (in) xn = x[j] / 3.0 + 2.0 / 3.0 * (u2[j] + dt * L(u2));
-        __syncthreads();  // every read of x in this step is done
-        if (in) x[j] = xn;
-        __syncthreads();
-        bc(x, t + dt);
+    __shared__ double inlet[2 * kInletSteps];
+    const int pitch = per + 6;
+    double *A = sh, *B = sh + 2 * pitch, *C = sh + 3 * pitch;  // x (two buffers), u1, u2
+    const int prob = CLUSTER ? blockIdx.x / ctas : blockIdx.x, rank = CLUSTER ? blockIdx.x - prob * ctas : 0;
+    // nodes [lo, hi) are this CTA's; slot j holds node lo - 3 + j
+    const int lo = rank * per, hi = min(n, lo + per);
+    const int j = threadIdx.x, k = lo - 3 + j;
+    double *g = u + (size_t)prob * n;
+    const double th1 = theta[2 * prob], th2 = theta[2 * prob + 1];
+    const bool held = j < pitch && k >= 0 && k < min(n, hi + 3);
+    const bool own = held && k >= lo && k < hi;
+    const bool first = held && k == 0, last = held && k == n - 1, before_last = held && k == n - 2;
+    // nodes with both neighbours in this CTA
+    const bool in = held && k > 0 && k < n - 1 && j > 0 && k < hi + 2;
+    if (held) {
+        A[j] = g[k];
+        B[j] = C[j] = A[pitch + j] = 0.0;
     }
-    __syncthreads();
-    if (j < n) g[j] = x[j];
+    const double k1 = 1.0 - 2.0 * c2;
+    const double c1b = 0.25 * c1, c2b = 0.25 * c2, k1b = 0.25 * k1;
+    const double c1c = 2.0 / 3.0 * c1, c2c = 2.0 / 3.0 * c2, k1c = 2.0 / 3.0 * k1, third = 1.0 / 3.0;
+    if (CLUSTER) {
+        // every CTA of the cluster runs and its buffers are set
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    }
+    for (int s = 0; s < nsteps; ++s) {
+        if (s % kInletSteps == 0 && lo == 0) {
+            if (j < 2 * min(kInletSteps, nsteps - s)) {
+                const double t = t0 + (s + (j >> 1)) * dt;
+                inlet[j] = u0 * (1.0 + th1 * sin(omega * (j & 1 ? t + 0.5 * dt : t + dt) + th2));
+            }
+        }
+        if (!CLUSTER || s % kInletSteps == 0) __syncthreads();
+        const double bc = inlet[2 * (s % kInletSteps)], bch = inlet[2 * (s % kInletSteps) + 1];
+        const double *a = A + (s & 1) * pitch;
+        double *an = A + ((s & 1) ^ 1) * pitch;
+        double x = 0.0, y = 0.0;
+        if (in) {
+            x = a[j];
+            const double vm = a[j - 1], vp = before_last && s > 0 ? 2.0 * x - vm : a[j + 1];
+            y = fma(vp + vm, fma(-c1, vp - vm, c2), k1 * x);
+            B[j] = y;
+        }
+        if (first) B[j] = bc;
+        __syncthreads();
+        double z = 0.0;
+        if (in) {
+            const double vm = B[j - 1], vp = before_last ? 2.0 * y - vm : B[j + 1];
+            z = fma(vp + vm, fma(-c1b, vp - vm, c2b), fma(k1b, y, 0.75 * x));
+            C[j] = z;
+        }
+        if (first) C[j] = bch;
+        __syncthreads();
+        double w = first ? bc : 0.0;
+        if (in) {
+            const double vm = C[j - 1], vp = before_last ? 2.0 * z - vm : C[j + 1];
+            w = fma(vp + vm, fma(-c1c, vp - vm, c2c), fma(k1c, z, third * x));
+        }
+        if (own) {
+            an[j] = w;
+            if (CLUSTER) {
+                // slot of node k in a neighbour: k - (its lo - 3)
+                if (j < 6 && rank > 0) inlet_push(an + j + per, rank - 1, w);
+                if (j >= per && rank + 1 < ctas) inlet_push(an + j - per, rank + 1, w);
+            }
+        }
+        if (CLUSTER) {
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        }
+    }
+    if (!CLUSTER) __syncthreads();
+    const double *a = A + (nsteps & 1) * pitch;
+    if (own) g[k] = last && nsteps > 0 ? 2.0 * a[j - 1] - a[j - 2] : a[j];
 }
 
 // theta^f = theta^a + sqrt(q) tau
@@ -84,29 +148,65 @@ __global__ void k_theta_walk(const double *__restrict__ theta, const double *__r
 }
 
 // theta^a_i = theta^f_i + sum_a Theta[p][a] T[a][i], Theta the normalised
-// parameter anomalies; T column i at Tm[i ne ..]; then (thread 0) the mean
-__global__ void k_theta_update(const double *__restrict__ theta_f, const double *__restrict__ Tm, int ne,
-                               double *__restrict__ theta_a, double *__restrict__ theta_mean, const int *status) {
-    if (*status) return;
-    __shared__ double mean[2];
-    if (threadIdx.x < 2) {
-        double m = 0.0;
-        for (int a = 0; a < ne; ++a) m += theta_f[2 * a + threadIdx.x];
-        mean[threadIdx.x] = m / ne;
+// parameter anomalies (T column i at Tm[i ne ..]), and the mean of theta^a.  A
+// cluster of kThetaCtas: each takes ne / kThetaCtas members, a warp per member
+// over the lanes, and the first sums the CTAs' means (one CTA with a thread per
+// member and parameter, chains of 3 ne FP64 instructions: 37 us for 100
+// members, 15 us so).
+constexpr int kThetaCtas = 8, kThetaWarps = 8;
+__device__ __forceinline__ double warp_sum(double v) {
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__global__ void __cluster_dims__(kThetaCtas, 1, 1) __launch_bounds__(32 * kThetaWarps)
+    k_theta_update(const double *__restrict__ theta_f, const double *__restrict__ Tm, int ne,
+                   double inv_ne, double isq, double *__restrict__ theta_a, double *__restrict__ theta_mean,
+                   const int *status) {
+    __shared__ double part[kThetaCtas][2], mine[kThetaWarps][2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = blockIdx.x;
+    const bool ok = *status == 0;
+    double s0 = 0.0, s1 = 0.0;
+    if (ok) {
+        double m0 = 0.0, m1 = 0.0;
+        for (int a = lane; a < ne; a += 32) {
+            m0 += theta_f[2 * a];
+            m1 += theta_f[2 * a + 1];
+        }
+        m0 = warp_sum(m0) * inv_ne;
+        m1 = warp_sum(m1) * inv_ne;
+        for (int i = rank * kThetaWarps + warp; i < ne; i += kThetaCtas * kThetaWarps) {
+            double a0 = 0.0, a1 = 0.0;
+            for (int a = lane; a < ne; a += 32) {
+                const double t = Tm[(size_t)i * ne + a];
+                a0 = fma(theta_f[2 * a] - m0, t, a0);
+                a1 = fma(theta_f[2 * a + 1] - m1, t, a1);
+            }
+            a0 = fma(warp_sum(a0), isq, theta_f[2 * i]);
+            a1 = fma(warp_sum(a1), isq, theta_f[2 * i + 1]);
+            if (lane == 0) {
+                theta_a[2 * i] = a0;
+                theta_a[2 * i + 1] = a1;
+            }
+            s0 += a0;
+            s1 += a1;
+        }
+        if (lane == 0) {
+            mine[warp][0] = s0;
+            mine[warp][1] = s1;
+        }
+        __syncthreads();
+        if (threadIdx.x < 2) {
+            double m = 0.0;
+            for (int w = 0; w < kThetaWarps; ++w) m += mine[w][threadIdx.x];
+            inlet_push(&part[rank][threadIdx.x], 0, m);
+        }
     }
-    __syncthreads();
-    const double isq = 1.0 / sqrt((double)(ne - 1));
-    for (int e = threadIdx.x; e < 2 * ne; e += blockDim.x) {
-        const int i = e >> 1, p = e & 1;
-        double acc = 0.0;
-        for (int a = 0; a < ne; ++a) acc = fma((theta_f[2 * a + p] - mean[p]) * isq, Tm[(size_t)i * ne + a], acc);
-        theta_a[e] = theta_f[e] + acc;
-    }
-    __syncthreads();
-    if (threadIdx.x < 2) {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (ok && rank == 0 && threadIdx.x < 2) {
         double m = 0.0;
-        for (int a = 0; a < ne; ++a) m += theta_a[2 * a + threadIdx.x];
-        theta_mean[threadIdx.x] = m / ne;
+        for (int r = 0; r < kThetaCtas; ++r) m += part[r][threadIdx.x];
+        theta_mean[threadIdx.x] = m * inv_ne;
     }
 }
 
@@ -176,11 +276,37 @@ void free_dual(mgenkf_dual *d) {
     if (d->aux) cudaStreamDestroy(d->aux);
 }
 
+// CTAs per grid: the fewest that leave one warp to each scheduler, while the
+// grids do not exceed the SMs (then each gets one)
+int inlet_ctas(int nprob, int n) {
+    int c = 1;
+    while (c < 8 && ceil_div(n, c) + 6 > 128 && nprob * 2 * c <= kNumSMs) c *= 2;
+    return c;
+}
+
 void forecast(mgenkf_dual *d, double *grids, int nprob, int n, const double *theta, int nsteps,
               cudaStream_t s = nullptr) {
     count_launches(1);
-    k_burgers_inlet<<<nprob, ((n + 31) / 32) * 32, 3 * n * sizeof(double), s ? s : d->stream>>>(
-        grids, n, d->cfg.length / n, d->cfg.nu, d->cfg.dt, nsteps, d->t, theta, d->cfg.u0, d->cfg.omega);
+    const int ctas = inlet_ctas(nprob, n), per = ceil_div(n, ctas);
+    const double dx = d->cfg.length / n, dt = d->cfg.dt;
+    const double c1 = dt / (4.0 * dx), c2 = dt * d->cfg.nu / (dx * dx);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nprob * ctas);
+    cfg.blockDim = dim3(std::max(64, ceil_div(per + 6, 32) * 32));  // 64 threads form the inlet values
+    cfg.dynamicSmemBytes = 4 * (per + 6) * sizeof(double);
+    cfg.stream = s ? s : d->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (ctas > 1)
+        cudaLaunchKernelEx(&cfg, k_burgers_inlet<true>, grids, n, ctas, per, c1, c2, dt, nsteps, d->t, theta, d->cfg.u0,
+                           d->cfg.omega);
+    else
+        cudaLaunchKernelEx(&cfg, k_burgers_inlet<false>, grids, n, ctas, per, c1, c2, dt, nsteps, d->t, theta,
+                           d->cfg.u0, d->cfg.omega);
 }
 
 // perturbations (generated once per cycle), anomalies and T = S^-1 B (ensemble space)
@@ -352,7 +478,8 @@ extern "C" mgenkf_status mgenkf_dual_cycle(mgenkf_dual_t d, int32_t nsteps, cons
     gain_solve(d, 1, d->xstar_a);
     D_CUDA(cudaStreamWaitEvent(s, d->ev[1], 0));  // join: the fine forecast has read theta_mean
     count_launches(1);
-    k_theta_update<<<1, 256, 0, s>>>(d->theta_f, d->Bt, ne, d->theta, d->theta_mean, d->status);
+    k_theta_update<<<kThetaCtas, 32 * kThetaWarps, 0, s>>>(
+        d->theta_f, d->Bt, ne, 1.0 / ne, 1.0 / std::sqrt(ne - 1.0), d->theta, d->theta_mean, d->status);
     // steps 6-8: members forecast again from the previous analysis with theta^a, state update
     D_CUDA(cudaMemcpyAsync(d->members, d->prev, (size_t)ne * nc * 8, cudaMemcpyDeviceToDevice, s));
     forecast(d, d->members, ne, nc, d->theta, nsteps);
