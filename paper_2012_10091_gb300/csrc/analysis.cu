@@ -913,33 +913,56 @@ void launch_spd_solve(const double *A, const double *At, int n, const double *rh
 // member update x^a,(i) = x^f,(i) + X T_i and coarse correction dC = X T_ne
 // (Eq. ensemble_update with K = X T; Algorithm 4 step 5)
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) k_update_f64(T *__restrict__ members, T *__restrict__ dC,
-                                                    const double *__restrict__ X,
-                                                    const double *__restrict__ Tm, size_t nx, int ne,
-                                                    const int *status) {
-    extern __shared__ double Ts[];  // [32 columns][ne]
+// A warp takes 32 points and Q columns (the columns of T in shared memory, read
+// by broadcast; X eight members ahead in registers), a CTA one warp per
+// scheduler.  Bound by the FP64 pipes, 64 cycles of a scheduler per warp
+// instruction whatever its lanes hold, so Q is the number of columns whose CTAs
+// fill the SMs most evenly (update_cols): a fixed 8 columns in CTAs of 8 warps
+// left half the SMs idle in the last round and multiplied 31 columns of padding
+// at ne + 1 = 129.  4096 points x 128 members: 199 -> 122 us (Q = 7); 200 x 100:
+// 68 -> 16 us; 64 x 32: 27 -> 6.5 us (Q = 1).
+constexpr int kUpdateWarps = 4, kUpdateMaxCols = 8;
+template <typename T, int Q>
+__global__ void __launch_bounds__(32 * kUpdateWarps) k_update_f64(T *__restrict__ members, T *__restrict__ dC,
+                                                                  const double *__restrict__ X,
+                                                                  const double *__restrict__ Tm, size_t nx, int ne,
+                                                                  const int *status) {
+    extern __shared__ double2 Ts2[];  // [Q columns][ne rounded up to 8]
     if (*status) return;
-    const int c0 = blockIdx.y * 32;
-    for (int e = threadIdx.x; e < 32 * ne; e += blockDim.x) {
-        const int cc = e / ne, a = e % ne;
-        Ts[e] = c0 + cc <= ne ? Tm[(size_t)(c0 + cc) * ne + a] : 0.0;
-    }
+    double *Ts = reinterpret_cast<double *>(Ts2);
+    const int c0 = blockIdx.y * Q, pitch = (ne + 7) & ~7;
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        for (int a = threadIdx.x; a < pitch; a += blockDim.x)
+            Ts[q * pitch + a] = a < ne && c0 + q <= ne ? Tm[(size_t)(c0 + q) * ne + a] : 0.0;
+    const size_t p = blockIdx.x * (size_t)(32 * kUpdateWarps) + threadIdx.x;
+    const bool in = p < nx;
+    double x[8], acc[Q];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = in && i < ne ? X[(size_t)i * nx + p] : 0.0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[q] = 0.0;
     __syncthreads();
-    const size_t p = blockIdx.x * (size_t)64 + (threadIdx.x & 63);
-    const int cg = threadIdx.x >> 6;
-    if (p >= nx) return;
-    double acc[8];
+    if (blockIdx.x * (size_t)(32 * kUpdateWarps) + (threadIdx.x & ~31) >= nx) return;  // no point of this warp
+    for (int a = 0; a < pitch; a += 8) {
+        double xn[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    for (int a = 0; a < ne; ++a) {
-        const double x = X[(size_t)a * nx + p];
+        for (int i = 0; i < 8; ++i) xn[i] = in && a + 8 + i < ne ? X[(size_t)(a + 8 + i) * nx + p] : 0.0;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) acc[q] = fma(x, Ts[(cg * 8 + q) * ne + a], acc[q]);
+        for (int i = 0; i < 8; i += 2)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const double2 t = Ts2[(q * pitch + a + i) >> 1];
+                acc[q] = fma(x[i], t.x, acc[q]);
+                acc[q] = fma(x[i + 1], t.y, acc[q]);
+            }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = xn[i];
     }
+    if (!in) return;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int c = c0 + cg * 8 + q;
+    for (int q = 0; q < Q; ++q) {
+        const int c = c0 + q;
         if (c < ne)
             members[(size_t)c * nx + p] = (T)((double)members[(size_t)c * nx + p] + acc[q]);
         else if (c == ne)
@@ -947,15 +970,38 @@ __global__ void __launch_bounds__(256) k_update_f64(T *__restrict__ members, T *
     }
 }
 
+// columns per warp: the fewest rounds of CTAs times the work of one (its
+// columns, and about 16 instructions to start and end); of equal ones the most
+static int update_cols(size_t nx, int ne) {
+    const long long pb = (long long)((nx + 32 * kUpdateWarps - 1) / (32 * kUpdateWarps));
+    int best = 1;
+    long long cost = 0;
+    for (int q = 1; q <= kUpdateMaxCols; ++q) {
+        const long long ctas = pb * ceil_div(ne + 1, q);
+        const long long c = (ctas + kNumSMs - 1) / kNumSMs * ((long long)q * ne + 16);
+        if (q == 1 || c <= cost) {
+            cost = c;
+            best = q;
+        }
+    }
+    return best;
+}
+
+template <typename T, int Q>
+static void update_launch(int cols, T *members, T *dC, const double *X, const double *Tm, size_t nx, int ne,
+                          const int *status, cudaStream_t s) {
+    if constexpr (Q > 1)
+        if (cols < Q) return update_launch<T, Q - 1>(cols, members, dC, X, Tm, nx, ne, status, s);
+    const dim3 grid(ceil_div(nx, 32 * kUpdateWarps), ceil_div(ne + 1, Q));
+    const size_t smem = sizeof(double) * Q * (size_t)((ne + 7) & ~7);  // <= 32 KB for ne <= 512
+    k_update_f64<T, Q><<<grid, 32 * kUpdateWarps, smem, s>>>(members, dC, X, Tm, nx, ne, status);
+}
+
 template <typename T>
 void launch_update_f64(T *members, T *dC, const double *X, const double *Tm, size_t nx, int ne,
                        const int *status, cudaStream_t s) {
     count_launches(1);
-    dim3 grid(ceil_div(nx, 64), ceil_div(ne + 1, 32));
-    const size_t smem = sizeof(double) * 32 * (size_t)ne;  // <= 128 KB for ne <= 512
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_update_f64<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_update_f64<T><<<grid, 256, smem, s>>>(members, dC, X, Tm, nx, ne, status);
+    update_launch<T, kUpdateMaxCols>(update_cols(nx, ne), members, dC, X, Tm, nx, ne, status, s);
 }
 
 // BF16 anomaly product with FP32 accumulation (CUDA-core version): X^T tile of
