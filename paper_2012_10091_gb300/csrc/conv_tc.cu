@@ -38,16 +38,18 @@
 // bytes on, the next 8 channels one plane on): M = 128 = the splits of d
 // stacked (their rows are added at the end), N = the input channels of one
 // tap, all nine taps and the bias column (ones) in TMEM for the whole run of
-// rows of a CTA.  Input rows live in a ring, so each is loaded once.  Five warps
-// issue two taps each (the last layer: 187 us with one issuing thread, 138 with
-// five warps); each MMA then takes about 54 cycles, 32 of them the reads of
-// its 4 KB A operand from shared memory.  Every FLUSH rows the accumulators are
+// rows of a CTA.  Input rows live in a ring, so each is loaded once (two of eight
+// twice, see WgradShape).  An MMA takes the three taps of one dx, the channel
+// groups of three consecutive rows being evenly spaced: N = 96 instead of 32
+// for the same 4 KB of A read from shared memory (32 cycles of the 54 an MMA of
+// N = 32 takes; one warp per dx and one for the bias issue).  8 x 256^2:
+// last layer 97 us, one tap at a time 147; middle 56 (80), first 49 (74).  Every FLUSH rows the accumulators are
 // added to sums in registers (10 us more for the last layer): the tensor cores
 // truncate, and over a whole run of rows the bias grew to 2e-6 of the gradient
 // against 9e-7 now and 8e-7 on the FP32 pipes.
 //
 // Measured, 8 samples of 256^2 coarse points: the loss and all gradients 5.4 ms
-// with the backward pass on the CUDA cores, 0.70 ms here; inference of one
+// with the backward pass on the CUDA cores, 0.60 ms here; inference of one
 // sample 80 us, 27 us here.
 //
 // Rows and pixels past the map's edge are computed from wrapped inputs (zeros
@@ -502,7 +504,9 @@ struct WgradShape {
     static constexpr int B_ROW = CGB * BPL;                 // one row of the input
     static constexpr int USED = 9 * N + 16;                 // TMEM columns: nine taps and the bias
     static constexpr int TMEM_COLS = tmem_cols(USED);
-    static constexpr int NEED = 1024 + NST * A_STAGE + 8 * B_ROW + 2 * APL;
+    // a ring of eight input rows, the first two once more behind them: the three
+    // rows around a gradient row are always consecutive in memory
+    static constexpr int NEED = 1024 + NST * A_STAGE + 10 * B_ROW + 2 * APL;
     static constexpr int SMEM = NEED > tmem_min_smem(TMEM_COLS) ? NEED : tmem_min_smem(TMEM_COLS);
     static_assert(COUT == 32 || COUT == 64, "the stacked splits fill one or two M = 128 operands");
     static_assert(NST * A_STAGE >= 128 * (N + 1) * 4, "the epilogue's tile of one tap reuses the stages");
@@ -522,15 +526,15 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sa = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    unsigned char *sb = sa + S::NST * S::A_STAGE;  // ring of eight input rows
-    unsigned char *s1 = sb + 8 * S::B_ROW;         // two planes of ones: the bias operand
+    unsigned char *sb = sa + S::NST * S::A_STAGE;  // ring of eight input rows, and two again
+    unsigned char *s1 = sb + 10 * S::B_ROW;        // two planes of ones: the bias operand
     __shared__ uint64_t bar[S::NST];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         s_fail = status ? *status : 0;
-        for (int q = 0; q < S::NST; ++q) tc::mbar_init(&bar[q], 5);
+        for (int q = 0; q < S::NST; ++q) tc::mbar_init(&bar[q], 4);
         fence_async_proxy();
     }
     __syncthreads();
@@ -548,7 +552,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
         reinterpret_cast<uint4 *>(sa + st * S::A_STAGE + S::ZERO * S::AG * S::APL)[k] = make_uint4(0, 0, 0, 0);
     }
     if (CGI < 2)
-        for (int e = tid; e < 8 * kRowW; e += kConvThreads)
+        for (int e = tid; e < 10 * kRowW; e += kConvThreads)
             reinterpret_cast<uint4 *>(sb + (e / kRowW) * S::B_ROW + S::BPL)[e % kRowW] = make_uint4(0, 0, 0, 0);
     for (int e = tid; e < 2 * S::PXS; e += kConvThreads) {
         const uint32_t one2 = 0x3F803F80u;  // two BF16 ones
@@ -558,16 +562,20 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
     int gx[XC];
 #pragma unroll
     for (int q = 0; q < XC; ++q) gx[q] = wrap_c8(x0 - 1 + lane + 32 * q, n);
-    // input row y (map row, may be -1 .. n) into ring slot (y - r0 + 1) mod 8
+    // input row y (map row, may be -1 .. n) into ring slot s = (y - r0 + 1) mod 8
+    // (and s + 8)
     auto load_in = [&](int y) {
-        const int gy = wrap_c8(y, n);
-        const uint32_t dst = tc::smem_u32(sb + ((y - r0 + 1) & 7) * S::B_ROW);
+        const int gy = wrap_c8(y, n), slot = (y - r0 + 1) & 7;
+        const uint32_t dst = tc::smem_u32(sb + slot * S::B_ROW);
         for (int g = warp; g < CGI; g += kConvThreads / 32) {
             const __nv_bfloat16 *src = in + (((size_t)b * CGI + g) * pl + (size_t)gy * n) * 8;
 #pragma unroll
             for (int q = 0; q < XC; ++q)
-                if (q < XC - 1 || lane + 32 * q < kPix + 2)
+                if (q < XC - 1 || lane + 32 * q < kPix + 2) {
                     cp_async16_cg(dst + g * S::BPL + (lane + 32 * q) * 16, src + (size_t)gx[q] * 8);
+                    if (slot < 2)
+                        cp_async16_cg(dst + 8 * S::B_ROW + g * S::BPL + (lane + 32 * q) * 16, src + (size_t)gx[q] * 8);
+                }
         }
     };
     // step q: pixels PXS (q mod SPR) .. of gradient row r0 + q / SPR into stage
@@ -597,8 +605,9 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
     }
     uint32_t tmem = 0;
     bool ok = true;
-    // the running sums: warps 0-3 hold taps 0-4 of their 32 accumulator rows,
-    // warps 4-7 taps 5-8 and the bias
+    // the running sums: warps 0-3 hold five taps of their 32 accumulator rows,
+    // warps 4-7 four and the bias; block t of the accumulators is tap
+    // (t mod 3, t / 3)
     const int half = warp >> 2;
     constexpr int HT = 5;
     float sum[HT * S::N];
@@ -614,25 +623,21 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
         }
         tc::fence_after_sync();
         tmem = tmem_slot;
-        if (uwarp < 5) {
+        if (uwarp < 4) {
             // both operands MN-major (instruction bits 15, 16); K groups 128 bytes
-            // apart, channel groups one plane apart.  Warp w issues taps 2 w and
-            // 2 w + 1 (tap 9: the bias)
+            // apart, channel groups one plane apart.  Warp w < 3 issues the taps
+            // (0 .. 2, w), whose operands are the channel groups of three
+            // consecutive rows; warp 3 the bias
             constexpr uint32_t mn = (1u << 15) | (1u << 16);
-            constexpr uint32_t idesc = tc::idesc_bf16(128, S::N) | mn, idesc1 = tc::idesc_bf16(128, 16) | mn;
+            const uint32_t idesc = (uwarp == 3 ? tc::idesc_bf16(128, 16) : tc::idesc_bf16(128, 3 * S::N)) | mn;
             const bool lead = tc::elect_one();
             const int i = q / SPR, px = (q % SPR) * S::PXS;
-            const uint32_t aa = tc::smem_u32(sa + (q % S::NST) * S::A_STAGE), bb = tc::smem_u32(sb),
-                           b1 = tc::smem_u32(s1);
-            // row r0 + i - 1 + dy sits in slot (i + dy) mod 8
-            uint32_t bt[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int t = 2 * uwarp + h;
-                bt[h] = t == 9 ? b1 : bb + (uint32_t)(((i + t / 3) & 7) * S::B_ROW + (px + t % 3) * 16);
-            }
-            const uint32_t id1 = uwarp == 4 ? idesc1 : idesc, pitch1 = uwarp == 4 ? S::APL : S::BPL;
-            const uint32_t dt = tmem + (uint32_t)(2 * uwarp * S::N);
+            const uint32_t aa = tc::smem_u32(sa + (q % S::NST) * S::A_STAGE);
+            // row r0 + i - 1 + dy sits in slot i mod 8 + dy
+            const uint32_t bt = uwarp == 3 ? tc::smem_u32(s1)
+                                           : tc::smem_u32(sb) + (uint32_t)((i & 7) * S::B_ROW + (px + uwarp) * 16);
+            const uint32_t pitch = uwarp == 3 ? S::APL : S::BPL;
+            const uint32_t dt = tmem + (uint32_t)(3 * uwarp * S::N);
 #pragma unroll
             for (int k = 0; k < S::PXS / 16; ++k) {
 #pragma unroll
@@ -640,9 +645,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
                     const uint64_t ad =
                         tc::smem_desc_interleave(aa + (uint32_t)(m * 16 * S::APL + k * 256), 128, S::APL);
                     const uint32_t acc = ((q % (S::FLUSH * SPR)) | k | m) ? 1u : 0u;
-                    tc::mma_bf16_lead(lead, dt, ad, tc::smem_desc_interleave(bt[0] + k * 256, 128, S::BPL), idesc, acc);
-                    tc::mma_bf16_lead(lead, dt + S::N, ad, tc::smem_desc_interleave(bt[1] + k * 256, 128, pitch1), id1,
-                                      acc);
+                    tc::mma_bf16_lead(lead, dt, ad, tc::smem_desc_interleave(bt + k * 256, 128, pitch), idesc, acc);
                 }
             }
             if (lead) tc::mma_commit(&bar[q % S::NST]);
@@ -703,7 +706,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
                 const int o = e / width, c = e - o * width;
                 float v = tile[o * LD + c] + tile[(o + COUT) * LD + c];
                 if (COUT == 32) v += tile[(o + 2 * COUT) * LD + c];
-                out[(size_t)t * COUT * CIN + e] = v;
+                out[(size_t)(t < 9 ? t % 3 * 3 + t / 3 : t) * COUT * CIN + e] = v;
             }
             __syncthreads();
         }
