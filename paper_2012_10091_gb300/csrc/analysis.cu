@@ -454,35 +454,40 @@ void launch_ens_anom(const T *members, size_t nx, int ne, double *X64, __nv_bflo
 // FP64 GEMMs of the gain (Algorithm 3 step 8)
 // ---------------------------------------------------------------------------
 // [out1 | out2^T] = A [B1; B2]^T / divisor (+ diag on out1's diagonal), FP64.
-// One 16 x 16 output tile per CTA of 256 threads, one output per thread, k in
-// chunks of 32 staged in shared memory; the next chunk's loads are issued
-// before the current chunk's FMAs, so they are in flight while GB300's slow
-// FP64 pipe works.  When B1 is A and n1 = m, out1 = A A^T / divisor + diag I is
-// symmetric: tiles strictly below its diagonal are not computed (a quarter of
-// the FMAs of S = I + Y^T R^-1 Y [Y | D | d*]), their values are the mirror
-// of the tiles above (the same products, so the same bits).
+// One 8 x 16 output tile per CTA of 128 threads (a warp on each scheduler), one
+// output per thread, k in chunks of 32 staged in shared memory; the next
+// chunk's loads are issued before the current chunk's FMAs, so they are in
+// flight while GB300's slow FP64 pipe works.  When B1 is A and n1 = m, out1 = A
+// A^T / divisor + diag I is symmetric: 16 x 16 tiles strictly below its diagonal
+// are not computed (a quarter of the FMAs of S = I + Y^T R^-1 Y [Y | D | d*]),
+// their values are the mirror of the tiles above (the same products, so the
+// same bits).  The K splits of a tile are a cluster: the partial sums stay in
+// shared memory and are added, in the order of the splits, by the CTA that
+// writes the output.  Bound by the FP64 pipes of the SM with the most CTAs:
+// half the tile of before (16 x 16, two warps per scheduler) evens them out.
+// S and T of 128 members, 512 observations: 36 us and 5 us for a reduction
+// launch, 38 us so; 100 members, 80 observations: 12 and 9.5 us.
+constexpr int kGemmThreads = 128, kGemmRows = 8;
+constexpr int kGemmMaxPer = 4;  // splits per CTA of a cluster of 8
 __device__ __forceinline__ double gemm_nt_tile(const double *__restrict__ A, int m, const double *__restrict__ B1,
                                                int n1, const double *__restrict__ B2, int n2, int K, int kb,
-                                               int ke, int a0, int c0, double (&As)[16][33],
-                                               double (&Bs)[16][33]) {
+                                               int ke, int a0, int c0) {
+    __shared__ double As[kGemmRows][33], Bs[16][33];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const double *arow[2], *brow[2];
-    int rr[2], kq[2];
+    const int kq = threadIdx.x & 31, rr = threadIdx.x >> 5;  // staging: column, and rows rr, rr + 4, ...
+    const double *arow[2], *brow[4];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int e = threadIdx.x + 256 * q;
-        rr[q] = e >> 5;
-        kq[q] = e & 31;
-        const int a = a0 + rr[q], c = c0 + rr[q];
-        arow[q] = a < m ? A + (size_t)a * K : nullptr;
+    for (int q = 0; q < 4; ++q) {
+        const int a = a0 + rr + 4 * q, c = c0 + rr + 4 * q;
+        if (q < 2) arow[q] = a < m ? A + (size_t)a * K : nullptr;
         brow[q] = c < n1 ? B1 + (size_t)c * K : (c < n1 + n2 ? B2 + (size_t)(c - n1) * K : nullptr);
     }
-    double va[2], vb[2];
+    double va[2], vb[4];
     auto fetch = [&](int k0) {
+        const int k = k0 + kq;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int k = k0 + kq[q];
-            va[q] = (arow[q] && k < ke) ? arow[q][k] : 0.0;
+        for (int q = 0; q < 4; ++q) {
+            if (q < 2) va[q] = (arow[q] && k < ke) ? arow[q][k] : 0.0;
             vb[q] = (brow[q] && k < ke) ? brow[q][k] : 0.0;
         }
     };
@@ -490,61 +495,90 @@ __device__ __forceinline__ double gemm_nt_tile(const double *__restrict__ A, int
     double acc = 0.0;
     for (int k0 = kb; k0 < ke; k0 += 32) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            As[rr[q]][kq[q]] = va[q];
-            Bs[rr[q]][kq[q]] = vb[q];
+        for (int q = 0; q < 4; ++q) {
+            if (q < 2) As[rr + 4 * q][kq] = va[q];
+            Bs[rr + 4 * q][kq] = vb[q];
         }
         __syncthreads();
         if (k0 + 32 < ke) fetch(k0 + 32);
+        for (int k8 = 0; k8 < min(32, ke - k0); k8 += 8)  // zeros past ke
 #pragma unroll
-        for (int kk = 0; kk < 32; ++kk) acc = fma(As[ty][kk], Bs[tx][kk], acc);
+            for (int kk = 0; kk < 8; ++kk) acc = fma(As[ty][k8 + kk], Bs[tx][k8 + kk], acc);
         __syncthreads();
     }
     return acc;
 }
 
-// Output tile (bx, by) of [out1 | out2^T]: over the whole of K with the
-// epilogue (part == NULL), or over K chunk bz into the split-K partial sums.
-__device__ __forceinline__ void gemm_nt_block(const double *__restrict__ A, int m, const double *__restrict__ B1,
-                                              int n1, const double *__restrict__ B2, int n2, int K, double divisor,
-                                              double diag, double *__restrict__ out1, double *__restrict__ out2,
-                                              int bx, int by, int bz, int kchunk, double *__restrict__ part) {
+// output (a, c) of [out1 | out2^T] from its sum; mirror: also out1's (c, a)
+__device__ __forceinline__ void gemm_put(double acc, int a, int c, int m, int n1, int n2, bool mirror, double divisor,
+                                         double diag, double *__restrict__ out1, double *__restrict__ out2) {
+    if (a >= m) return;
+    if (c < n1) {
+        out1[(size_t)a * n1 + c] = (a == c ? diag : 0.0) + acc / divisor;
+        if (mirror) out1[(size_t)c * n1 + a] = acc / divisor;
+    } else if (c < n1 + n2) {
+        out2[(size_t)(c - n1) * m + a] = acc / divisor;
+    }
+}
+
+// The sums of a tile of E outputs over the splits of its cluster (gridDim.z
+// CTAs, `per` splits each): part[l][e] holds this CTA's; put(e, sum) is called
+// for the outputs of this CTA, E / gridDim.z of them.
+template <int E, class Put>
+__device__ __forceinline__ void gemm_cluster_sum(double (*part)[E], int per, Put put) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int ctas = gridDim.z, rank = blockIdx.z;
+    cl.sync();
+    const int share = E / ctas, e = rank * share + threadIdx.x;
+    if ((int)threadIdx.x < share) {
+        double acc = 0.0;
+#pragma unroll 4
+        for (int z = 0; z < ctas * per; ++z) acc += cl.map_shared_rank(&part[0][0], z / per)[(z % per) * E + e];
+        put(e, acc);
+    }
+    cl.sync();  // no CTA leaves while another may still read its partial sums
+}
+
+// tile (blockIdx.x, blockIdx.y), splits of kchunk, `per` of them in each CTA of
+// the cluster along z
+__global__ void __launch_bounds__(kGemmThreads)
+    k_gemm_nt(const double *__restrict__ A, int m, const double *__restrict__ B1, int n1,
+              const double *__restrict__ B2, int n2, int K, int per, int kchunk, double divisor, double diag,
+              double *__restrict__ out1, double *__restrict__ out2, const int *status) {
+    if (status && *status) return;
+    __shared__ double part[kGemmMaxPer][kGemmThreads];
     const bool sym = B1 == A && n1 == m;
-    if (sym && bx < by) return;  // mirrored from tile (by, bx) (by the reduce when split)
-    __shared__ double As[16][33];
-    __shared__ double Bs[16][33];
-    const int a0 = by * 16, c0 = bx * 16;
-    const int kb = part ? bz * kchunk : 0, ke = part ? min(K, kb + kchunk) : K;
-    const double acc = gemm_nt_tile(A, m, B1, n1, B2, n2, K, kb, ke, a0, c0, As, Bs);
+    const int a0 = blockIdx.y * kGemmRows, c0 = blockIdx.x * 16;
+    if (sym && c0 < (a0 & ~15)) return;  // mirrored from the tile above the diagonal
+    const bool mirror = sym && c0 > (a0 & ~15);
+    auto put = [&](int e, double acc) {
+        gemm_put(acc, a0 + (e >> 4), c0 + (e & 15), m, n1, n2, mirror, divisor, diag, out1, out2);
+    };
+    double acc = 0.0;
+    for (int l = 0; l < per; ++l) {
+        const int kb = (blockIdx.z * per + l) * kchunk;
+        acc = gemm_nt_tile(A, m, B1, n1, B2, n2, K, kb, min(K, kb + kchunk), a0, c0);
+        part[l][threadIdx.x] = acc;
+    }
+    if (gridDim.z == 1)
+        put(threadIdx.x, acc);
+    else
+        gemm_cluster_sum(part, per, put);
+}
+
+// Partial sums over K chunks in memory, for more splits than a cluster takes.
+__global__ void __launch_bounds__(kGemmThreads)
+    k_gemm_nt_split(const double *__restrict__ A, int m, const double *__restrict__ B1, int n1,
+                    const double *__restrict__ B2, int n2, int K, int kchunk, double *__restrict__ part,
+                    const int *status) {
+    if (status && *status) return;
+    const int a0 = blockIdx.y * kGemmRows, c0 = blockIdx.x * 16;
+    if (B1 == A && n1 == m && c0 < (a0 & ~15)) return;
+    const int kb = blockIdx.z * kchunk;
+    const double acc = gemm_nt_tile(A, m, B1, n1, B2, n2, K, kb, min(K, kb + kchunk), a0, c0);
     const int a = a0 + (threadIdx.x >> 4), c = c0 + (threadIdx.x & 15);
-    if (part) {
-        if (a < m && c < n1 + n2) part[((size_t)bz * m + a) * (n1 + n2) + c] = acc;
-        return;
-    }
-    if (a < m) {
-        if (c < n1) {
-            out1[(size_t)a * n1 + c] = (a == c ? diag : 0.0) + acc / divisor;
-            if (sym && bx > by) out1[(size_t)c * n1 + a] = acc / divisor;
-        } else if (c < n1 + n2) {
-            out2[(size_t)(c - n1) * m + a] = acc / divisor;
-        }
-    }
-}
-
-__global__ void k_gemm_nt(const double *__restrict__ A, int m, const double *__restrict__ B1, int n1,
-                          const double *__restrict__ B2, int n2, int K, double divisor, double diag,
-                          double *__restrict__ out1, double *__restrict__ out2, const int *status) {
-    if (status && *status) return;
-    gemm_nt_block(A, m, B1, n1, B2, n2, K, divisor, diag, out1, out2, blockIdx.x, blockIdx.y, 0, K, nullptr);
-}
-
-// Partial sums of k_gemm_nt over K chunks (split-K), combined in chunk order.
-__global__ void k_gemm_nt_split(const double *__restrict__ A, int m, const double *__restrict__ B1,
-                                int n1, const double *__restrict__ B2, int n2, int K, int kchunk,
-                                double *__restrict__ part, const int *status) {
-    if (status && *status) return;
-    gemm_nt_block(A, m, B1, n1, B2, n2, K, 1.0, 0.0, nullptr, nullptr, blockIdx.x, blockIdx.y, blockIdx.z, kchunk,
-                  part);
+    if (a < m && c < n1 + n2) part[((size_t)blockIdx.z * m + a) * (n1 + n2) + c] = acc;
 }
 
 __device__ __forceinline__ void gemm_nt_reduce_body(const double *__restrict__ part, int nsplit, int m, int n1,
@@ -599,31 +633,29 @@ __device__ __forceinline__ void df_mac(float ah, float al, float bh, float bl, f
     s = t;
 }
 
-constexpr int kDfThreads = 64;  // a 16 x 16 output tile, 2 x 2 outputs per thread
-constexpr int kDfK = 32;        // K chunk staged in shared memory
+constexpr int kDfThreads = 256;  // a 16 x 16 output tile: four groups of 64 threads, 2 x 2 outputs per thread
+constexpr int kDfK = 32;         // K chunk staged in shared memory
 
-// Output tile (bx, by) of [S | Y^T R^-1 [D | d*]] as gemm_nt_block (A = B1 = Y,
-// m = n1 = ne, B2 = Z, n2 = ne + 1, symmetric S: tiles with bx < by are not
-// computed), from the double-FP32 operands.
-__device__ __forceinline__ void gemm_df_block(const DfOperands &df, int ne, int K, double divisor, double diag,
-                                              double *__restrict__ out1, double *__restrict__ out2, int bx, int by,
-                                              int bz, int kchunk, double *__restrict__ part) {
-    if (bx < by) return;
+// One output, (a0 + t / 16, c0 + t % 16) for thread t, of [Y^T R^-1 Y | Y^T R^-1
+// [D | d*]] over k in [kb, ke), from the double-FP32 operands.  Each group takes
+// a quarter of every K chunk, so that eight warps and not two hide the latency
+// of the error-free sums (64 members, 2048 observations: 24 us and a reduction
+// of 8, 17 us with the cluster's sums); the groups' sums are added in FP64.
+__device__ __forceinline__ double gemm_df_tile(const DfOperands &df, int ne, int K, int kb, int ke, int a0, int c0) {
     __shared__ float sAh[16][kDfK + 1], sAl[16][kDfK + 1], sBh[16][kDfK + 1], sBl[16][kDfK + 1];
+    __shared__ double red[4][256];
     const int m = ne, n1 = ne, n2 = ne + 1;
-    const int a0 = by * 16, c0 = bx * 16;
-    const int kb = part ? bz * kchunk : 0, ke = part ? min(K, kb + kchunk) : K;
-    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
-    // staging: row tid / 4 of the A and B tiles, k = (tid mod 4) * 8 .. + 7 of the chunk
-    const int sr = tid >> 2, sk = (tid & 3) * 8;
+    const int tid = threadIdx.x, grp = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
+    // staging: row tid / 16 of the A and B tiles, k = (tid mod 16) * 2 and the next of the chunk
+    const int sr = tid >> 4, sk = (tid & 15) * 2;
     const int ar = a0 + sr, cr = c0 + sr;
     const float *ah = ar < m ? df.Yh + (size_t)ar * K : nullptr, *al = ar < m ? df.Yl + (size_t)ar * K : nullptr;
     const float *bh = cr < n1 ? df.Yh + (size_t)cr * K : (cr < n1 + n2 ? df.Zh + (size_t)(cr - n1) * K : nullptr);
     const float *bl = cr < n1 ? df.Yl + (size_t)cr * K : (cr < n1 + n2 ? df.Zl + (size_t)(cr - n1) * K : nullptr);
-    float va[2][8], vb[2][8];
+    float va[2][2], vb[2][2];
     auto fetch = [&](int k0) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 2; ++j) {
             const int k = k0 + sk + j;
             const bool ok = k < ke;
             va[0][j] = (ah && ok) ? ah[k] : 0.f;
@@ -636,7 +668,7 @@ __device__ __forceinline__ void gemm_df_block(const DfOperands &df, int ne, int 
     fetch(kb);
     for (int k0 = kb; k0 < ke; k0 += kDfK) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 2; ++j) {
             sAh[sr][sk + j] = va[0][j];
             sAl[sr][sk + j] = va[1][j];
             sBh[sr][sk + j] = vb[0][j];
@@ -645,7 +677,7 @@ __device__ __forceinline__ void gemm_df_block(const DfOperands &df, int ne, int 
         __syncthreads();
         if (k0 + kDfK < ke) fetch(k0 + kDfK);  // in flight during the chunk's products
 #pragma unroll 4
-        for (int kk = 0; kk < kDfK; ++kk) {
+        for (int kk = grp * (kDfK / 4); kk < (grp + 1) * (kDfK / 4); ++kk) {
             float xh[2], xl[2], yh[2], yl[2];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
@@ -664,39 +696,75 @@ __device__ __forceinline__ void gemm_df_block(const DfOperands &df, int ne, int 
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int a = a0 + 2 * ty + i, cc = c0 + 2 * tx + j;
-            const double acc = (double)s[i][j] + (double)c[i][j];
-            if (part) {
-                if (a < m && cc < n1 + n2) part[((size_t)bz * m + a) * (n1 + n2) + cc] = acc;
-                continue;
-            }
-            if (a < m) {
-                if (cc < n1) {
-                    out1[(size_t)a * n1 + cc] = (a == cc ? diag : 0.0) + acc / divisor;
-                    if (bx > by) out1[(size_t)cc * n1 + a] = acc / divisor;
-                } else if (cc < n1 + n2) {
-                    out2[(size_t)(cc - n1) * m + a] = acc / divisor;
-                }
-            }
-        }
+        for (int j = 0; j < 2; ++j)
+            red[grp][(2 * ty + i) * 16 + 2 * tx + j] = (double)s[i][j] + (double)c[i][j];
+    __syncthreads();
+    const double acc = ((red[0][tid] + red[1][tid]) + red[2][tid]) + red[3][tid];
+    __syncthreads();  // red may be written again
+    return acc;
 }
 
-__global__ void __launch_bounds__(kDfThreads) k_gemm_df(DfOperands df, int ne, int K, double divisor, double diag,
-                                                        double *__restrict__ out1, double *__restrict__ out2,
-                                                        int kchunk, double *__restrict__ part, const int *status) {
+__global__ void __launch_bounds__(kDfThreads) k_gemm_df(DfOperands df, int ne, int K, int per, int kchunk,
+                                                        double divisor, double diag, double *__restrict__ out1,
+                                                        double *__restrict__ out2, double *__restrict__ parts,
+                                                        const int *status) {
     if (*status) return;
-    gemm_df_block(df, ne, K, divisor, diag, out1, out2, blockIdx.x, blockIdx.y, blockIdx.z, kchunk, part);
+    __shared__ double part[kGemmMaxPer][kDfThreads];
+    const int a0 = blockIdx.y * 16, c0 = blockIdx.x * 16, m = ne, n1 = ne, n2 = ne + 1;
+    if (c0 < a0) return;  // mirrored from the tile above the diagonal
+    auto put = [&](int e, double acc) {
+        gemm_put(acc, a0 + (e >> 4), c0 + (e & 15), m, n1, n2, c0 > a0, divisor, diag, out1, out2);
+    };
+    double acc = 0.0;
+    for (int l = 0; l < per; ++l) {
+        const int kb = (blockIdx.z * per + l) * kchunk;
+        acc = gemm_df_tile(df, ne, K, kb, min(K, kb + kchunk), a0, c0);
+        part[l][threadIdx.x] = acc;
+    }
+    if (parts) {  // more splits than a cluster takes: partial sums in memory
+        const int a = a0 + (threadIdx.x >> 4), c = c0 + (threadIdx.x & 15);
+        if (a < m && c < n1 + n2) parts[((size_t)blockIdx.z * m + a) * (n1 + n2) + c] = acc;
+    } else if (gridDim.z == 1) {
+        put(threadIdx.x, acc);
+    } else {
+        gemm_cluster_sum(part, per, put);
+    }
+}
+
+// cluster of the K splits (a power of two): CTAs and splits per CTA, or 0 CTAs
+// if there are more than a portable cluster takes
+struct GemmCluster {
+    int ctas, per;
+};
+static GemmCluster gemm_cluster(int splits) {
+    const int ctas = std::min(splits, 8), per = splits / ctas;
+    return per <= kGemmMaxPer ? GemmCluster{ctas, per} : GemmCluster{0, 1};
+}
+template <class... P, class... Args>
+static void gemm_launch(void (*kernel)(P...), dim3 grid, int threads, int cluster, cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = cluster;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 void launch_gemm_df(const DfOperands &df, int ne, int ny, double s2, double *S, double *Bt, const int *status,
                     cudaStream_t s, double *part) {
     const int splits = part ? gemm_nt_splits(ne, ne, ne + 1, ny) : 1;
     const int kchunk = ceil_div(ceil_div(ny, splits), 32) * 32;
-    dim3 grid(ceil_div(2 * ne + 1, 16), ceil_div(ne, 16), splits);
-    count_launches(splits > 1 ? 2 : 1);
-    k_gemm_df<<<grid, kDfThreads, 0, s>>>(df, ne, ny, s2, 1.0, S, Bt, kchunk, splits > 1 ? part : nullptr, status);
-    if (splits > 1)
+    const GemmCluster g = gemm_cluster(splits);
+    const dim3 grid(ceil_div(2 * ne + 1, 16), ceil_div(ne, 16), g.ctas ? g.ctas : splits);
+    count_launches(g.ctas ? 1 : 2);
+    gemm_launch(k_gemm_df, grid, kDfThreads, g.ctas, s, df, ne, ny, g.per, kchunk, s2, 1.0, S, Bt,
+                g.ctas ? (double *)nullptr : part, status);
+    if (!g.ctas)
         k_gemm_nt_reduce<<<grid_for((size_t)ne * (2 * ne + 1), 256), 256, 0, s>>>(part, splits, ne, ne, ne + 1, true,
                                                                                 s2, 1.0, S, Bt, status);
 }
@@ -705,18 +773,18 @@ void launch_gemm_nt_f64(const double *A, int m, const double *B1, int n1, const 
                         int K, double scale_div, double diag, double *out1, double *out2,
                         const int *status, cudaStream_t s, double *part) {
     const int splits = part ? gemm_nt_splits(m, n1, n2, K) : 1;
-    if (splits > 1) {
-        count_launches(2);
-        const int kchunk = ceil_div(ceil_div(K, splits), 32) * 32;
-        dim3 grid(ceil_div(n1 + n2, 16), ceil_div(m, 16), splits);
-        k_gemm_nt_split<<<grid, 256, 0, s>>>(A, m, B1, n1, B2, n2, K, kchunk, part, status);
-        k_gemm_nt_reduce<<<grid_for((size_t)m * (n1 + n2), 256), 256, 0, s>>>(
-            part, splits, m, n1, n2, B1 == A && n1 == m, scale_div, diag, out1, out2, status);
+    const int kchunk = ceil_div(ceil_div(K, splits), 32) * 32;
+    const GemmCluster g = gemm_cluster(splits);
+    const dim3 grid(ceil_div(n1 + n2, 16), ceil_div(m, kGemmRows), g.ctas ? g.ctas : splits);
+    count_launches(g.ctas ? 1 : 2);
+    if (g.ctas) {
+        gemm_launch(k_gemm_nt, grid, kGemmThreads, g.ctas, s, A, m, B1, n1, B2, n2, K, g.per, kchunk, scale_div, diag,
+                    out1, out2, status);
         return;
     }
-    count_launches(1);
-    dim3 grid(ceil_div(n1 + n2, 16), ceil_div(m, 16));
-    k_gemm_nt<<<grid, 256, 0, s>>>(A, m, B1, n1, B2, n2, K, scale_div, diag, out1, out2, status);
+    k_gemm_nt_split<<<grid, kGemmThreads, 0, s>>>(A, m, B1, n1, B2, n2, K, kchunk, part, status);
+    k_gemm_nt_reduce<<<grid_for((size_t)m * (n1 + n2), 256), 256, 0, s>>>(
+        part, splits, m, n1, n2, B1 == A && n1 == m, scale_div, diag, out1, out2, status);
 }
 
 __global__ void k_gemm_tn(const double *__restrict__ Y, int ne, int ny, double diag,
@@ -1343,7 +1411,15 @@ __global__ void __launch_bounds__(kDfThreads) kg_gemm(const GroupProb *__restric
     if (*g.status) return;
     const int ne = g.ne, tx = ceil_div(2 * ne + 1, 16), ty = ceil_div(ne, 16);
     const int bx = e.y % tx, by = (e.y / tx) % ty, bz = e.y / (tx * ty);
-    gemm_df_block(g.df, ne, g.ny, g.s2, 1.0, g.S, g.Bt, bx, by, bz, g.kchunk, g.splits > 1 ? g.part : nullptr);
+    const int a0 = by * 16, c0 = bx * 16, n1 = ne, n2 = ne + 1;
+    if (c0 < a0) return;  // mirrored from the tile above the diagonal (by the reduction when split)
+    const int kb = g.splits > 1 ? bz * g.kchunk : 0, ke = g.splits > 1 ? min(g.ny, kb + g.kchunk) : g.ny;
+    const double acc = gemm_df_tile(g.df, ne, g.ny, kb, ke, a0, c0);
+    const int a = a0 + (threadIdx.x >> 4), c = c0 + (threadIdx.x & 15);
+    if (g.splits == 1)
+        gemm_put(acc, a, c, ne, n1, n2, c0 > a0, g.s2, 1.0, g.S, g.Bt);
+    else if (a < ne && c < n1 + n2)
+        g.part[((size_t)bz * ne + a) * (n1 + n2) + c] = acc;
 }
 
 __global__ void __launch_bounds__(256) kg_gemm_reduce(const GroupProb *__restrict__ P, const int2 *__restrict__ map) {
