@@ -57,6 +57,7 @@ __device__ __forceinline__ void restrict_body(const T *__restrict__ fine, T *__r
 
 template <typename T>
 __global__ void k_restrict(const T *__restrict__ fine, T *__restrict__ xs, int dim, int V, int nc, int r) {
+    launch_wait();
     restrict_body<T>(fine, xs, dim, V, nc, r, blockIdx.x, gridDim.x, nullptr);
 }
 
@@ -64,7 +65,7 @@ template <typename T>
 void launch_restrict(const T *fine, T *xstar, int dim, int V, int nc, int r, cudaStream_t s) {
     count_launches(1);
     const size_t total = (size_t)V * (dim == 1 ? (size_t)nc : (size_t)nc * nc);
-    k_restrict<T><<<grid_for(total, 256), 256, 0, s>>>(fine, xstar, dim, V, nc, r);
+    launch_kernel(k_restrict<T>, grid_for(total, 256), 256, 0, s, LaunchHow{}, fine, xstar, dim, V, nc, r);
 }
 
 // ---------------------------------------------------------------------------
@@ -144,6 +145,7 @@ __global__ void __launch_bounds__(128) k_obs_apply(const T *__restrict__ members
                                                    const int32_t *__restrict__ tap_idx,
                                                    const double *__restrict__ tap_w, double *__restrict__ yf,
                                                    const float *__restrict__ wh, const float *__restrict__ wl) {
+    launch_wait();
     obs_apply_body<T>(members, xstar, nx, ne, ny, taps, tap_idx, tap_w, yf, blockIdx.x, blockIdx.y * kObsRowsOne,
                       kObsRowsOne, wh, wl);
 }
@@ -154,7 +156,8 @@ void launch_obs_apply(const T *members, const T *xstar, size_t nx, int ne, int n
                       const float *wl) {
     count_launches(1);
     dim3 grid(ceil_div(ny, 128), ceil_div(ne + 1, kObsRowsOne));
-    k_obs_apply<T><<<grid, 128, 0, s>>>(members, xstar, nx, ne, ny, taps, tap_idx, tap_w, yf, wh, wl);
+    launch_kernel(k_obs_apply<T>, grid, 128, 0, s, LaunchHow{}, members, xstar, nx, ne, ny, taps, tap_idx, tap_w, yf,
+                  wh, wl);
 }
 
 // ---------------------------------------------------------------------------
@@ -204,13 +207,15 @@ __global__ void __launch_bounds__(256) k_obs_mean(const double *__restrict__ yf,
                                                   int ne, double inv_ne, int ny, double *__restrict__ ybar,
                                                   double *__restrict__ Z, int *status, float *__restrict__ Zh,
                                                   float *__restrict__ Zl) {
+    launch_wait();
     obs_mean_body(yf, yo, ne, inv_ne, ny, ybar, Z, status, blockIdx.x, nullptr, Zh, Zl);
 }
 
 void launch_obs_mean(const double *yf, const double *yo, int ne, int ny, double *ybar, double *Z,
                      int *status, cudaStream_t s, float *Zh, float *Zl) {
     count_launches(1);
-    k_obs_mean<<<ceil_div(ny, 32), 256, 0, s>>>(yf, yo, ne, 1.0 / ne, ny, ybar, Z, status, Zh, Zl);
+    launch_kernel(k_obs_mean, ceil_div(ny, 32), 256, 0, s, LaunchHow{}, yf, yo, ne, 1.0 / ne, ny, ybar, Z, status, Zh,
+                  Zl);
 }
 
 // RMS of the innovation d* = y^o - H^C x^C* (one value; fixed-order FP64 sums)
@@ -228,11 +233,12 @@ __device__ __forceinline__ void innov_rms_body(const double *__restrict__ d, int
 }
 
 __global__ void __launch_bounds__(256) k_innov_rms(const double *__restrict__ d, int ny, double *__restrict__ out) {
+    launch_wait();
     innov_rms_body(d, ny, out);
 }
 
 void launch_innov_rms(const double *Z, int ne, int ny, double *out, cudaStream_t s) {
-    k_innov_rms<<<1, 256, 0, s>>>(Z + (size_t)ne * ny, ny, out);
+    launch_kernel(k_innov_rms, 1, 256, 0, s, LaunchHow{}, Z + (size_t)ne * ny, ny, out);
     count_launches(1);
 }
 
@@ -294,6 +300,7 @@ __global__ void k_obs_perturb(const double *__restrict__ yf, const double *__res
                               const uint64_t *__restrict__ cycle, double sigma, int ne, int ny, double isq,
                               double *__restrict__ Y, double *__restrict__ Z, float *__restrict__ Yh,
                               float *__restrict__ Yl, float *__restrict__ Zh, float *__restrict__ Zl) {
+    launch_wait();
     obs_perturb_body<F32>(yf, ybar, yo, eps, gen_eps, seed, cycle, sigma, ne, ny, isq, Y, Z, blockIdx.x, Yh, Yl, Zh,
                           Zl);
 }
@@ -307,11 +314,11 @@ void launch_obs_perturb(const double *yf, const double *ybar, const double *yo, 
     const unsigned grid = (unsigned)ceil_div(blocks, 128);
     const double isq = 1.0 / std::sqrt((double)(ne - 1));
     if (gen_eps == 2)
-        k_obs_perturb<true><<<grid, 128, 0, s>>>(yf, ybar, yo, eps, 1, seed, cycle, sigma, ne, ny, isq, Y, Z, df.Yh,
-                                                 df.Yl, df.Zh, df.Zl);
+        launch_kernel(k_obs_perturb<true>, grid, 128, 0, s, LaunchHow{}, yf, ybar, yo, eps, 1, seed, cycle, sigma, ne,
+                      ny, isq, Y, Z, df.Yh, df.Yl, df.Zh, df.Zl);
     else
-        k_obs_perturb<false><<<grid, 128, 0, s>>>(yf, ybar, yo, eps, gen_eps, seed, cycle, sigma, ne, ny, isq, Y, Z,
-                                                  df.Yh, df.Yl, df.Zh, df.Zl);
+        launch_kernel(k_obs_perturb<false>, grid, 128, 0, s, LaunchHow{}, yf, ybar, yo, eps, gen_eps, seed, cycle,
+                      sigma, ne, ny, isq, Y, Z, df.Yh, df.Yl, df.Zh, df.Zl);
 }
 
 // Fine-to-coarse feedback: the forecast ensemble re-centred on the restricted
@@ -320,6 +327,7 @@ void launch_obs_perturb(const double *yf, const double *ybar, const double *yo, 
 template <typename T>
 __global__ void __launch_bounds__(256) k_recentre(T *__restrict__ m, size_t nx, int ne, const T *__restrict__ xstar,
                                                   const int *status) {
+    launch_wait();
     if (*status) return;
     const size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (p >= nx) return;
@@ -332,7 +340,7 @@ __global__ void __launch_bounds__(256) k_recentre(T *__restrict__ m, size_t nx, 
 template <typename T>
 void launch_recentre(T *members, size_t nx, int ne, const T *xstar, const int *status, cudaStream_t s) {
     count_launches(1);
-    k_recentre<T><<<(unsigned)ceil_div(nx, 256), 256, 0, s>>>(members, nx, ne, xstar, status);
+    launch_kernel(k_recentre<T>, (unsigned)ceil_div(nx, 256), 256, 0, s, LaunchHow{}, members, nx, ne, xstar, status);
 }
 template void launch_recentre<float>(float *, size_t, int, const float *, const int *, cudaStream_t);
 template void launch_recentre<double>(double *, size_t, int, const double *, const int *, cudaStream_t);
@@ -430,6 +438,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_ens_anom(const T *__restrict__ m, size_t nx, int ne, double inv_ne,
                                                   double isq, double *__restrict__ X64,
                                                   __nv_bfloat16 *__restrict__ X16, int ldx, const int *status) {
+    launch_wait();
     ens_anom_body<T>(m, nx, ne, inv_ne, isq, X64, X16, ldx, status, blockIdx.x);
 }
 
@@ -446,8 +455,9 @@ void launch_ens_anom(const T *members, size_t nx, int ne, double *X64, __nv_bflo
     const size_t smem = ens_anom_smem(ldx);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_ens_anom<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_ens_anom<T><<<ceil_div(nx, 32), 256, smem, s>>>(members, nx, ne, 1.0 / ne, 1.0 / std::sqrt((double)(ne - 1)),
-                                                       X64, X16, ldx, status);
+    const int ctas = ceil_div(nx, 32);
+    launch_kernel(k_ens_anom<T>, ctas, 256, smem, s, LaunchHow{1, 1, 1, ctas <= kNumSMs / 4}, members, nx, ne,
+                  1.0 / ne, 1.0 / std::sqrt((double)(ne - 1)), X64, X16, ldx, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -546,6 +556,7 @@ __global__ void __launch_bounds__(kGemmThreads)
     k_gemm_nt(const double *__restrict__ A, int m, const double *__restrict__ B1, int n1,
               const double *__restrict__ B2, int n2, int K, int per, int kchunk, double divisor, double diag,
               double *__restrict__ out1, double *__restrict__ out2, const int *status) {
+    launch_wait();
     if (status && *status) return;
     __shared__ double part[kGemmMaxPer][kGemmThreads];
     const bool sym = B1 == A && n1 == m;
@@ -572,6 +583,7 @@ __global__ void __launch_bounds__(kGemmThreads)
     k_gemm_nt_split(const double *__restrict__ A, int m, const double *__restrict__ B1, int n1,
                     const double *__restrict__ B2, int n2, int K, int kchunk, double *__restrict__ part,
                     const int *status) {
+    launch_wait();
     if (status && *status) return;
     const int a0 = blockIdx.y * kGemmRows, c0 = blockIdx.x * 16;
     if (B1 == A && n1 == m && c0 < (a0 & ~15)) return;
@@ -603,6 +615,7 @@ __device__ __forceinline__ void gemm_nt_reduce_body(const double *__restrict__ p
 __global__ void k_gemm_nt_reduce(const double *__restrict__ part, int nsplit, int m, int n1, int n2, bool sym,
                                  double divisor, double diag, double *__restrict__ out1,
                                  double *__restrict__ out2, const int *status) {
+    launch_wait();
     if (status && *status) return;
     gemm_nt_reduce_body(part, nsplit, m, n1, n2, sym, divisor, diag, out1, out2, blockIdx.x, gridDim.x);
 }
@@ -708,6 +721,7 @@ __global__ void __launch_bounds__(kDfThreads) k_gemm_df(DfOperands df, int ne, i
                                                         double divisor, double diag, double *__restrict__ out1,
                                                         double *__restrict__ out2, double *__restrict__ parts,
                                                         const int *status) {
+    launch_wait();
     if (*status) return;
     __shared__ double part[kGemmMaxPer][kDfThreads];
     const int a0 = blockIdx.y * 16, c0 = blockIdx.x * 16, m = ne, n1 = ne, n2 = ne + 1;
@@ -740,21 +754,6 @@ static GemmCluster gemm_cluster(int splits) {
     const int ctas = std::min(splits, 8), per = splits / ctas;
     return per <= kGemmMaxPer ? GemmCluster{ctas, per} : GemmCluster{0, 1};
 }
-template <class... P, class... Args>
-static void gemm_launch(void (*kernel)(P...), dim3 grid, int threads, int cluster, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = cluster;
-    cfg.attrs = attr;
-    cfg.numAttrs = cluster > 1 ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 void launch_gemm_df(const DfOperands &df, int ne, int ny, double s2, double *S, double *Bt, const int *status,
                     cudaStream_t s, double *part) {
     const int splits = part ? gemm_nt_splits(ne, ne, ne + 1, ny) : 1;
@@ -762,11 +761,11 @@ void launch_gemm_df(const DfOperands &df, int ne, int ny, double s2, double *S, 
     const GemmCluster g = gemm_cluster(splits);
     const dim3 grid(ceil_div(2 * ne + 1, 16), ceil_div(ne, 16), g.ctas ? g.ctas : splits);
     count_launches(g.ctas ? 1 : 2);
-    gemm_launch(k_gemm_df, grid, kDfThreads, g.ctas, s, df, ne, ny, g.per, kchunk, s2, 1.0, S, Bt,
-                g.ctas ? (double *)nullptr : part, status);
+    launch_kernel(k_gemm_df, grid, kDfThreads, 0, s, LaunchHow{1, 1, (unsigned)std::max(g.ctas, 1)}, df, ne, ny,
+                  g.per, kchunk, s2, 1.0, S, Bt, g.ctas ? (double *)nullptr : part, status);
     if (!g.ctas)
-        k_gemm_nt_reduce<<<grid_for((size_t)ne * (2 * ne + 1), 256), 256, 0, s>>>(part, splits, ne, ne, ne + 1, true,
-                                                                                s2, 1.0, S, Bt, status);
+        launch_kernel(k_gemm_nt_reduce, grid_for((size_t)ne * (2 * ne + 1), 256), 256, 0, s, LaunchHow{}, part,
+                      splits, ne, ne, ne + 1, true, s2, 1.0, S, Bt, status);
 }
 
 void launch_gemm_nt_f64(const double *A, int m, const double *B1, int n1, const double *B2, int n2,
@@ -778,17 +777,20 @@ void launch_gemm_nt_f64(const double *A, int m, const double *B1, int n1, const 
     const dim3 grid(ceil_div(n1 + n2, 16), ceil_div(m, kGemmRows), g.ctas ? g.ctas : splits);
     count_launches(g.ctas ? 1 : 2);
     if (g.ctas) {
-        gemm_launch(k_gemm_nt, grid, kGemmThreads, g.ctas, s, A, m, B1, n1, B2, n2, K, g.per, kchunk, scale_div, diag,
-                    out1, out2, status);
+        const bool chained = grid.x * grid.y * grid.z <= 2u * kNumSMs;
+        launch_kernel(k_gemm_nt, grid, kGemmThreads, 0, s, LaunchHow{1, 1, (unsigned)g.ctas, chained}, A, m, B1, n1,
+                      B2, n2, K, g.per, kchunk, scale_div, diag, out1, out2, status);
         return;
     }
-    k_gemm_nt_split<<<grid, kGemmThreads, 0, s>>>(A, m, B1, n1, B2, n2, K, kchunk, part, status);
-    k_gemm_nt_reduce<<<grid_for((size_t)m * (n1 + n2), 256), 256, 0, s>>>(
-        part, splits, m, n1, n2, B1 == A && n1 == m, scale_div, diag, out1, out2, status);
+    launch_kernel(k_gemm_nt_split, grid, kGemmThreads, 0, s, LaunchHow{}, A, m, B1, n1, B2, n2, K, kchunk, part,
+                  status);
+    launch_kernel(k_gemm_nt_reduce, grid_for((size_t)m * (n1 + n2), 256), 256, 0, s, LaunchHow{}, part, splits, m, n1,
+                  n2, B1 == A && n1 == m, scale_div, diag, out1, out2, status);
 }
 
 __global__ void k_gemm_tn(const double *__restrict__ Y, int ne, int ny, double diag,
                           double *__restrict__ C, const int *status) {
+    launch_wait();
     if (*status) return;
     __shared__ double As[32][17];
     __shared__ double Bs[32][17];
@@ -814,7 +816,7 @@ void launch_gemm_tn_f64(const double *Y, int ne, int ny, double diag, double *C,
                         cudaStream_t s) {
     count_launches(1);
     dim3 grid(ceil_div(ny, 16), ceil_div(ny, 16));
-    k_gemm_tn<<<grid, 256, 0, s>>>(Y, ne, ny, diag, C, status);
+    launch_kernel(k_gemm_tn, grid, 256, 0, s, LaunchHow{}, Y, ne, ny, diag, C, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -862,6 +864,7 @@ __global__ void __launch_bounds__(256) k_cholesky(double *M, double *Lt, int n, 
 
 template <int C>
 __global__ void __launch_bounds__(kSpdThreads) k_spd_factor(double *A, double *At, int n, int *status) {
+    launch_wait();
     spd_factor_body<C>(A, At, n, status);
 }
 
@@ -875,24 +878,13 @@ static void spd_factor_launch(double *A, double *At, int n, int *status, cudaStr
             e = cudaFuncSetAttribute(k_spd_factor<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         return e;
     });
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(kSpdThreads);
-    cfg.dynamicSmemBytes = spd_factor_smem(n, C);
-    cfg.stream = s;
-    cudaLaunchAttribute a[1];
-    a[0].id = cudaLaunchAttributeClusterDimension;
-    a[0].val.clusterDim.x = C;
-    a[0].val.clusterDim.y = 1;
-    a[0].val.clusterDim.z = 1;
-    cfg.attrs = a;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_spd_factor<C>, A, At, n, status);
+    launch_kernel(k_spd_factor<C>, C, kSpdThreads, spd_factor_smem(n, C), s, LaunchHow{C}, A, At, n, status);
 }
 
 __global__ void __launch_bounds__(kSpdThreads) k_spd_apply(const double *__restrict__ A, const double *__restrict__ At,
                                                            int n, const double *rhs, double *out, int ncol,
                                                            __nv_bfloat16 *out16, int ld16, const int *status) {
+    launch_wait();
     spd_apply_body<1>(A, At, n, rhs, out, ncol, out16, ld16, status, blockIdx.x);
 }
 
@@ -970,7 +962,7 @@ void launch_spd_solve(const double *A, const double *At, int n, const double *rh
                       __nv_bfloat16 *out16, int ld16, const int *status, cudaStream_t s) {
     count_launches(1);
     if (n <= kSpdMax)
-        k_spd_apply<<<ncol, kSpdThreads, 0, s>>>(A, At, n, rhs, out, ncol, out16, ld16, status);
+        launch_kernel(k_spd_apply, ncol, kSpdThreads, 0, s, LaunchHow{}, A, At, n, rhs, out, ncol, out16, ld16, status);
     else if (n <= 512)
         k_chol_solve<16><<<ncol, 32, 0, s>>>(A, At, n, rhs, out, ncol, out16, ld16, status);
     else
@@ -995,6 +987,7 @@ __global__ void __launch_bounds__(32 * kUpdateWarps) k_update_f64(T *__restrict_
                                                                   const double *__restrict__ X,
                                                                   const double *__restrict__ Tm, size_t nx, int ne,
                                                                   const int *status) {
+    launch_wait();
     extern __shared__ double2 Ts2[];  // [Q columns][ne rounded up to 8]
     if (*status) return;
     double *Ts = reinterpret_cast<double *>(Ts2);
@@ -1062,7 +1055,8 @@ static void update_launch(int cols, T *members, T *dC, const double *X, const do
         if (cols < Q) return update_launch<T, Q - 1>(cols, members, dC, X, Tm, nx, ne, status, s);
     const dim3 grid(ceil_div(nx, 32 * kUpdateWarps), ceil_div(ne + 1, Q));
     const size_t smem = sizeof(double) * Q * (size_t)((ne + 7) & ~7);  // <= 32 KB for ne <= 512
-    k_update_f64<T, Q><<<grid, 32 * kUpdateWarps, smem, s>>>(members, dC, X, Tm, nx, ne, status);
+    launch_kernel(k_update_f64<T, Q>, grid, 32 * kUpdateWarps, smem, s,
+                  LaunchHow{1, 1, 1, grid.x * grid.y <= 2u * kNumSMs}, members, dC, X, Tm, nx, ne, status);
 }
 
 template <typename T>
@@ -1206,6 +1200,7 @@ __device__ __forceinline__ void prolong_stage_weights(const ProlongWeights &w, i
 template <typename T>
 __global__ void k_prolong_add(T *__restrict__ fine, const T *__restrict__ dC, int dim, int V, int nc,
                               int r, ProlongWeights w, const int *status) {
+    launch_wait();
     if (*status) return;
     const int nf = nc * r;
     if (dim == 1) {
@@ -1235,10 +1230,11 @@ void launch_prolong_add(T *fine, const T *dC, int dim, int V, int nc, int r,
     count_launches(1);
     const int nf = nc * r;
     if (dim == 1) {
-        k_prolong_add<T><<<grid_for((size_t)V * nf, 256), 256, 0, s>>>(fine, dC, dim, V, nc, r, w, status);
+        launch_kernel(k_prolong_add<T>, grid_for((size_t)V * nf, 256), 256, 0, s, LaunchHow{}, fine, dC, dim, V, nc,
+                      r, w, status);
     } else {
         const dim3 grid(ceil_div(nf, 128), std::min(V * nc, 65535));
-        k_prolong_add<T><<<grid, 128, 0, s>>>(fine, dC, dim, V, nc, r, w, status);
+        launch_kernel(k_prolong_add<T>, grid, 128, 0, s, LaunchHow{}, fine, dC, dim, V, nc, r, w, status);
     }
 }
 
@@ -1310,6 +1306,7 @@ void launch_rmse(const T *x, const double *truth, int V, size_t npts, double *pa
 // ---------------------------------------------------------------------------
 template <typename Tin, typename Tout>
 __global__ void k_convert(const Tin *__restrict__ in, Tout *__restrict__ out, size_t n) {
+    launch_wait();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
          i += (size_t)gridDim.x * blockDim.x)
         out[i] = (Tout)in[i];
@@ -1319,20 +1316,24 @@ template <typename Tin, typename Tout>
 void launch_convert(const Tin *in, Tout *out, size_t n, cudaStream_t s) {
     if (n == 0) return;
     count_launches(1);
-    k_convert<Tin, Tout><<<grid_for(n, 256), 256, 0, s>>>(in, out, n);
+    launch_kernel(k_convert<Tin, Tout>, grid_for(n, 256), 256, 0, s, LaunchHow{}, in, out, n);
 }
 
 // the analysis counter that keys the perturbation stream lives on the device,
 // so a captured cycle advances it on every replay
-__global__ void k_bump_counter(uint64_t *c) { *c += 1; }
+__global__ void k_bump_counter(uint64_t *c) {
+    launch_wait();
+    *c += 1;
+}
 
 void launch_bump_counter(uint64_t *c, cudaStream_t s) {
     count_launches(1);
-    k_bump_counter<<<1, 1, 0, s>>>(c);
+    launch_kernel(k_bump_counter, 1, 1, 0, s, LaunchHow{}, c);
 }
 
 __global__ void k_tt_bf16(const double *__restrict__ Tm, __nv_bfloat16 *__restrict__ Tt, int ne,
                           int ld, const int *status) {
+    launch_wait();
     if (*status) return;
     const int total = (ne + 1) * ne;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
@@ -1344,12 +1345,13 @@ __global__ void k_tt_bf16(const double *__restrict__ Tm, __nv_bfloat16 *__restri
 void launch_tt_bf16(const double *Tm, __nv_bfloat16 *Tt, int ne, int ld, const int *status,
                     cudaStream_t s) {
     count_launches(1);
-    k_tt_bf16<<<grid_for((size_t)(ne + 1) * ne, 256), 256, 0, s>>>(Tm, Tt, ne, ld, status);
+    launch_kernel(k_tt_bf16, grid_for((size_t)(ne + 1) * ne, 256), 256, 0, s, LaunchHow{}, Tm, Tt, ne, ld, status);
 }
 
 // one thread per Philox block (4 normals)
 __global__ void k_normals(uint64_t seed, uint64_t tag, uint64_t ctr0, int64_t count,
                           double *__restrict__ out) {
+    launch_wait();
     const int64_t nblk = (count + 3) / 4;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblk; b += (int64_t)gridDim.x * blockDim.x) {
         double z[4];
@@ -1364,7 +1366,8 @@ void launch_normals(uint64_t seed, uint64_t tag, uint64_t ctr0, int64_t count, d
                     cudaStream_t s) {
     if (count <= 0) return;
     count_launches(1);
-    k_normals<<<grid_for((size_t)((count + 3) / 4), 256), 256, 0, s>>>(seed, tag, ctr0, count, out);
+    launch_kernel(k_normals, grid_for((size_t)((count + 3) / 4), 256), 256, 0, s, LaunchHow{}, seed, tag, ctr0, count,
+                  out);
 }
 
 // ---------------------------------------------------------------------------

@@ -94,6 +94,7 @@ struct GradParts {
     int units, loss_parts;
 };
 __global__ void __launch_bounds__(128) k_reduce_grads(GradParts P, float *__restrict__ g, const int *status) {
+    launch_wait();
     if (*status) return;
     __shared__ float red[128];
     const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
@@ -135,6 +136,7 @@ __global__ void __launch_bounds__(128) k_reduce_grads(GradParts P, float *__rest
 __global__ void k_adam(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v,
                        const float *__restrict__ g, __nv_bfloat16 *__restrict__ fwd, __nv_bfloat16 *__restrict__ adj,
                        float lr, float b1, float b2, float eps, float c1, float c2) {
+    launch_wait();
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kCnnParams; e += gridDim.x * blockDim.x) {
         const float gi = g[e];
         const float mi = b1 * m[e] + (1.f - b1) * gi;
@@ -376,7 +378,7 @@ extern "C" mgenkf_status mgk_cnn_loss_grad(mgk_cnn_t c, const float *dC, const f
     launch_conv_wgrad<1, 32>(c->a0, c->d1, s2, n, B, part[0], c->status, s);
     const GradParts P{{part[0], part[1], part[2]}, c->loss_part, c->loss, units, conv_loss_parts(n, B)};
     count_launches(1);
-    k_reduce_grads<<<kCnnParams / 32 + 1, 128, 0, s>>>(P, c->g, c->status);
+    launch_kernel(k_reduce_grads, kCnnParams / 32 + 1, 128, 0, s, LaunchHow{}, P, c->g, c->status);
     if (loss_out) {
         if (cudaMemcpyAsync(loss_out, c->loss, sizeof(float), cudaMemcpyDefault, s) != cudaSuccess)
             return MGENKF_ERR_CUDA;
@@ -390,6 +392,7 @@ extern "C" mgenkf_status mgk_cnn_adam_step(mgk_cnn_t c, float lr, void *stream) 
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - powf(b1, (float)c->step), c2 = 1.f - powf(b2, (float)c->step);
     count_launches(1);
-    k_adam<<<118, 256, 0, (cudaStream_t)stream>>>(c->w, c->m, c->v, c->g, c->fwd, c->adj, lr, b1, b2, 1e-8f, c1, c2);
+    launch_kernel(k_adam, 118, 256, 0, (cudaStream_t)stream, LaunchHow{},
+                  c->w, c->m, c->v, c->g, c->fwd, c->adj, lr, b1, b2, 1e-8f, c1, c2);
     return cudaGetLastError() == cudaSuccess ? MGENKF_OK : MGENKF_ERR_CUDA;
 }

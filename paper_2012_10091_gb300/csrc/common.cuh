@@ -1,6 +1,7 @@
 // common.cuh -- shared device/host helpers of the MGEnKF GPU library.
 #pragma once
 
+#include <utility>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -59,6 +60,49 @@ __host__ __device__ inline int ceil_div(long long a, long long b) { return (int)
 inline size_t residency_smem(size_t need, int ctas) {
     const size_t limit = ctas >= 1 && ctas <= 3 ? (size_t)228 * 1024 / (ctas + 1) - 512 : 0;
     return need > limit ? need : limit;
+}
+
+// Launches that follow one another on a stream with programmatic serialisation
+// ("chained"): the CTAs of the next launch are placed, and its launch latency
+// passes, while the previous one runs.  Every kernel launched so starts with
+// launch_wait(): from there on the launches before it have completed and their
+// writes are visible, and the next one may be placed.  For the chains of small
+// kernels of an analysis (the smallest cycle, 14 launches: 122 us, 98 us chained; three
+// layers of the learned correction 26.6 and 20.4 us).
+// A launch bound by the FP64 pipes with about as many CTAs as SMs or more is
+// better placed on an empty GPU: chained, its CTAs take the SMs that have room
+// while the previous kernel runs, two where others get none (4096 points, 128
+// members: anomalies 17 us slower, the update 55).
+struct LaunchHow {
+    unsigned x = 1, y = 1, z = 1;  // cluster
+    bool chained = true;
+};
+__device__ __forceinline__ void launch_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... Args>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                 const LaunchHow &how, Args &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    cfg.numAttrs = 0;
+    if (how.chained) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (how.x * how.y * how.z > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = how.x;
+        attr[cfg.numAttrs].val.clusterDim.y = how.y;
+        attr[cfg.numAttrs++].val.clusterDim.z = how.z;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 // device status word values (a subset of mgenkf_status)

@@ -49,8 +49,8 @@
 // against 9e-7 now and 8e-7 on the FP32 pipes.
 //
 // Measured, 8 samples of 256^2 coarse points: the loss and all gradients 5.4 ms
-// with the backward pass on the CUDA cores, 0.60 ms here; inference of one
-// sample 80 us, 27 us here.
+// with the backward pass on the CUDA cores, 0.58 ms here; inference of one
+// sample 80 us, 20 us here.
 //
 // Rows and pixels past the map's edge are computed from wrapped inputs (zeros
 // in the gradients) and not stored.  Every mbarrier wait is bounded; on expiry
@@ -166,6 +166,7 @@ struct ConvShape {
 template <int CG, int NSPLIT, int COUT, int EPI, int ROWS>
 __global__ void __launch_bounds__(kConvThreads, EPI == kLoss ? 3 : 2) k_conv_tc(ConvArgs A) {
     using S = ConvShape<CG, NSPLIT, COUT, ROWS>;
+    launch_wait();
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -457,8 +458,7 @@ static cudaError_t conv_launch(const ConvArgs &A, int batch, cudaStream_t s) {
     });
     count_launches(1);
     const dim3 grid(ceil_div(A.n, kPix), ceil_div(A.n, ROWS), batch);
-    k_conv_tc<CG, NSPLIT, COUT, EPI, ROWS><<<grid, kConvThreads, S::SMEM, s>>>(A);
-    return cudaPeekAtLastError();
+    return launch_kernel(k_conv_tc<CG, NSPLIT, COUT, EPI, ROWS>, grid, kConvThreads, S::SMEM, s, LaunchHow{}, A);
 }
 
 // Four output rows per CTA read 1.5 input rows per output row, two read 2, but
@@ -523,6 +523,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_wgrad(const __nv_bfloa
                                                                 int *status) {
     using S = WgradShape<CGI, COUT>;
     constexpr int CIN = 8 * CGI;
+    launch_wait();
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sa = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -733,9 +734,8 @@ cudaError_t launch_conv_wgrad(const __nv_bfloat16 *in, const __nv_bfloat16 *d, s
         return cudaFuncSetAttribute(k_conv_wgrad<CGI, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
     });
     count_launches(1);
-    k_conv_wgrad<CGI, COUT><<<wgrad_units(n, batch), kConvThreads, S::SMEM, s>>>(in, d, d_split, n,
-                                                                               wgrad_rows(n, batch), part, status);
-    return cudaPeekAtLastError();
+    return launch_kernel(k_conv_wgrad<CGI, COUT>, wgrad_units(n, batch), kConvThreads, S::SMEM, s, LaunchHow{}, in, d,
+                         d_split, n, wgrad_rows(n, batch), part, status);
 }
 
 int conv_packed_elems(int cin, int cout) { return 9 * (cin < 16 ? 2 : cin / 8) * cout * 8; }

@@ -66,6 +66,7 @@ template <bool CLUSTER>
 __global__ void __launch_bounds__(1024) k_burgers_inlet(double *__restrict__ u, int n, int ctas, int per, double a,
                                                         double c, double dt, int nsteps, double t0,
                                                         const double *__restrict__ theta, double u0, double omega) {
+    launch_wait();
     extern __shared__ double sh[];
     __shared__ double inlet[2 * kInletSteps];
     const int pitch = per + 6;
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(1024) k_burgers_inlet(double *__restrict__ u, 
 // theta^f = theta^a + sqrt(q) tau
 __global__ void k_theta_walk(const double *__restrict__ theta, const double *__restrict__ tau, double sq, int count,
                              double *__restrict__ theta_f) {
+    launch_wait();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < count) theta_f[e] = theta[e] + sq * tau[e];
 }
@@ -170,6 +172,7 @@ __global__ void __cluster_dims__(kThetaCtas, 1, 1) __launch_bounds__(32 * kTheta
     k_theta_update(const double *__restrict__ theta_f, const double *__restrict__ Tm, int ne,
                    double inv_ne, double isq, double *__restrict__ theta_a, double *__restrict__ theta_mean,
                    const int *status) {
+    launch_wait();
     __shared__ double part[kThetaCtas][2], mine[kThetaWarps][2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = blockIdx.x;
     const bool ok = *status == 0;
@@ -221,6 +224,7 @@ __global__ void __cluster_dims__(kThetaCtas, 1, 1) __launch_bounds__(32 * kTheta
 // fine += Pi_F(dC) on the open grid: 4 taps from j0[k]
 __global__ void k_prolong_open(double *__restrict__ fine, const double *__restrict__ dC, int nf,
                                const int32_t *__restrict__ j0, const double *__restrict__ w, const int *status) {
+    launch_wait();
     if (*status) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nf) return;
@@ -298,23 +302,12 @@ void forecast(mgenkf_dual *d, double *grids, int nprob, int n, const double *the
     const int ctas = inlet_ctas(nprob, n), per = ceil_div(n, ctas);
     const double dx = d->cfg.length / n, dt = d->cfg.dt;
     const double a = dt / (4.0 * dx), c = 4.0 * d->cfg.nu / dx;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nprob * ctas);
-    cfg.blockDim = dim3(std::max(64, ceil_div(per + 6, 32) * 32));  // 64 threads form the inlet values
-    cfg.dynamicSmemBytes = 4 * (per + 6) * sizeof(double);
-    cfg.stream = s ? s : d->stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (ctas > 1)
-        cudaLaunchKernelEx(&cfg, k_burgers_inlet<true>, grids, n, ctas, per, a, c, dt, nsteps, d->t, theta, d->cfg.u0,
-                           d->cfg.omega);
-    else
-        cudaLaunchKernelEx(&cfg, k_burgers_inlet<false>, grids, n, ctas, per, a, c, dt, nsteps, d->t, theta,
-                           d->cfg.u0, d->cfg.omega);
+    // 64 threads form the inlet values
+    const int threads = std::max(64, ceil_div(per + 6, 32) * 32);
+    const size_t smem = 4 * (per + 6) * sizeof(double);
+    launch_kernel(ctas > 1 ? k_burgers_inlet<true> : k_burgers_inlet<false>, nprob * ctas, threads, smem,
+                  s ? s : d->stream, LaunchHow{(unsigned)ctas}, grids, n, ctas, per, a, c, dt, nsteps, d->t, theta,
+                  d->cfg.u0, d->cfg.omega);
 }
 
 // perturbations (generated once per cycle), anomalies and T = S^-1 B (ensemble space)
@@ -479,15 +472,15 @@ extern "C" mgenkf_status mgenkf_dual_cycle(mgenkf_dual_t d, int32_t nsteps, cons
     D_CUDA(cudaMemcpyAsync(d->prev, d->members, (size_t)ne * nc * 8, cudaMemcpyDeviceToDevice, s));
     launch_normals(d->cfg.seed, kThetaTag, d->cycle, 2 * (int64_t)ne, d->tau, s);
     count_launches(1);
-    k_theta_walk<<<ceil_div(2 * ne, 256), 256, 0, s>>>(d->theta, d->tau, std::sqrt(d->cfg.theta_q), 2 * ne,
-                                                        d->theta_f);
+    launch_kernel(k_theta_walk, ceil_div(2 * ne, 256), 256, 0, s, LaunchHow{},
+                  d->theta, d->tau, std::sqrt(d->cfg.theta_q), 2 * ne, d->theta_f);
     forecast(d, d->members, ne, nc, d->theta_f, nsteps);
     // steps 3-5: perturbed observations, parameter update theta^a = theta^f + Theta T
     gain_solve(d, 1, d->xstar_a);
     D_CUDA(cudaStreamWaitEvent(s, d->ev[1], 0));  // join: the fine forecast has read theta_mean
     count_launches(1);
-    k_theta_update<<<kThetaCtas, 32 * kThetaWarps, 0, s>>>(
-        d->theta_f, d->Bt, ne, 1.0 / ne, 1.0 / std::sqrt(ne - 1.0), d->theta, d->theta_mean, d->status);
+    launch_kernel(k_theta_update, kThetaCtas, 32 * kThetaWarps, 0, s, LaunchHow{},
+                  d->theta_f, d->Bt, ne, 1.0 / ne, 1.0 / std::sqrt(ne - 1.0), d->theta, d->theta_mean, d->status);
     // steps 6-8: members forecast again from the previous analysis with theta^a, state update
     D_CUDA(cudaMemcpyAsync(d->members, d->prev, (size_t)ne * nc * 8, cudaMemcpyDeviceToDevice, s));
     forecast(d, d->members, ne, nc, d->theta, nsteps);
@@ -497,7 +490,8 @@ extern "C" mgenkf_status mgenkf_dual_cycle(mgenkf_dual_t d, int32_t nsteps, cons
     launch_update_f64<double>(d->members, d->dC, d->X, d->Bt, nc, ne, d->status, s);
     // Algorithm 4 step 5: x^F += Pi_F(x^C' - x^C*)
     count_launches(1);
-    k_prolong_open<<<ceil_div(d->nf, 256), 256, 0, s>>>(d->fine, d->dC, d->nf, d->pro_j0, d->pro_w, d->status);
+    launch_kernel(k_prolong_open, ceil_div(d->nf, 256), 256, 0, s, LaunchHow{}, d->fine, d->dC, d->nf, d->pro_j0,
+                  d->pro_w, d->status);
     launch_bump_counter(d->cycle_d, s);
     D_CUDA(cudaGetLastError());
     d->t += nsteps * d->cfg.dt;

@@ -79,6 +79,7 @@ struct UpdateLaunchArgs {
 // the copies in flight awaited (default bound), TMEM freed.
 __global__ void __launch_bounds__(kUpdateThreads) k_update_tc(const __grid_constant__ UpdateLaunchArgs a,
                                                    const int2 *__restrict__ map, int nent) {
+    launch_wait();
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte aligned operand buffers
     unsigned char *base = reinterpret_cast<unsigned char *>(
@@ -448,7 +449,7 @@ static cudaError_t update_launch(UpdateLaunchArgs &args, int nprob, const int2 *
     const int per_sm = std::max(1, std::min(8, (int)((size_t)228 * 1024 / (smem + stat + 1024))));
     const int grid = std::min(nent, std::max(1, sms) * per_sm);
     count_launches(1);
-    k_update_tc<<<grid, kUpdateThreads, smem, s>>>(args, map, nent);
+    launch_kernel(k_update_tc, grid, kUpdateThreads, smem, s, LaunchHow{}, args, map, nent);
     return cudaGetLastError();
 }
 
