@@ -243,10 +243,11 @@ void launch_innov_rms(const double *Z, int ne, int ny, double *out, cudaStream_t
 }
 
 // perturbed observations (Eq. perturbed_y) and normalised anomalies Y (Algorithm 3 step 7)
-// One thread per Philox block: the 4 consecutive elements o = 4b .. 4b + 3 of
-// the Ne x Ny perturbation matrix (flat index o = i Ny + j).  gen_eps: 0 = eps
-// given, 1 = normals in FP64, 2 = Box-Muller in FP32 (the mixed path).
-template <bool F32>
+// One thread per Philox block, the 4 consecutive elements o = 4b .. 4b + 3 of
+// the Ne x Ny perturbation matrix (flat index o = i Ny + j), or (L = 1, CTAs of
+// 128 threads) a warp per element of 32 blocks.  gen_eps: 0 = eps given, 1 =
+// normals in FP64, 2 = Box-Muller in FP32 (the mixed path).
+template <bool F32, int L = 4>
 __device__ __forceinline__ void obs_perturb_body(const double *__restrict__ yf, const double *__restrict__ ybar,
                                                  const double *__restrict__ yo, double *__restrict__ eps,
                                                  int gen_eps, uint64_t seed, const uint64_t *__restrict__ cycle,
@@ -255,19 +256,22 @@ __device__ __forceinline__ void obs_perturb_body(const double *__restrict__ yf, 
                                                  float *__restrict__ Yl = nullptr, float *__restrict__ Zh = nullptr,
                                                  float *__restrict__ Zl = nullptr) {
     const size_t total = (size_t)ne * ny;
-    const size_t b = blk * blockDim.x + threadIdx.x;
-    if (4 * b >= total) return;
-    double z[4];
+    const size_t b = L == 1 ? blk * 32 + (threadIdx.x & 31) : blk * blockDim.x + threadIdx.x;
+    const size_t o0 = L == 1 ? 4 * b + (threadIdx.x >> 5) : 4 * b;
+    if (o0 >= total) return;
+    double z[L];
     if (gen_eps) {
-        if (F32)
+        if constexpr (L == 1)
+            z[0] = philox_normal1(seed, kEpsTag, *cycle, (uint64_t)b, threadIdx.x >> 5);
+        else if constexpr (F32)
             philox_normals4_f32(seed, kEpsTag, *cycle, (uint64_t)b, z);
         else
             philox_normals4(seed, kEpsTag, *cycle, (uint64_t)b, z);
     }
-    int i = (int)((4 * b) / ny), j = (int)(4 * b - (size_t)i * ny);
+    int i = (int)(o0 / ny), j = (int)(o0 - (size_t)i * ny);
 #pragma unroll
-    for (int l = 0; l < 4; ++l) {
-        const size_t o = 4 * b + l;
+    for (int l = 0; l < L; ++l) {
+        const size_t o = o0 + l;
         if (o < total) {
             // explicit roundings: no contraction into an FMA, whatever the
             // kernel the body is inlined into
@@ -294,15 +298,15 @@ __device__ __forceinline__ void obs_perturb_body(const double *__restrict__ yf, 
     }
 }
 
-template <bool F32>
-__global__ void k_obs_perturb(const double *__restrict__ yf, const double *__restrict__ ybar,
+template <bool F32, int L>
+__global__ void __launch_bounds__(128) k_obs_perturb(const double *__restrict__ yf, const double *__restrict__ ybar,
                               const double *__restrict__ yo, double *__restrict__ eps, int gen_eps, uint64_t seed,
                               const uint64_t *__restrict__ cycle, double sigma, int ne, int ny, double isq,
                               double *__restrict__ Y, double *__restrict__ Z, float *__restrict__ Yh,
                               float *__restrict__ Yl, float *__restrict__ Zh, float *__restrict__ Zl) {
     launch_wait();
-    obs_perturb_body<F32>(yf, ybar, yo, eps, gen_eps, seed, cycle, sigma, ne, ny, isq, Y, Z, blockIdx.x, Yh, Yl, Zh,
-                          Zl);
+    obs_perturb_body<F32, L>(yf, ybar, yo, eps, gen_eps, seed, cycle, sigma, ne, ny, isq, Y, Z, blockIdx.x, Yh, Yl,
+                             Zh, Zl);
 }
 
 void launch_obs_perturb(const double *yf, const double *ybar, const double *yo, double *eps,
@@ -314,10 +318,13 @@ void launch_obs_perturb(const double *yf, const double *ybar, const double *yo, 
     const unsigned grid = (unsigned)ceil_div(blocks, 128);
     const double isq = 1.0 / std::sqrt((double)(ne - 1));
     if (gen_eps == 2)
-        launch_kernel(k_obs_perturb<true>, grid, 128, 0, s, LaunchHow{}, yf, ybar, yo, eps, 1, seed, cycle, sigma, ne,
+        launch_kernel(k_obs_perturb<true, 4>, grid, 128, 0, s, LaunchHow{}, yf, ybar, yo, eps, 1, seed, cycle, sigma, ne,
                       ny, isq, Y, Z, df.Yh, df.Yl, df.Zh, df.Zl);
+    else if (gen_eps && single_normals(blocks))
+        launch_kernel(k_obs_perturb<false, 1>, ceil_div(blocks, 32), 128, 0, s, LaunchHow{}, yf, ybar, yo, eps,
+                      gen_eps, seed, cycle, sigma, ne, ny, isq, Y, Z, df.Yh, df.Yl, df.Zh, df.Zl);
     else
-        launch_kernel(k_obs_perturb<false>, grid, 128, 0, s, LaunchHow{}, yf, ybar, yo, eps, gen_eps, seed, cycle,
+        launch_kernel(k_obs_perturb<false, 4>, grid, 128, 0, s, LaunchHow{}, yf, ybar, yo, eps, gen_eps, seed, cycle,
                       sigma, ne, ny, isq, Y, Z, df.Yh, df.Yl, df.Zh, df.Zl);
 }
 
@@ -1362,10 +1369,23 @@ __global__ void k_normals(uint64_t seed, uint64_t tag, uint64_t ctr0, int64_t co
     }
 }
 
+// the same with a warp per element of 32 Philox blocks (CTAs of 128 threads)
+__global__ void __launch_bounds__(128) k_normals1(uint64_t seed, uint64_t tag, uint64_t ctr0, int64_t count,
+                                                  double *__restrict__ out) {
+    launch_wait();
+    const int64_t b = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31), o = 4 * b + (threadIdx.x >> 5);
+    if (o < count) out[o] = philox_normal1(seed, tag, ctr0, (uint64_t)b, threadIdx.x >> 5);
+}
+
 void launch_normals(uint64_t seed, uint64_t tag, uint64_t ctr0, int64_t count, double *out,
                     cudaStream_t s) {
     if (count <= 0) return;
     count_launches(1);
+    const size_t blocks = (size_t)(count + 3) / 4;
+    if (single_normals(blocks)) {
+        launch_kernel(k_normals1, ceil_div(blocks, 32), 128, 0, s, LaunchHow{}, seed, tag, ctr0, count, out);
+        return;
+    }
     launch_kernel(k_normals, grid_for((size_t)((count + 3) / 4), 256), 256, 0, s, LaunchHow{}, seed, tag, ctr0, count,
                   out);
 }

@@ -157,6 +157,25 @@ __device__ __forceinline__ void philox_normals4(uint64_t seed, uint64_t tag, uin
     }
 }
 
+// one of those four, l (where a warp has one l, it runs one trigonometric function)
+__device__ __forceinline__ double philox_normal1(uint64_t seed, uint64_t tag, uint64_t ctr0, uint64_t blk, int l) {
+    const U64x4 x = philox4x64_10(ctr0, blk, 0, 0, seed, tag);
+    const double inv53 = 1.0 / 9007199254740992.0;
+    const uint64_t a = l < 2 ? x.v[0] : x.v[2], b = l < 2 ? x.v[1] : x.v[3];
+    const double u1 = (double)((a >> 11) + 1) * inv53;
+    const double u2 = (double)((b >> 11) + 1) * inv53;
+    const double rad = sqrt(-2.0 * log(u1));
+    const double th = 6.283185307179586 * u2;
+    return l & 1 ? rad * sin(th) : rad * cos(th);
+}
+
+// Normals per thread: the four of a Philox block, or one each on the four warps of
+// a CTA of 128 threads while that gives at most two CTAs per SM (`blocks` Philox
+// blocks).  A normal is a chain of some 100 FP64 instructions of 64 cycles and
+// four share part of it: 512 normals 11 us by fours, 7 us one each; 65536 take
+// 11 us by fours and would take more one each.
+inline bool single_normals(size_t blocks) { return blocks <= (size_t)2 * kNumSMs * 32; }
+
 // The same four normals with the Box-Muller transform evaluated in FP32 on
 // the same Philox words (each uniform rounded to FP32 first): within about
 // 1e-6 of the FP64 values, without GB300's slow FP64 logarithm and sines.

@@ -802,24 +802,14 @@ static SegPlan seg_plan(int n0, int np0, int n1, int np1, int nsteps, int sms) {
 }
 
 template <int Q>
-static cudaError_t seg_launch(const SegArgs &A, int ctas, int threads, int per_sm, bool follows,
-                              cudaStream_t stream) {
+static cudaError_t seg_launch(const SegArgs &A, int ctas, int threads, int per_sm, cudaStream_t stream) {
     static OncePerDevice once;
     once.run([](int) {
         return cudaFuncSetAttribute(burgers_seg64<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024);
     });
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = residency_smem(sizeof(double) * 4 * threads, per_sm);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = follows ? 1 : 0;  // after the first launch: start while the previous one ends
     count_launches(1);
-    return cudaLaunchKernelEx(&cfg, burgers_seg64<Q>, A);
+    return launch_kernel(burgers_seg64<Q>, ctas, threads, residency_smem(sizeof(double) * 4 * threads, per_sm), stream,
+                         LaunchHow{}, A);
 }
 
 static int device_sms() {
@@ -881,10 +871,10 @@ cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, do
         }
         cudaError_t e;
         switch (pl.Q) {
-            case 1: e = seg_launch<1>(A, ctas, threads, per_sm, l > 0, stream); break;
-            case 2: e = seg_launch<2>(A, ctas, threads, per_sm, l > 0, stream); break;
-            case 4: e = seg_launch<4>(A, ctas, threads, per_sm, l > 0, stream); break;
-            default: e = seg_launch<8>(A, ctas, threads, per_sm, l > 0, stream); break;
+            case 1: e = seg_launch<1>(A, ctas, threads, per_sm, stream); break;
+            case 2: e = seg_launch<2>(A, ctas, threads, per_sm, stream); break;
+            case 4: e = seg_launch<4>(A, ctas, threads, per_sm, stream); break;
+            default: e = seg_launch<8>(A, ctas, threads, per_sm, stream); break;
         }
         if (e != cudaSuccess) return e;
     }

@@ -1268,23 +1268,14 @@ static long long n64_ctas(int n, int grids, int rows) {
 }
 
 template <int STAGE>
-static cudaError_t n64_launch(const Ns64Args &A, long long ctas, int per_sm, bool follows, cudaStream_t s) {
+static cudaError_t n64_launch(const Ns64Args &A, long long ctas, int per_sm, cudaStream_t s) {
     static OncePerDevice once;
     once.run([](int) {
         return cudaFuncSetAttribute(ns2d_march64<STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024);
     });
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ctas);
-    cfg.blockDim = dim3(kN64Threads);
-    cfg.dynamicSmemBytes = residency_smem(sizeof(double) * n64_smem_doubles(A.rows), per_sm);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = follows ? 1 : 0;
     count_launches(1);
-    return cudaLaunchKernelEx(&cfg, ns2d_march64<STAGE>, A);
+    return launch_kernel(ns2d_march64<STAGE>, (unsigned)ctas, kN64Threads,
+                         residency_smem(sizeof(double) * n64_smem_doubles(A.rows), per_sm), s, LaunchHow{}, A);
 }
 
 static cudaError_t n64_forecast(const NsGroup<double> (&g)[2], double gm1, double mu, double kappa, int nsteps,
@@ -1336,9 +1327,9 @@ static cudaError_t n64_forecast(const NsGroup<double> (&g)[2], double gm1, doubl
     if (total > INT32_MAX) return cudaErrorInvalidConfiguration;
     cudaError_t e = cudaSuccess;
     for (int st = 0; st < nsteps && e == cudaSuccess; ++st) {
-        e = n64_launch<0>(A, total, per_sm, st > 0, s);
-        if (e == cudaSuccess) e = n64_launch<1>(A, total, per_sm, true, s);
-        if (e == cudaSuccess) e = n64_launch<2>(A, total, per_sm, true, s);
+        e = n64_launch<0>(A, total, per_sm, s);
+        if (e == cudaSuccess) e = n64_launch<1>(A, total, per_sm, s);
+        if (e == cudaSuccess) e = n64_launch<2>(A, total, per_sm, s);
     }
     return e;
 }
