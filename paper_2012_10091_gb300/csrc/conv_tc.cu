@@ -252,6 +252,18 @@ __global__ void __launch_bounds__(kConvThreads, EPI == kLoss ? 3 : 2) k_conv_tc(
         cp_async_commit();
     }
     const int rows = min(ROWS, n - y0);
+    if (EPI == kLoss) {
+        // the target values of this thread's pixel on their way to L2 while the
+        // tensor cores work (a line holds eight lanes' 16 bytes)
+        const int x = x0 + (warp & 3) * 32 + lane, nf = 4 * n;
+        for (int r = warp >> 2; r < rows; r += 2)
+            if (x < n && (lane & 7) == 0)
+                for (int q = 0; q < 16; ++q) {
+                    const float *t = A.target + (((size_t)b * 4 + (q >> 2)) * nf + 4 * (y0 + r) + (q & 3)) * (size_t)nf +
+                                     4 * (size_t)x;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(t));
+                }
+    }
     const uint32_t a0 = tc::smem_u32(sin), b0 = tc::smem_u32(sw);
     uint32_t tmem = 0;
     bool ok = true;
