@@ -64,21 +64,21 @@ WORKLOADS = {
     # The handle's forecast is the column march (autotuned layout), the members
     # and the fine run on two streams: one launch each per model step, side by
     # side; the roofline takes the whole forecast as one unit.
-    "ns2d": dict(flops=423, bytes=32, kernel="ns2d_rk3_march<TableUnits> members + fine run",
+    "ns2d": dict(flops=423, bytes=32, kernel="ns2d_rk3_march members + fine run",
                  launches_per_step=None, traffic=None, truth="fp64"),
     # NS-2D 1024^2 / 256^2 with the learned correction of the prolongation
-    "ns2d_cnn": dict(flops=423, bytes=32, kernel="ns2d_rk3_march<TableUnits> members + fine run",
+    "ns2d_cnn": dict(flops=423, bytes=32, kernel="ns2d_rk3_march members + fine run",
                      launches_per_step=None, traffic=None, truth="fp64"),
-    # Dual EnKF parameter estimation on the Burgers inlet model (latency-bound: small grids)
+    # Dual EnKF parameter estimation on the Burgers inlet model (FP64, small grids)
     "dual": dict(kernel="k_burgers_inlet"),
     # 96 independent NS-2D problems: one march launch per model step and grid
     # size.  traffic_per_point_step: dram__bytes_read.sum + dram__bytes_write.sum
     # per point-step of the march launches of one cycle, measured by ncu on the
-    # 8-problem batch (16.71 B read, 4.45 B written: ncu counts the lines L2
+    # 8-problem batch (16.72 B read, 4.72 B written: ncu counts the lines L2
     # evicts during a launch; two-part cycle, autotuned choices), scaled to this
     # batch by its point-steps; None once the kernel changes.
-    "batched": dict(flops=423, bytes=32, kernel="ns2d_rk3_march<TableUnits>", launches_per_step=None,
-                    traffic_per_point_step=21.15, truth="fp32"),
+    "batched": dict(flops=423, bytes=32, kernel="ns2d_rk3_march", launches_per_step=None,
+                    traffic_per_point_step=21.44, truth="fp32"),
 }
 CNN_FLOPS_PER_PIXEL = 2 * 9 * (8 * 32 + 32 * 32 + 32 * 64)  # three 3x3 convolutions per coarse pixel
 

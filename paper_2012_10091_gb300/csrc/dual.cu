@@ -53,8 +53,8 @@ constexpr int kDualMaxPts = 1024;               // points per grid
 // add up, 1e-13).
 // The inlet values of 32 steps are formed together by 64 threads (a sine takes
 // some 50 dependent FP64 instructions); the outlet is extrapolated by the one
-// thread that reads it.  30 steps: 100 grids of 200 nodes 176 -> 51 us, one of
-// 800 (a cluster of 8, where one SM did all of it) 441 -> 43 us.
+// thread that reads it.  30 steps: 100 grids of 200 nodes 176 -> 60 us, one of
+// 800 (a cluster of 8, where one SM did all of it) 441 -> 48 us.
 constexpr int kInletSteps = 32;  // steps of inlet values formed together
 __device__ __forceinline__ void inlet_push(double *local, int rank, double v) {
     uint32_t a = (uint32_t)__cvta_generic_to_shared(local), r;

@@ -611,10 +611,11 @@ static cudaError_t launch_burgers(BurgersArgs<T> A, cudaStream_t stream) {
 // (measured with dependent chains; 76 cycles with all four sub-partitions
 // busy), so a model step costs the FP64 instructions of the busiest
 // sub-partition and nothing else matters much.  One point per thread and 128
-// points per CTA put one warp on each sub-partition: 26 instructions, about
-// 1 us, per step.  Measured, one 16384-point grid, 4331 steps: 157 ms on one
-// cluster of four CTAs of 4096 points (36 us per step), 6.7 ms in segments
-// (1.56 us per step, 149 CTAs of 128 points with their halo, 3 steps a launch).
+// points per CTA put one warp on each sub-partition: 20 instructions, 0.7 us,
+// per step.  Measured, one 16384-point grid, 4331 steps: 157 ms on one
+// cluster of four CTAs of 4096 points (36 us per step), 5.84 ms in segments
+// (1.35 us per step, 149 CTAs of 128 points with their halo, 3 steps a launch;
+// 6.74 ms with 26 instructions).
 //
 // A CTA advances the points of its segment and H = 3 steps of halo on both
 // sides by a few steps with one barrier per RK stage; the halo's outermost
@@ -749,7 +750,7 @@ static SegShape seg_shape(int n, int W, int m, int Q) {
 // warp (20 per point and step) at 19 cycles per
 // warp, at least 64 each, and 100 cycles per stage for the barrier and the
 // exchange; CTAs on one SM add up; a launch costs
-// kSegLaunch (16384 points, 110-point segments, m = 3: 1.56 us per step, 1.25 / 3
+// kSegLaunch (16384 points, 110-point segments, m = 3: 1.35 us per step, 1.4 / 3
 // of it the launches).
 struct SegPlan {
     int W[2] = {0, 0}, m = 0, launches = 0, Q = 0;
