@@ -73,9 +73,20 @@ void launch_restrict(const T *fine, T *xstar, int dim, int V, int nc, int r, cud
 // ---------------------------------------------------------------------------
 // Thread: observation j = bx * blockDim.x + threadIdx.x, rows i = i0 .. i0 +
 // rows - 1 of yf (members, then x^C* as row ne); its taps (<= 16) stay in
-// registers for those rows.  One problem alone takes 2 rows per thread (enough
-// threads to hide the gathers); a grouped launch over many problems 8.
-constexpr int kObsRows = 8, kObsRowsOne = 2;
+// registers for those rows, loaded 16 bytes at a time (the rows of the tables are
+// 16 or 64 bytes: scalar loads of a warp touched 32 segments each).  One problem
+// alone takes a row per thread (enough threads to hide the gathers; two rows
+// with scalar loads: NS analysis of 64 members and 2048 observations 185 us, 179
+// with 16-byte loads, 176 with one row); a grouped launch over many problems 8.
+constexpr int kObsRows = 8, kObsRowsOne = 1;
+
+// a 16-byte load of consecutive values (the tap rows are 4 or 16 long and start at
+// the beginning of their buffers)
+template <class V, class S>
+__device__ __forceinline__ void load_vec(const S *p, S *out) {
+    const V v = __ldg(reinterpret_cast<const V *>(p));
+    memcpy(out, &v, sizeof(V));
+}
 
 // With FP32 states and the weights split into FP32 pairs (wh, wl: w = wh + wl
 // up to 2^-48 |w|, mixed precision) the taps are summed in double-FP32
@@ -97,11 +108,12 @@ __device__ __forceinline__ void obs_apply_body(const T *__restrict__ members, co
         if (wh) {
             float w1[16], w2[16];
 #pragma unroll
-            for (int t = 0; t < 16; ++t)
+            for (int t = 0; t < 16; t += 4)
                 if (t < taps) {
-                    idx[t] = tap_idx[(size_t)j * taps + t];
-                    w1[t] = wh[(size_t)j * taps + t];
-                    w2[t] = wl[(size_t)j * taps + t];
+                    const size_t o = (size_t)j * taps + t;
+                    load_vec<int4>(tap_idx + o, idx + t);
+                    load_vec<float4>(wh + o, w1 + t);
+                    load_vec<float4>(wl + o, w2 + t);
                 }
             for (int i = i0; i < i1; ++i) {
                 const float *x = i < ne ? members + (size_t)i * nx : xstar;
@@ -124,10 +136,12 @@ __device__ __forceinline__ void obs_apply_body(const T *__restrict__ members, co
     }
     double w[16];
 #pragma unroll
-    for (int t = 0; t < 16; ++t)
+    for (int t = 0; t < 16; t += 4)
         if (t < taps) {
-            idx[t] = tap_idx[(size_t)j * taps + t];
-            w[t] = tap_w[(size_t)j * taps + t];
+            const size_t o = (size_t)j * taps + t;
+            load_vec<int4>(tap_idx + o, idx + t);
+            load_vec<double2>(tap_w + o, w + t);
+            load_vec<double2>(tap_w + o + 2, w + t + 2);
         }
     for (int i = i0; i < i1; ++i) {
         const T *x = i < ne ? members + (size_t)i * nx : xstar;
