@@ -792,10 +792,11 @@ static SegPlan seg_plan(int n0, int np0, int n1, int np1, int nsteps, int sms) {
     for (int P : {96, 128, 192, 256, 384, 512, 1024, 2048, 4096, 8 * kSegMaxThreads})
         for (int m : {1, 2, 3, 4, 5, 6, 8, 10, 13, 16, 24, 32}) {
             const int mm = std::min(m, nsteps), w = std::min(P - 6 * mm, kBurgersMaxPtsPerCta);
-            if (w < 32) continue;
+            if (w < 32) break;  // and for every larger m
             seg_try(best, tbest, n, np, nsteps, sms, {w, w}, mm, seg_q(P));
             if (both && n0 <= kBurgersMaxPtsPerCta && w < n0)
                 seg_try(best, tbest, n, np, nsteps, sms, {n0, w}, mm, seg_q(std::max(n0, P)));
+            if (m >= nsteps) break;  // the same again
         }
     if ((np0 <= 0 || n0 <= kBurgersMaxPtsPerCta) && (np1 <= 0 || n1 <= kBurgersMaxPtsPerCta))
         for (int Q : {1, 2, 4, 8}) seg_try(best, tbest, n, np, nsteps, sms, {n0, n1}, 1, Q);

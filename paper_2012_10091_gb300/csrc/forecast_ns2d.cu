@@ -1231,13 +1231,14 @@ static double march_estimate(int count, const int *n, const int *grids, const in
 void ns2d_default_choices(int count, const int *n, const int *grids, int sms, int *choice) {
     std::vector<int> c(count);
     double best = 0;
-    for (int rows = 0; rows < kNsSegChoices; ++rows) {
+    const int starts = count > 1 ? kNsSegChoices : 1;  // one size alone: every choice is tried in the first pass
+    for (int rows = 0; rows < starts; ++rows) {
         // from segments of these rows everywhere, one size at a time until no
         // change of one choice helps
         for (int k = 0; k < count; ++k) c[k] = n[k] > 128 ? kNsSegChoices + rows : rows;
         double now = march_estimate(count, n, grids, c.data(), sms);
         bool better = true;
-        for (int pass = 0; pass < 4 && better; ++pass) {
+        for (int pass = 0; pass < (count > 1 ? 4 : 1) && better; ++pass) {
             better = false;
             for (int k = 0; k < count; ++k)
                 for (int q = 0; q < kNsTileShapes; ++q) {
