@@ -318,11 +318,11 @@ __device__ __forceinline__ void step_x2(float2 (&hv)[Q + 6], float2 (&lo)[Q], fl
 
 template <int Q>
 __global__ void __launch_bounds__(512) burgers_f32x2_kernel(BurgersArgs<float> A) {
-    // A launch that follows this one with programmatic serialisation (the
-    // members after the fine run, see launch_burgers) may start once every CTA
-    // here is resident; before leaving, a CTA waits for the grid it follows
-    // (a no-op for a launch that follows none).
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // A launch that follows the fine run with programmatic serialisation (the
+    // members, see launch_burgers) may start once every CTA here is resident;
+    // before leaving, a CTA waits for the grid it follows (a no-op for a launch
+    // that follows none).  The members let nothing be placed beside them.
+    if (A.n_whole_probs == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *sh = reinterpret_cast<float2 *>(smem_raw);  // [2 buffers][first 3 | last 3][blockDim]
     const int t = threadIdx.x, nt = blockDim.x;
