@@ -147,15 +147,17 @@ __global__ void __launch_bounds__(kN64Threads) ns2d_march64(Ns64Args A) {
     const NsGroup<double> G = gi ? A.g[1] : A.g[0];
     const double c1 = gi ? A.c1[1] : A.c1[0], c2 = gi ? A.c2[1] : A.c2[0];
     const int n = G.n, TX = (n + G.tx - 1) / G.tx, pitch = (TX + 31) & ~31, upc = NT / pitch;
-    const int sub = tid / pitch, i = tid - sub * pitch;
+    // with halo columns (strips: one unit per CTA) every thread has the CTA's unit,
+    // also those past its columns or its pitch: they all fill in halo nodes
+    const bool halo = G.tx > 1;
+    const int sub = halo ? 0 : tid / pitch, i = tid - sub * pitch;
     const long long unit = (long long)((int)blockIdx.x - (gi ? A.ctas0 : 0)) * upc + sub;
     const int per_grid = G.tx * G.ty;
     const int prob = (int)(unit / per_grid), rem = (int)(unit - (long long)prob * per_grid);
     const int strip = rem / G.ty, seg = rem - strip * G.ty;
     const int x0 = strip * TX, w = min(TX, n - x0), y0 = seg * A.rows, rows = min(A.rows, n - y0);
-    const bool act = sub < upc && prob < G.nprob && i < w;
-    const bool halo = G.tx > 1;  // one unit per CTA then
-    const size_t plane = (size_t)n * n, off = (size_t)(act ? prob : 0) * 4 * plane;
+    const bool mine = sub < upc && prob < G.nprob, act = mine && i < w;  // has a unit, has a column of it
+    const size_t plane = (size_t)n * n, off = (size_t)(mine ? prob : 0) * 4 * plane;
     const double *u0 = G.u0 + off;
     const double *in = STAGE == 0 ? u0 : (STAGE == 1 ? G.s1 : G.s2) + off;
     double *out = (STAGE == 0 ? G.s1 : STAGE == 1 ? G.s2 : G.u0) + off;
