@@ -177,6 +177,7 @@ __global__ void __cluster_dims__(kThetaCtas, 1, 1) __launch_bounds__(32 * kTheta
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = blockIdx.x;
     const bool ok = *status == 0;
     double s0 = 0.0, s1 = 0.0;
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     if (ok) {
         double m0 = 0.0, m1 = 0.0;
         for (int a = lane; a < ne; a += 32) {
@@ -206,11 +207,13 @@ __global__ void __cluster_dims__(kThetaCtas, 1, 1) __launch_bounds__(32 * kTheta
             mine[warp][1] = s1;
         }
         __syncthreads();
-        if (threadIdx.x < 2) {
-            double m = 0.0;
-            for (int w = 0; w < kThetaWarps; ++w) m += mine[w][threadIdx.x];
-            inlet_push(&part[rank][threadIdx.x], 0, m);
-        }
+    }
+    // every CTA of the cluster runs (its shared memory may be written)
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (ok && threadIdx.x < 2) {
+        double m = 0.0;
+        for (int w = 0; w < kThetaWarps; ++w) m += mine[w][threadIdx.x];
+        inlet_push(&part[rank][threadIdx.x], 0, m);
     }
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
