@@ -270,8 +270,8 @@ mgenkf_status mgenkf_set_recentre(mgenkf_handle h, int32_t on);
  * in mgenkf_analyse); member forecast again from the previous analysis with
  * theta^a and state update with the same perturbations; fine correction with
  * the open-grid 4-point Lagrange Pi_F (one-sided at the ends).  H^C is the
- * Pi_F row at each observed fine node.  Limits: n_fine <= 1024 (one CTA per
- * grid), n_fine / ratio >= 8, ratio in [1, 16], 2 <= n_members <= 256. */
+ * Pi_F row at each observed fine node.  Limits: n_fine <= 1024 (one CTA or
+ * one cluster of up to 8 per grid), n_fine / ratio >= 8, ratio in [1, 16], 2 <= n_members <= 256. */
 typedef struct mgenkf_dual *mgenkf_dual_t;
 typedef struct {
     int32_t n_fine, ratio, n_members, n_obs;

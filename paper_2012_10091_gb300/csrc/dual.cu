@@ -36,9 +36,9 @@ constexpr uint64_t kThetaTag = 0x54485441ULL;  // "THTA": parameter random walk
 constexpr int kDualMaxPts = 1024;               // points per grid
 
 // SSP-RK3 steps of nprob inlet-Burgers grids of n points, each on a cluster of
-// CTAs (gridDim.x / nprob of them; one CTA where CLUSTER is false).  CTA r of a
-// cluster owns nodes [r per, (r + 1) per) and carries 3 nodes of its neighbours
-// on each side, one thread per node: stage 1 is evaluated two nodes into them,
+// CTAs (gridDim.x / nprob of them; one CTA where CLUSTER is false, a thread per
+// node of the grid).  CTA r of a cluster owns nodes [r per, (r + 1) per) and
+// carries 3 nodes of its neighbours on each side, one thread per node: stage 1 is evaluated two nodes into them,
 // stage 2 one node, so that the CTAs exchange values once per step (3 nodes
 // written to each neighbour's shared memory, double-buffered: a neighbour may
 // still be in the step before) and a stage ends in a barrier of the CTA.
@@ -56,6 +56,7 @@ constexpr int kDualMaxPts = 1024;               // points per grid
 // thread that reads it.  30 steps: 100 grids of 200 nodes 176 -> 60 us, one of
 // 800 (a cluster of 8, where one SM did all of it) 441 -> 48 us.
 constexpr int kInletSteps = 32;  // steps of inlet values formed together
+constexpr int kInletHalo = 3;    // nodes of each neighbour that a CTA of a cluster carries
 __device__ __forceinline__ void inlet_push(double *local, int rank, double v) {
     uint32_t a = (uint32_t)__cvta_generic_to_shared(local), r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
@@ -69,15 +70,16 @@ __global__ void __launch_bounds__(1024) k_burgers_inlet(double *__restrict__ u, 
     launch_wait();
     extern __shared__ double sh[];
     __shared__ double inlet[2 * kInletSteps];
-    const int pitch = per + 6;
+    constexpr int H = CLUSTER ? kInletHalo : 0;
+    const int pitch = per + 2 * H;
     double *X = sh, *B = sh + 2 * pitch, *C = sh + 3 * pitch;  // x (two buffers), u1, u2
     const int prob = CLUSTER ? blockIdx.x / ctas : blockIdx.x, rank = CLUSTER ? blockIdx.x - prob * ctas : 0;
-    // nodes [lo, hi) are this CTA's; slot j holds node lo - 3 + j
+    // nodes [lo, hi) are this CTA's; slot j holds node lo - H + j
     const int lo = rank * per, hi = min(n, lo + per);
-    const int j = threadIdx.x, k = lo - 3 + j;
+    const int j = threadIdx.x, k = lo - H + j;
     double *g = u + (size_t)prob * n;
     const double th1 = theta[2 * prob], th2 = theta[2 * prob + 1];
-    const bool held = j < pitch && k >= 0 && k < min(n, hi + 3);
+    const bool held = j < pitch && k >= 0 && k < min(n, hi + H);
     const bool own = held && k >= lo && k < hi;
     const bool first = held && k == 0, last = held && k == n - 1, before_last = held && k == n - 2;
     // nodes with both neighbours in this CTA
@@ -134,8 +136,8 @@ __global__ void __launch_bounds__(1024) k_burgers_inlet(double *__restrict__ u, 
         if (own) {
             an[j] = w;
             if (CLUSTER) {
-                // slot of node k in a neighbour: k - (its lo - 3)
-                if (j < 6 && rank > 0) inlet_push(an + j + per, rank - 1, w);
+                // slot of node k in a neighbour: k - (its lo - H)
+                if (j < 2 * H && rank > 0) inlet_push(an + j + per, rank - 1, w);
                 if (j >= per && rank + 1 < ctas) inlet_push(an + j - per, rank + 1, w);
             }
         }
@@ -295,22 +297,26 @@ void free_dual(mgenkf_dual *d) {
 // grids do not exceed the SMs (then each gets one)
 int inlet_ctas(int nprob, int n) {
     int c = 1;
-    while (c < 8 && ceil_div(n, c) + 6 > 128 && nprob * 2 * c <= kNumSMs) c *= 2;
+    while (c < 8 && ceil_div(n, c) + 2 * kInletHalo > 128 && nprob * 2 * c <= kNumSMs) c *= 2;
     return c;
 }
 
-void forecast(mgenkf_dual *d, double *grids, int nprob, int n, const double *theta, int nsteps,
-              cudaStream_t s = nullptr) {
+cudaError_t forecast(mgenkf_dual *d, double *grids, int nprob, int n, const double *theta, int nsteps,
+                     cudaStream_t s = nullptr) {
     count_launches(1);
     const int ctas = inlet_ctas(nprob, n), per = ceil_div(n, ctas);
     const double dx = d->cfg.length / n, dt = d->cfg.dt;
     const double a = dt / (4.0 * dx), c = 4.0 * d->cfg.nu / dx;
+    // a thread per node held (1024 for the largest grid, which one CTA holds alone);
     // 64 threads form the inlet values
-    const int threads = std::max(64, ceil_div(per + 6, 32) * 32);
-    const size_t smem = 4 * (per + 6) * sizeof(double);
-    launch_kernel(ctas > 1 ? k_burgers_inlet<true> : k_burgers_inlet<false>, nprob * ctas, threads, smem,
-                  s ? s : d->stream, LaunchHow{(unsigned)ctas}, grids, n, ctas, per, a, c, dt, nsteps, d->t, theta,
-                  d->cfg.u0, d->cfg.omega);
+    const int held = per + (ctas > 1 ? 2 * kInletHalo : 0);
+    const int threads = std::max(64, ceil_div(held, 32) * 32);
+    const cudaError_t e = launch_kernel(ctas > 1 ? k_burgers_inlet<true> : k_burgers_inlet<false>, nprob * ctas,
+                                        threads, 4 * held * sizeof(double), s ? s : d->stream,
+                                        LaunchHow{(unsigned)ctas}, grids, n, ctas, per, a, c, dt, nsteps, d->t, theta,
+                                        d->cfg.u0, d->cfg.omega);
+    if (e != cudaSuccess) cudaGetLastError();  // reported by the caller, not left pending
+    return e;
 }
 
 // perturbations (generated once per cycle), anomalies and T = S^-1 B (ensemble space)
@@ -450,8 +456,8 @@ extern "C" mgenkf_status mgenkf_dual_free_run(mgenkf_dual_t d, int32_t nsteps) {
     if (!d || nsteps < 0) return MGENKF_ERR_INVALID_ARG;
     d->err.clear();
     if (nsteps == 0) return MGENKF_OK;
-    forecast(d, d->fine, 1, d->nf, d->theta_mean, nsteps);
-    forecast(d, d->members, d->ne, d->nc, d->theta, nsteps);
+    D_CUDA(forecast(d, d->fine, 1, d->nf, d->theta_mean, nsteps));
+    D_CUDA(forecast(d, d->members, d->ne, d->nc, d->theta, nsteps));
     D_CUDA(cudaGetLastError());
     d->t += nsteps * d->cfg.dt;
     return MGENKF_OK;
@@ -468,7 +474,7 @@ extern "C" mgenkf_status mgenkf_dual_cycle(mgenkf_dual_t d, int32_t nsteps, cons
     // (theta_mean is rewritten only after the join below)
     D_CUDA(cudaEventRecord(d->ev[0], s));
     D_CUDA(cudaStreamWaitEvent(d->aux, d->ev[0], 0));
-    forecast(d, d->fine, 1, d->nf, d->theta_mean, nsteps, d->aux);
+    const cudaError_t fine = forecast(d, d->fine, 1, d->nf, d->theta_mean, nsteps, d->aux);
     launch_restrict<double>(d->fine, d->xstar, 1, 1, nc, d->cfg.ratio, d->aux);
     D_CUDA(cudaEventRecord(d->ev[1], d->aux));
     // Algorithm 3 step 2: parameter random walk, members forecast with theta^f
@@ -477,16 +483,18 @@ extern "C" mgenkf_status mgenkf_dual_cycle(mgenkf_dual_t d, int32_t nsteps, cons
     count_launches(1);
     launch_kernel(k_theta_walk, ceil_div(2 * ne, 256), 256, 0, s, LaunchHow{},
                   d->theta, d->tau, std::sqrt(d->cfg.theta_q), 2 * ne, d->theta_f);
-    forecast(d, d->members, ne, nc, d->theta_f, nsteps);
+    const cudaError_t members = forecast(d, d->members, ne, nc, d->theta_f, nsteps);
     // steps 3-5: perturbed observations, parameter update theta^a = theta^f + Theta T
-    gain_solve(d, 1, d->xstar_a);
+    if (members == cudaSuccess) gain_solve(d, 1, d->xstar_a);
     D_CUDA(cudaStreamWaitEvent(s, d->ev[1], 0));  // join: the fine forecast has read theta_mean
+    D_CUDA(fine);                                 // no analysis of grids that have not moved
+    D_CUDA(members);
     count_launches(1);
     launch_kernel(k_theta_update, kThetaCtas, 32 * kThetaWarps, 0, s, LaunchHow{},
                   d->theta_f, d->Bt, ne, 1.0 / ne, 1.0 / std::sqrt(ne - 1.0), d->theta, d->theta_mean, d->status);
     // steps 6-8: members forecast again from the previous analysis with theta^a, state update
     D_CUDA(cudaMemcpyAsync(d->members, d->prev, (size_t)ne * nc * 8, cudaMemcpyDeviceToDevice, s));
-    forecast(d, d->members, ne, nc, d->theta, nsteps);
+    D_CUDA(forecast(d, d->members, ne, nc, d->theta, nsteps));
     gain_solve(d, 0, d->xstar);  // the same perturbations
     launch_ens_anom<double>(d->members, nc, ne, d->X, nullptr, d->status, s);
     D_CUDA(cudaMemsetAsync(d->dC, 0, nc * sizeof(double), s));
