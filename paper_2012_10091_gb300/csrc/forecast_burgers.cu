@@ -611,10 +611,10 @@ static cudaError_t launch_burgers(BurgersArgs<T> A, cudaStream_t stream) {
 // (measured with dependent chains; 76 cycles with all four sub-partitions
 // busy), so a model step costs the FP64 instructions of the busiest
 // sub-partition and nothing else matters much.  One point per thread and 128
-// points per CTA put one warp on each sub-partition: 20 instructions, 0.7 us,
+// points per CTA put one warp on each sub-partition: 22 instructions, 0.7 us,
 // per step.  Measured, one 16384-point grid, 4331 steps: 157 ms on one
-// cluster of four CTAs of 4096 points (36 us per step), 5.84 ms in segments
-// (1.35 us per step, 149 CTAs of 128 points with their halo, 3 steps a launch;
+// cluster of four CTAs of 4096 points (36 us per step), 6.11 ms in segments
+// (1.41 us per step, 149 CTAs of 128 points with their halo, 3 steps a launch;
 // 6.74 ms with 26 instructions).
 //
 // A CTA advances the points of its segment and H = 3 steps of halo on both
@@ -625,15 +625,16 @@ static cudaError_t launch_burgers(BurgersArgs<T> A, cudaStream_t stream) {
 // in one launch, in place.  seg_plan() picks the segment length and the steps
 // per launch from the cost of a step and of a launch.
 //
-// Arithmetic (per stage, s = u_{j-1} + u_{j+1}): with c = 4 nu / dx,
-// a = dt / (4 dx),
-//   k = c (s - 2 u_j) + (u_{j-1} - u_{j+1}) s,  dt L = a k,
+// Arithmetic (per stage): with c = 4 nu / dx, a = dt / (4 dx), and the differences
+// d = u_{j-1} - u_{j+1}, f = u_{j+1} - u_j, exact for neighbours within a factor 2,
+//   k = c (d + 2 f) + d (u_{j-1} + u_{j+1}),  dt L = a k,
 //   u1 = u + a k0,  u2 = u + a/4 (k0 + k1),  u' = u + a/6 (k0 + k1 + 4 k2):
-// 20 instructions per point and step, and of the roundings at the size of u one
-// per stage counts in full (the one of s is damped by dt nu / dx^2).  From edge
-// differences it is 26 instructions; against extended precision over 600 to 3000
-// steps on 64 to 16384 points the two are equally good (rms 3e-16 to 6e-15 and
-// 3e-16 to 3e-15).
+// 22 instructions per point and step, the sums of k0, k1 and 4 k2 taken into the
+// products.  Against extended precision (24 to 240 states per size, 64 to 16384
+// points, dt nu / dx^2 of 0.02 to 0.4, smooth and rough) its rms error is 0.97 to
+// 1.01 of that of the Shu-Osher form from edge differences with 30 instructions.
+// d + 2 f as u_{j-1} + u_{j+1} - 2 u_j takes 20 and is 1.13 to 1.16 times off at dt
+// nu / dx^2 = 0.31 (the sum is rounded at the size of u): 5.84 ms for the run above.
 // ---------------------------------------------------------------------------
 struct SegGroup {
     const double *src;
@@ -675,7 +676,7 @@ __global__ void __launch_bounds__(Q == 1 ? 1024 : kSegMaxThreads) burgers_seg64(
             if (++j == G.n) j = 0;
         }
     }
-    const double a = G.a, c = G.c, a4 = 0.25 * a, a6 = a / 6.0;
+    const double a = G.a, c = G.c, c4 = 4.0 * c, a4 = 0.25 * a, a6 = a / 6.0;
     const int lt = t == 0 ? last : t - 1, rt = t == last ? 0 : t + 1;
     int buf = 0, lo = 0, hi = P;  // points [lo, hi) hold current values
     for (int step = 0; step < A.steps; ++step) {
@@ -697,16 +698,15 @@ __global__ void __launch_bounds__(Q == 1 ? 1024 : kSegMaxThreads) burgers_seg64(
 #pragma unroll
                 for (int k = 0; k < Q; ++k) {
                     const double cur = s[k], nxt = k + 1 < Q ? s[k + 1] : rgt;
-                    const double sum = prev + nxt;
-                    const double kq = fma(c, fma(-2.0, cur, sum), (prev - nxt) * sum);
+                    const double d = prev - nxt, sum = prev + nxt, lap = fma(2.0, nxt - cur, d);
                     if (stage == 0) {
-                        kk[k] = kq;
-                        s[k] = fma(a, kq, u[k]);
+                        kk[k] = fma(c, lap, d * sum);
+                        s[k] = fma(a, kk[k], u[k]);
                     } else if (stage == 1) {
-                        kk[k] += kq;
+                        kk[k] = fma(c, lap, fma(d, sum, kk[k]));
                         s[k] = fma(a4, kk[k], u[k]);
                     } else {
-                        u[k] = fma(a6, fma(4.0, kq, kk[k]), u[k]);
+                        u[k] = fma(a6, fma(c4, lap, fma(d, 4.0 * sum, kk[k])), u[k]);
                         s[k] = u[k];
                     }
                     prev = cur;
@@ -747,10 +747,10 @@ static SegShape seg_shape(int n, int W, int m, int Q) {
 // points (warps on all four sub-partitions of the SM) for every step count m
 // per launch, W = P - 6 m, and whole grids as rings, alone or (the members)
 // beside a segmented fine run.  A CTA's step costs its FP64 instructions per
-// warp (20 per point and step) at 19 cycles per
+// warp (22 per point and step) at 19 cycles per
 // warp, at least 64 each, and 100 cycles per stage for the barrier and the
 // exchange; CTAs on one SM add up; a launch costs
-// kSegLaunch (16384 points, 110-point segments, m = 3: 1.35 us per step, 1.4 / 3
+// kSegLaunch (16384 points, 110-point segments, m = 3: 1.41 us per step, 1.4 / 3
 // of it the launches).
 struct SegPlan {
     int W[2] = {0, 0}, m = 0, launches = 0, Q = 0;
@@ -759,7 +759,7 @@ struct SegPlan {
 constexpr double kSegLaunch = 2600.0;
 static void seg_try(SegPlan &best, double &tbest, const int (&n)[2], const int (&np)[2], int nsteps, int sms,
                     const int (&W)[2], int m, int Q) {
-    const int ops = 20 * Q;
+    const int ops = 22 * Q;
     long long ctas = 0;
     double slowest = 0.0, total = 0.0;
     bool rings = true;
