@@ -902,11 +902,15 @@ static void spd_factor_launch(double *A, double *At, int n, int *status, cudaStr
     launch_kernel(k_spd_factor<C>, C, kSpdThreads, spd_factor_smem(n, C), s, LaunchHow{C}, A, At, n, status);
 }
 
-__global__ void __launch_bounds__(kSpdThreads) k_spd_apply(const double *__restrict__ A, const double *__restrict__ At,
-                                                           int n, const double *rhs, double *out, int ncol,
-                                                           __nv_bfloat16 *out16, int ld16, const int *status) {
+// NT: 256, or 384 for orders above 224, where the registers are limited so that
+// two CTAs share an SM (there are more columns than SMs; n = 256: 86 us with one, 59)
+template <int NT>
+__global__ void __launch_bounds__(NT, NT > 256 ? 2 : 1)
+    k_spd_apply(const double *__restrict__ A, const double *__restrict__ At, int n, const double *rhs, double *out,
+                __nv_bfloat16 *out16, int ld16, const int *status) {
     launch_wait();
-    spd_apply_body<1>(A, At, n, rhs, out, ncol, out16, ld16, status, blockIdx.x);
+    const size_t c = blockIdx.x;
+    spd_apply_body(A, At, n, rhs + c * n, out + c * n, out16 ? out16 + c * ld16 : nullptr, status);
 }
 
 void launch_spd_factor(double *A, double *At, int n, int *status, cudaStream_t s) {
@@ -983,7 +987,8 @@ void launch_spd_solve(const double *A, const double *At, int n, const double *rh
                       __nv_bfloat16 *out16, int ld16, const int *status, cudaStream_t s) {
     count_launches(1);
     if (n <= kSpdMax)
-        launch_kernel(k_spd_apply, ncol, kSpdThreads, 0, s, LaunchHow{}, A, At, n, rhs, out, ncol, out16, ld16, status);
+        launch_kernel(spd_apply_threads(n) > 256 ? k_spd_apply<384> : k_spd_apply<256>, ncol, spd_apply_threads(n), 0,
+                      s, LaunchHow{}, A, At, n, rhs, out, out16, ld16, status);
     else if (n <= 512)
         k_chol_solve<16><<<ncol, 32, 0, s>>>(A, At, n, rhs, out, ncol, out16, ld16, status);
     else
@@ -1507,12 +1512,12 @@ __global__ void __cluster_dims__(kSpdGroupCluster, 1, 1) __launch_bounds__(kSpdT
     spd_factor_body<kSpdGroupCluster>(g.S, g.Lt, g.ne, g.status);
 }
 
-__global__ void __launch_bounds__(kSpdThreads)
+__global__ void __launch_bounds__(256)  // n <= 160 (group_supported)
     kg_spd_apply(const GroupProb *__restrict__ P, const int2 *__restrict__ map) {
     const int2 e = map[blockIdx.x];
     const GroupProb &g = P[e.x];
-    spd_apply_body<kSolveColsPerCta>(g.S, g.Lt, g.ne, g.Bt, g.Bt, g.ne + 1, g.Tt, g.ldx, g.status,
-                                     e.y * kSolveColsPerCta);
+    double *x = g.Bt + (size_t)e.y * g.ne;
+    spd_apply_body(g.S, g.Lt, g.ne, x, x, g.Tt + (size_t)e.y * g.ldx, g.status);
 }
 
 // prolongation of the coarse intervals vj = kProlongIntervals e.y .. + 7 of
@@ -1583,11 +1588,12 @@ bool group_plan_build(GroupPlan *plan, const std::vector<GroupProb> &probs, cons
         }
         if (g.splits > 1) add(kGsReduce, ceil_div((long long)g.ne * (2 * g.ne + 1), 256));
         add(kGsFactor, 1);
-        add(kGsSolve, ceil_div(g.ne + 1, kSolveColsPerCta));
+        add(kGsSolve, g.ne + 1);
         add(kGsProlong, ceil_div(4 * g.nc, kProlongIntervals));
     }
     // launch shapes (the largest problem's shared memory)
     plan->factor_smem = spd_factor_smem(maxne, kSpdGroupCluster);
+    plan->solve_threads = spd_apply_threads(maxne);
     // update: problems grouped by the CTAs per SM their shared memory and TMEM
     // columns allow, one launch per group of at most kUpdateLaunchMax
     {
@@ -1684,7 +1690,7 @@ cudaError_t group_analyse(const GroupPlan &plan, cudaStream_t s) {
     if (step(kGsReduce)) kg_gemm_reduce<<<n(kGsReduce), 256, 0, s>>>(P, M(kGsReduce));
     if (step(kGsFactor))
         kg_spd_factor<<<n(kGsFactor) * kSpdGroupCluster, kSpdThreads, plan.factor_smem, s>>>(P, M(kGsFactor));
-    if (step(kGsSolve)) kg_spd_apply<<<n(kGsSolve), kSpdThreads, 0, s>>>(P, M(kGsSolve));
+    if (step(kGsSolve)) kg_spd_apply<<<n(kGsSolve), plan.solve_threads, 0, s>>>(P, M(kGsSolve));
     count_launches(launches);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -52,14 +52,12 @@ enum GroupStep {
     kGsInnov,        // RMS of d*
     kGsGemm,         // S and Y^T R^-1 [D | d*] in double-FP32 arithmetic (tiles or K chunks)
     kGsReduce,       // sum of the K chunks
-    kGsFactor,       // S = L D L^T and L^-1, one 8-CTA cluster per problem
+    kGsFactor,       // S = L D L^T, one 8-CTA cluster per problem
     kGsSolve,        // T = S^-1 [Y^T R^-1 D | Y^T R^-1 d*], BF16 copy
     kGsUpdate,       // anomalies X, members += X T_i, dC = X T_ne (tensor cores)
     kGsProlong,      // x^F += Pi_F(dC), analysis counter + 1
     kGsSteps
 };
-
-constexpr int kSolveColsPerCta = 4;  // right-hand sides per CTA of the grouped solve
 
 // host side of a grouped analysis: the device table, the block maps of every
 // step and the launch shapes
@@ -69,6 +67,7 @@ struct GroupPlan {
     int nprob = 0;
     int map_off[kGsSteps] = {}, nblocks[kGsSteps] = {};
     size_t factor_smem = 0;  // the largest problem's
+    int solve_threads = 0;   // the largest problem's
     // update: one launch per class of problems that fit the same number of
     // CTAs per SM (at most kUpdateLaunchMax problems each), over the tiles
     // [map_begin, map_end) of the update map (entry = (index in probs, tile))
