@@ -86,16 +86,6 @@ struct Ns64Args {
     double c1[2], c2[2];   // -dt / (2h), dt mu / h^2 of each group
 };
 
-// 1 / x to about one unit in the last place: with e = 1 - x y of an approximate
-// reciprocal y (relative error 2^-20 or better), y (1 + e + e^2) = (1 - e^3) / x
-// (third-order Newton / Householder iteration)
-__device__ __forceinline__ double recip64(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
 // what a node contributes: u, v, T' = k2 T, rho u, rho v and the nodal fluxes
 // F = (rho u, F1, F2, F3), G = (rho v, F2, G2, G3)
 struct Node64 {

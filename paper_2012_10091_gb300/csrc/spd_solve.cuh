@@ -56,7 +56,7 @@ __device__ __forceinline__ int spd_owner(int i, int j) {
     return 1 + (i + j) % (C - 1);
 }
 // block slots per CTA for nb block rows: a worker owns at most i / (C - 1) + 1
-// blocks of row i; CTA 0 keeps nb inverse diagonal blocks and its two work blocks
+// blocks of row i; CTA 0 keeps the nb diagonal blocks of L and its two work blocks
 __host__ __device__ inline int spd_slots(int nb, int C) {
     int c = 0;
     for (int i = 0; i < nb; ++i) c += i / (C - 1) + 1;
@@ -69,25 +69,19 @@ inline size_t spd_factor_smem(int n, int C) {
     return sizeof(double) * ((size_t)(spd_slots((n + kSpdB - 1) / kSpdB, C) + 6 + 4) * kSpdBlk + kSpdMax);
 }
 
-// 1 / d of a pivot, to about one unit in the last place: with e = 1 - d y of an
-// approximate reciprocal y, y (1 + e + e^2) = (1 - e^3) / d (third-order
-// Newton iteration).  A pivot that is not positive and finite raises *fail and
+// 1 / d of a pivot.  A pivot that is not positive and finite raises *fail and
 // yields 1, so that the factorisation runs on.
 __device__ __forceinline__ double spd_pivot(double d, int *fail) {
-    // comparisons of doubles would take the FP64 pipe (64 cycles each): a high
-    // word in this range is a positive number between about 1e-300 and 1e300
-    const int hi = __double2hiint(d);
-    if (hi < 0x01c00000 || hi > 0x7e000000) {
+    // comparisons of doubles would take the FP64 pipe (64 cycles each): one test of
+    // the high word on the chain, sign included
+    if (!recip64_range(d) || __double2hiint(d) < 0) {
         if (!(d > 0.0) || !isfinite(d)) {
             *fail = 1;
             return 1.0;
         }
         return 1.0 / d;
     }
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-    const double e = fma(-d, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    return recip64_in_range(d);
 }
 
 // A diagonal block by warps 0-3 (128 threads): e[0] holds it (both triangles);
