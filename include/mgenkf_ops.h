@@ -29,7 +29,11 @@ extern "C" {
  *   Burgers).
  * Limits: Burgers n in [4, 32768]; NS n in [8, 4096] and n % 8 == 0; NS FP32
  * states start on a 16-byte boundary (the halo is copied in 16-byte chunks).
- * Outside them: MGENKF_ERR_INVALID_ARG. */
+ * Outside them: MGENKF_ERR_INVALID_ARG.
+ * Memory: NS states take stream-ordered scratch of twice their size
+ * (MGENKF_ERR_CUDA without it), FP64 Burgers states that one launch cannot hold
+ * scratch of their size (without it they are stepped in place, slower for few
+ * grids); a captured graph then holds memory nodes. */
 mgenkf_status mgk_forecast(int32_t model, int32_t precision, void *state, int32_t nprob, int32_t n,
                            double length, double dt, double nu, double gamma, double prandtl,
                            int32_t nsteps, void *stream);

@@ -854,7 +854,16 @@ cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, do
         if (g == 0) A.ctas0 = ctas;
         P = std::max(P, x.P);
     }
-    if (!rings && !scratch) return cudaErrorInvalidValue;
+    // no second buffer: in place, a grid per CTA or cluster (for the many grids whose
+    // buffer may not be had it fills the GPU as well)
+    if (!rings && !scratch) {
+        if (n_whole_probs > 0 && n_whole > kBurgersMaxPtsPerCta) {  // grids of one size, more than a CTA holds
+            if (n_split_probs > 0) return cudaErrorInvalidValue;
+            return burgers_forecast<double>(nullptr, 0, 0, whole, n_whole, n_whole_probs, length, dt, nu, nsteps, stream);
+        }
+        return burgers_forecast<double>(whole, n_whole, n_whole_probs, split, n_split, n_split_probs, length, dt, nu,
+                                        nsteps, stream);
+    }
     const int threads = ceil_div(ceil_div(P, pl.Q), 32) * 32;
     // segments: the CTAs spread over the SMs (rings run once, whatever their place)
     const int per_sm = rings ? 0 : ceil_div(ctas, device_sms());
@@ -927,5 +936,7 @@ cudaError_t burgers_forecast(T *whole, int n_whole, int n_whole_probs, T *split,
 
 template cudaError_t burgers_forecast<float>(float *, int, int, float *, int, int, double, double,
                                              double, int, cudaStream_t);
+template cudaError_t burgers_forecast<double>(double *, int, int, double *, int, int, double, double,
+                                              double, int, cudaStream_t);
 
 }  // namespace mgk

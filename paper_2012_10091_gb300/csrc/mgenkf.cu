@@ -325,8 +325,10 @@ static mgenkf_status create_impl(mgenkf_ctx *h, const mgenkf_config *cfg, const 
     }
     if (cfg->model == MGENKF_NS2D)
         H_ALLOC(h->ns_scratch, ns2d_scratch_elems(h->nc, h->ne, h->nf, 1) * ts);
-    else if (!h->mixed)
-        H_ALLOC(h->bur_scratch, (ne * nx + h->nxf) * ts);
+    else if (!h->mixed && cudaMalloc((void **)&h->bur_scratch, (ne * nx + h->nxf) * ts) != cudaSuccess) {
+        cudaGetLastError();  // the forecasts run in place then
+        h->bur_scratch = nullptr;
+    }
     {
         const size_t p1 = (size_t)gemm_nt_splits((int)ne, (int)ne, (int)ne + 1, (int)ny) * ne * (2 * ne + 1);
         const size_t p2 = (size_t)gemm_nt_splits((int)ne, 0, (int)ne + 1, (int)ny) * ne * (ne + 1);
@@ -1147,10 +1149,15 @@ extern "C" mgenkf_status mgk_forecast(int32_t model, int32_t precision, void *st
             e = whole ? burgers_forecast<float>((float *)state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, s)
                       : burgers_forecast<float>(nullptr, 0, 0, (float *)state, n, nprob, length, dt, nu, nsteps, s);
         else {
-            // stream-ordered scratch
+            // stream-ordered scratch; where there is no room for it, the steps run in place
             double *scratch = nullptr;
             const size_t elems = burgers64_scratch_elems(n, nprob, 0, 0, nsteps);
             e = elems ? cudaMallocAsync((void **)&scratch, elems * sizeof(double), s) : cudaSuccess;
+            if (e == cudaErrorMemoryAllocation) {
+                cudaGetLastError();
+                scratch = nullptr;
+                e = cudaSuccess;
+            }
             if (e == cudaSuccess)
                 e = burgers_forecast64((double *)state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, scratch, s);
             if (scratch) {
