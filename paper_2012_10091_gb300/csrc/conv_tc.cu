@@ -385,7 +385,11 @@ __global__ void __launch_bounds__(kConvThreads, EPI == kLoss ? 3 : 2) k_conv_tc(
                         }
                     } else if (EPI == kLoss) {
                         const int c = c0 >> 4, nf = 4 * n;
-                        const float s = __ldg(A.stats + 16 + c), rs = 1.f / s;
+                        const float s = __ldg(A.stats + 16 + c);
+                        // s and the differences times 2^+-64 where the reciprocal would
+                        // over- or underflow
+                        const float f = fabsf(s) < 0x1p-60f ? 0x1p64f : fabsf(s) > 0x1p60f ? 0x1p-64f : 1.f;
+                        const float sf = s * f, rs = 1.f / sf;
                         // Pi_F(dC) at the pixel's 16 fine points: 4-tap sums along x, then along y
                         const float *d = A.dC + ((size_t)b * 4 + c) * pl;
                         float sx[4][4];
@@ -414,9 +418,11 @@ __global__ void __launch_bounds__(kConvThreads, EPI == kLoss ? 3 : 2) k_conv_tc(
 #pragma unroll
                                 for (int ty = 0; ty < 4; ++ty) pf = fmaf(A.pw[4 * sy + ty], sx[ty][m], pf);
                                 // the quotient by s: a product with the reciprocal and one
-                                // correction by its remainder
-                                const float x1 = s * v[4 * sy + m] - (tv[m] - pf), q1 = x1 * rs;
-                                const float dv = fmaf(fmaf(-q1, s, x1), rs, q1);
+                                // correction by its remainder (a Newton step for the quotient);
+                                // the remainder of an infinite quotient is not a number and
+                                // becomes a finite one here
+                                const float x1 = s * v[4 * sy + m] - (tv[m] - pf), x2 = x1 * f, q1 = x2 * rs;
+                                const float dv = fmaf(fminf(fmaf(-q1, sf, x2), 3e38f), rs, q1);
                                 lsum += dv * dv;
                                 v[4 * sy + m] = 2.f * dv * A.inv_count;
                             }
