@@ -164,7 +164,7 @@ __global__ void k_theta_walk(const double *__restrict__ theta, const double *__r
 // cluster of kThetaCtas: each takes ne / kThetaCtas members, a warp per member
 // over the lanes, and the first sums the CTAs' means (one CTA with a thread per
 // member and parameter, chains of 3 ne FP64 instructions: 37 us for 100
-// members, 15 us so).
+// members, 17 us so).
 constexpr int kThetaCtas = 8, kThetaWarps = 8;
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -1196,7 +1196,9 @@ void ns2d_march_layout(int n, int shape, int *bands, int *segs, int *threads) {
 // the longest march decides; beyond that the work does, plus a tenth of the
 // longest march (and a little of each) for the ends of the launches.  CTAs of
 // more than four warps have an SM to themselves: they lose a tenth at their
-// barriers, and more where CTAs of many sizes leave few SMs empty.  (24
+// barriers, and half with more than two sizes at once (two: the members and the
+// fine run of one handle, or problems alike), as an SM whose large CTA has ended
+// is then taken by small CTAs of other sizes before it is empty again.  (24
 // problems of 64^2 .. 768^2, one choice for all: the estimates for 32, 48, 64,
 // 128 and 256 rows, wide and narrow, are proportional to the measured 6.2 ..
 // 7.9 ms within 5%; with the defaults 6.2 ms.)
