@@ -477,7 +477,9 @@ void launch_ens_anom(const T *members, size_t nx, int ne, double *X64, __nv_bflo
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_ens_anom<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int ctas = ceil_div(nx, 32);
-    launch_kernel(k_ens_anom<T>, ctas, 256, smem, s, LaunchHow{1, 1, 1, ctas <= kNumSMs / 4}, members, nx, ne,
+    // chained while a CTA is short (2 to 38 CTAs: 2 to 4 us gained up to 192 members, 30 to
+    // 39 us lost at 400)
+    launch_kernel(k_ens_anom<T>, ctas, 256, smem, s, LaunchHow{1, 1, 1, ctas <= kNumSMs / 4 && ne <= 192}, members, nx, ne,
                   1.0 / ne, 1.0 / std::sqrt((double)(ne - 1)), X64, X16, ldx, status);
 }
 
@@ -782,7 +784,13 @@ void launch_gemm_df(const DfOperands &df, int ne, int ny, double s2, double *S, 
     const GemmCluster g = gemm_cluster(splits);
     const dim3 grid(ceil_div(2 * ne + 1, 16), ceil_div(ne, 16), g.ctas ? g.ctas : splits);
     count_launches(g.ctas ? 1 : 2);
-    launch_kernel(k_gemm_df, grid, kDfThreads, 0, s, LaunchHow{1, 1, (unsigned)std::max(g.ctas, 1)}, df, ne, ny,
+    // chained unless its CTAs are long and about as many as the SMs (gained or lost:
+    // up to 80 CTAs 2 us gained, 144 of 128 products of K 1 gained, 168 to 288 of 128
+    // 3 lost, 220 of 512 17 lost, 210 of 2048 76 lost, 528 CTAs of any length 1 to 3
+    // gained; NS analysis of 64 members and 2048 observations 178 us chained, 172)
+    const unsigned ctas = grid.x * grid.y * grid.z, length = g.per * kchunk;
+    const bool chained = ctas <= kNumSMs / 2 || ctas > 2u * kNumSMs || length <= (ctas <= kNumSMs ? 128u : 64u);
+    launch_kernel(k_gemm_df, grid, kDfThreads, 0, s, LaunchHow{1, 1, (unsigned)std::max(g.ctas, 1), chained}, df, ne, ny,
                   g.per, kchunk, s2, 1.0, S, Bt, g.ctas ? (double *)nullptr : part, status);
     if (!g.ctas)
         launch_kernel(k_gemm_nt_reduce, grid_for((size_t)ne * (2 * ne + 1), 256), 256, 0, s, LaunchHow{}, part,
@@ -798,7 +806,10 @@ void launch_gemm_nt_f64(const double *A, int m, const double *B1, int n1, const 
     const dim3 grid(ceil_div(n1 + n2, 16), ceil_div(m, kGemmRows), g.ctas ? g.ctas : splits);
     count_launches(g.ctas ? 1 : 2);
     if (g.ctas) {
-        const bool chained = grid.x * grid.y * grid.z <= 2u * kNumSMs;
+        // S and T follow short kernels (up to 288 CTAs 2 to 3 us gained); the direct form's
+        // T (n1 = 0) follows the solves, which hold most SMs while its CTAs are placed on
+        // the others (60 CTAs 2 to 4 us gained, 144 of 60 to 250 products 10 to 43 lost)
+        const bool chained = grid.x * grid.y * grid.z <= (n1 == 0 ? 64u : 2u * kNumSMs);
         launch_kernel(k_gemm_nt, grid, kGemmThreads, 0, s, LaunchHow{1, 1, (unsigned)g.ctas, chained}, A, m, B1, n1,
                       B2, n2, K, g.per, kchunk, scale_div, diag, out1, out2, status);
         return;
@@ -1081,8 +1092,12 @@ static void update_launch(int cols, T *members, T *dC, const double *X, const do
         if (cols < Q) return update_launch<T, Q - 1>(cols, members, dC, X, Tm, nx, ne, status, s);
     const dim3 grid(ceil_div(nx, 32 * kUpdateWarps), ceil_div(ne + 1, Q));
     const size_t smem = sizeof(double) * Q * (size_t)((ne + 7) & ~7);  // <= 32 KB for ne <= 512
-    launch_kernel(k_update_f64<T, Q>, grid, 32 * kUpdateWarps, smem, s,
-                  LaunchHow{1, 1, 1, grid.x * grid.y <= 2u * kNumSMs}, members, dC, X, Tm, nx, ne, status);
+    // chained while a thread has few FMAs, ne of each column: it follows the solves, which
+    // hold most SMs while its CTAs are placed on the others (66 to 144 CTAs of up to
+    // 104 FMAs: 2 to 4 us gained; 152 of 896: 157 lost, 126 of 512: 117 lost)
+    const bool chained = grid.x * grid.y <= 2u * kNumSMs && Q * ((ne + 7) & ~7) <= 112;
+    launch_kernel(k_update_f64<T, Q>, grid, 32 * kUpdateWarps, smem, s, LaunchHow{1, 1, 1, chained}, members, dC, X,
+                  Tm, nx, ne, status);
 }
 
 template <typename T>

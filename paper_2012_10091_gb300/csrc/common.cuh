@@ -69,10 +69,11 @@ inline size_t residency_smem(size_t need, int ctas) {
 // writes are visible, and the next one may be placed.  For the chains of small
 // kernels of an analysis (the smallest cycle, 14 launches: 122 us, 98 us chained; three
 // layers of the learned correction 26.6 and 20.4 us).
-// A launch bound by the FP64 pipes with about as many CTAs as SMs or more is
-// better placed on an empty GPU: chained, its CTAs take the SMs that have room
-// while the previous kernel runs, two where others get none (4096 points, 128
-// members: anomalies 17 us slower, the update 55).
+// A launch of long CTAs, about as many as SMs, is better placed on an empty GPU:
+// chained, its CTAs take the SMs that have most room while the previous kernel
+// runs, several on one where others get none (4096 points, 128 members:
+// anomalies 17 us slower, the update 55; 2048 points: the update 190).  Such
+// launches say so by their size (the rules stand at the launches).
 struct LaunchHow {
     unsigned x = 1, y = 1, z = 1;  // cluster
     bool chained = true;
