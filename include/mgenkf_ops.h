@@ -31,7 +31,7 @@ extern "C" {
  * states start on a 16-byte boundary (the halo is copied in 16-byte chunks).
  * Outside them: MGENKF_ERR_INVALID_ARG.
  * Memory: NS states take stream-ordered scratch of twice their size
- * (MGENKF_ERR_CUDA without it), FP64 Burgers states that one launch cannot hold
+ * (MGENKF_ERR_CUDA without it), FP64 Burgers states of more than a few steps
  * scratch of their size (without it they are stepped in place, slower for few
  * grids); a captured graph then holds memory nodes. */
 mgenkf_status mgk_forecast(int32_t model, int32_t precision, void *state, int32_t nprob, int32_t n,

@@ -19,11 +19,15 @@ cudaError_t burgers_forecast(T *whole, int n_whole, int n_whole_probs, T *split,
                              int n_split_probs, double length, double dt, double nu, int nsteps,
                              cudaStream_t stream);
 
-// The same for FP64 states, as launches over halo'd segments.  scratch: at
-// least burgers64_scratch_elems() values (0: not used); NULL: burgers_forecast.
-size_t burgers64_scratch_elems(int n_whole, int n_whole_probs, int n_split, int n_split_probs, int nsteps);
+// The same for FP64 states, as launches over halo'd segments.  scratch: a second
+// state (n_whole n_whole_probs + n_split n_split_probs values); NULL: in place
+// (burgers_forecast) unless the grids are whole segments.
 cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, double *split, int n_split,
                                int n_split_probs, double length, double dt, double nu, int nsteps, double *scratch,
                                cudaStream_t stream);
+// nprob grids of n points, FP64, with stream-ordered scratch where it pays; in
+// place where there is no room for it.
+cudaError_t burgers_forecast64_stateless(double *state, int n, int nprob, double length, double dt, double nu,
+                                         int nsteps, cudaStream_t stream);
 
 }  // namespace mgk

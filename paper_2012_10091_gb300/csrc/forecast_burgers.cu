@@ -755,10 +755,11 @@ static SegShape seg_shape(int n, int W, int m, int Q) {
 struct SegPlan {
     int W[2] = {0, 0}, m = 0, launches = 0, Q = 0;
     bool rings = false;  // no halo: every step in one launch, in place
+    double t = 1e300;    // its cost
 };
 constexpr double kSegLaunch = 2600.0;
-static void seg_try(SegPlan &best, double &tbest, const int (&n)[2], const int (&np)[2], int nsteps, int sms,
-                    const int (&W)[2], int m, int Q) {
+static void seg_try(SegPlan &best, const int (&n)[2], const int (&np)[2], int nsteps, int sms, const int (&W)[2], int m,
+                    int Q) {
     const int ops = 22 * Q;
     long long ctas = 0;
     double slowest = 0.0, total = 0.0;
@@ -779,27 +780,46 @@ static void seg_try(SegPlan &best, double &tbest, const int (&n)[2], const int (
     const double step = std::max(slowest, per_sm * total / ctas) + 300.0 * per_sm;
     // a single segmented launch is followed by a copy back
     const double t = step * nsteps + kSegLaunch * (launches + (!rings && launches == 1));
-    if (t < tbest) {
-        tbest = t;
-        best = SegPlan{{W[0], W[1]}, rings ? nsteps : m, launches, Q, rings};
-    }
+    if (t < best.t) best = SegPlan{{W[0], W[1]}, rings ? nsteps : m, launches, Q, rings, t};
 }
 static SegPlan seg_plan(int n0, int np0, int n1, int np1, int nsteps, int sms) {
     SegPlan best;
-    double tbest = 1e300;
     const int n[2] = {n0, n1}, np[2] = {np0, np1};
     const bool both = np0 > 0 && np1 > 0;
     for (int P : {96, 128, 192, 256, 384, 512, 1024, 2048, 4096, 8 * kSegMaxThreads})
         for (int m : {1, 2, 3, 4, 5, 6, 8, 10, 13, 16, 24, 32}) {
             const int mm = std::min(m, nsteps), w = std::min(P - 6 * mm, kBurgersMaxPtsPerCta);
             if (w < 32) break;  // and for every larger m
-            seg_try(best, tbest, n, np, nsteps, sms, {w, w}, mm, seg_q(P));
+            seg_try(best, n, np, nsteps, sms, {w, w}, mm, seg_q(P));
             if (both && n0 <= kBurgersMaxPtsPerCta && w < n0)
-                seg_try(best, tbest, n, np, nsteps, sms, {n0, w}, mm, seg_q(std::max(n0, P)));
+                seg_try(best, n, np, nsteps, sms, {n0, w}, mm, seg_q(std::max(n0, P)));
             if (m >= nsteps) break;  // the same again
         }
     if ((np0 <= 0 || n0 <= kBurgersMaxPtsPerCta) && (np1 <= 0 || n1 <= kBurgersMaxPtsPerCta))
-        for (int Q : {1, 2, 4, 8}) seg_try(best, tbest, n, np, nsteps, sms, {n0, n1}, 1, Q);
+        for (int Q : {8, 4, 2, 1}) seg_try(best, n, np, nsteps, sms, {n0, n1}, 1, Q);  // of equal ones fewer threads
+    return best;
+}
+
+// A stateless call of few steps on np grids of n points: whole grids, as rings or
+// a CTA or cluster each in place (burgers_forecast), where the segments' gain would
+// not pay for the second buffer (kSegScratch: the stream's memory pool and the
+// copy back, 13 us; 384 points, one step: 35 us with it, 18 without).  The costs
+// leave out a launch's loads and stores, which count for a single step: there the
+// segments have to be a tenth faster (300 grids of 4093 points: 103 us in place, 118
+// in segments; of 12288: 272 and 204).  Returns the plan; Q = 0: burgers_forecast.
+constexpr double kSegScratch = 25000.0;
+static SegPlan seg_plan_stateless(int n, int np, int nsteps, int sms) {
+    SegPlan best = seg_plan(n, np, 0, 0, nsteps, sms);
+    if (best.rings) return best;
+    best.t += kSegScratch;
+    if (n <= kBurgersMaxPtsPerCta)
+        for (int Q : {8, 4, 2, 1})
+            if (n % Q == 0) seg_try(best, {n, 0}, {np, 0}, nsteps, sms, {n, 0}, 1, Q);
+    const int cs = burgers_split_factor(n), pts = ceil_div(n, std::max(cs, 1)), P = choose_pts(pts);
+    const int warps = ceil_div(ceil_div(pts, P), 32), per_sm = ceil_div((long long)np * cs, sms);
+    const double step = 30.0 * P * std::max(warps <= 3 ? 64.0 : 76.0 * ceil_div(warps, 4), per_sm * warps * 19.0) +
+                        300.0 * per_sm + (cs > 1 ? 1200.0 : 0.0);
+    if (cs > 0 && step * nsteps + kSegLaunch < (nsteps == 1 ? 1.1 : 1.0) * best.t) best.Q = 0;
     return best;
 }
 
@@ -822,20 +842,9 @@ static int device_sms() {
     return dev >= 0 && sms[dev] > 0 ? sms[dev] : kNumSMs;
 }
 
-size_t burgers64_scratch_elems(int n_whole, int n_whole_probs, int n_split, int n_split_probs, int nsteps) {
-    if (nsteps <= 0 || (n_whole_probs <= 0 && n_split_probs <= 0)) return 0;
-    if (seg_plan(n_whole, n_whole_probs, n_split, n_split_probs, nsteps, device_sms()).rings) return 0;
-    return (size_t)n_whole * std::max(n_whole_probs, 0) + (size_t)n_split * std::max(n_split_probs, 0);
-}
-
-cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, double *split, int n_split,
-                               int n_split_probs, double length, double dt, double nu, int nsteps, double *scratch,
-                               cudaStream_t stream) {
-    double *st[2] = {whole, split};
-    const int n[2] = {n_whole, n_split}, np[2] = {n_whole_probs, n_split_probs};
-    if (nsteps <= 0 || (np[0] <= 0 && np[1] <= 0)) return cudaSuccess;
-    const SegPlan pl = seg_plan(n[0], np[0], n[1], np[1], nsteps, device_sms());
-    if (pl.Q == 0) return cudaErrorInvalidConfiguration;
+// the launches of a plan; scratch may be NULL for rings
+static cudaError_t seg_run(const SegPlan &pl, double *const (&st)[2], const int (&n)[2], const int (&np)[2],
+                           double length, double dt, double nu, int nsteps, double *scratch, cudaStream_t stream) {
     SegArgs A = {};
     const size_t off[2] = {0, np[0] > 0 ? (size_t)n[0] * np[0] : 0};
     const bool rings = pl.rings;
@@ -853,16 +862,6 @@ cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, do
         ctas += np[g] * x.nseg;
         if (g == 0) A.ctas0 = ctas;
         P = std::max(P, x.P);
-    }
-    // no second buffer: in place, a grid per CTA or cluster (for the many grids whose
-    // buffer may not be had it fills the GPU as well)
-    if (!rings && !scratch) {
-        if (n_whole_probs > 0 && n_whole > kBurgersMaxPtsPerCta) {  // grids of one size, more than a CTA holds
-            if (n_split_probs > 0) return cudaErrorInvalidValue;
-            return burgers_forecast<double>(nullptr, 0, 0, whole, n_whole, n_whole_probs, length, dt, nu, nsteps, stream);
-        }
-        return burgers_forecast<double>(whole, n_whole, n_whole_probs, split, n_split, n_split_probs, length, dt, nu,
-                                        nsteps, stream);
     }
     const int threads = ceil_div(ceil_div(P, pl.Q), 32) * 32;
     // segments: the CTAs spread over the SMs (rings run once, whatever their place)
@@ -897,6 +896,45 @@ cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, do
                 if (e != cudaSuccess) return e;
             }
     return cudaSuccess;
+}
+
+cudaError_t burgers_forecast64(double *whole, int n_whole, int n_whole_probs, double *split, int n_split,
+                               int n_split_probs, double length, double dt, double nu, int nsteps, double *scratch,
+                               cudaStream_t stream) {
+    if (nsteps <= 0 || (n_whole_probs <= 0 && n_split_probs <= 0)) return cudaSuccess;
+    const SegPlan pl = seg_plan(n_whole, n_whole_probs, n_split, n_split_probs, nsteps, device_sms());
+    if (pl.Q == 0) return cudaErrorInvalidConfiguration;
+    if (!pl.rings && !scratch)
+        return burgers_forecast<double>(whole, n_whole, n_whole_probs, split, n_split, n_split_probs, length, dt, nu,
+                                        nsteps, stream);
+    return seg_run(pl, {whole, split}, {n_whole, n_split}, {n_whole_probs, n_split_probs}, length, dt, nu, nsteps,
+                   scratch, stream);
+}
+
+cudaError_t burgers_forecast64_stateless(double *state, int n, int nprob, double length, double dt, double nu,
+                                         int nsteps, cudaStream_t stream) {
+    if (nsteps <= 0 || nprob <= 0) return cudaSuccess;
+    const SegPlan pl = seg_plan_stateless(n, nprob, nsteps, device_sms());
+    double *scratch = nullptr;
+    if (pl.Q > 0 && !pl.rings) {
+        const cudaError_t e = cudaMallocAsync((void **)&scratch, (size_t)n * nprob * sizeof(double), stream);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            scratch = nullptr;
+        } else if (e != cudaSuccess) {
+            return e;
+        }
+    }
+    if (pl.Q == 0 || (!pl.rings && !scratch))
+        return n <= kBurgersMaxPtsPerCta
+                   ? burgers_forecast<double>(state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, stream)
+                   : burgers_forecast<double>(nullptr, 0, 0, state, n, nprob, length, dt, nu, nsteps, stream);
+    cudaError_t e = seg_run(pl, {state, nullptr}, {n, 0}, {nprob, 0}, length, dt, nu, nsteps, scratch, stream);
+    if (scratch) {
+        const cudaError_t e2 = cudaFreeAsync(scratch, stream);
+        if (e == cudaSuccess) e = e2;
+    }
+    return e;
 }
 
 int burgers_split_factor(int n) {

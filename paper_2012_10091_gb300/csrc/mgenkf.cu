@@ -1148,23 +1148,8 @@ extern "C" mgenkf_status mgk_forecast(int32_t model, int32_t precision, void *st
         if (precision == MGENKF_MIXED)
             e = whole ? burgers_forecast<float>((float *)state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, s)
                       : burgers_forecast<float>(nullptr, 0, 0, (float *)state, n, nprob, length, dt, nu, nsteps, s);
-        else {
-            // stream-ordered scratch; where there is no room for it, the steps run in place
-            double *scratch = nullptr;
-            const size_t elems = burgers64_scratch_elems(n, nprob, 0, 0, nsteps);
-            e = elems ? cudaMallocAsync((void **)&scratch, elems * sizeof(double), s) : cudaSuccess;
-            if (e == cudaErrorMemoryAllocation) {
-                cudaGetLastError();
-                scratch = nullptr;
-                e = cudaSuccess;
-            }
-            if (e == cudaSuccess)
-                e = burgers_forecast64((double *)state, n, nprob, nullptr, 0, 0, length, dt, nu, nsteps, scratch, s);
-            if (scratch) {
-                const cudaError_t e2 = cudaFreeAsync(scratch, s);
-                if (e == cudaSuccess) e = e2;
-            }
-        }
+        else
+            e = burgers_forecast64_stateless((double *)state, n, nprob, length, dt, nu, nsteps, s);
     } else if (model == MGENKF_NS2D) {
         const char *why = ns2d_check_size(n, n);
         if (why) {
